@@ -42,8 +42,8 @@ __host__ __device__ inline void tri_decode(int64_t t, int64_t *i, int64_t *j) {
 struct KernelFn {
     int ibs, gram;
     float two_m, m;
-    __device__ __forceinline__ float value(float gamma, int32_t d, float dc = 0.f) const {
-        return ibs ? __fdiv_rn(two_m - (float)d, m) : expf(-gamma * ((float)d + dc));
+    __device__ __forceinline__ float value(float gamma, float d, float dc = 0.f) const {
+        return ibs ? __fdiv_rn(two_m - d, m) : expf(-gamma * (d + dc));
     }
 };
 

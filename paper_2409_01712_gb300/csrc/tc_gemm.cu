@@ -511,6 +511,35 @@ __device__ __forceinline__ int64_t pair_item(const TcParams &p, int64_t u, uint3
 // ---------------------------------------------------------------------------
 constexpr int CH_PER_HALF = BN / 16 / 2;
 
+// Squared distance of two encoded rows from their squared norms and the
+// accumulated inner product s: every term is an integer of magnitude at most
+// 2^24 (norms and s at most 4 M, M <= 2^22), so the three FP32 additions are
+// exact.  The integer form needed two conversions per entry (F2I, I2F), which
+// run at an eighth of the FP32 rate.
+__device__ __forceinline__ float dist_f32(float ni, float nj, float s) { return (ni - s) + (nj - s); }
+
+// Running sum in two FP32 terms grown by error-free transformations (Knuth's
+// TwoSum): about 48 significant bits.  FP64 additions run at 1/64 of the FP32
+// rate here, and the two sums of a Build block (its entries and their squares)
+// kept its epilogue longer than its tensor work.  Build at N = 32768,
+// M = 8192: 4.03 ms with the FP64 sums and integer distances, 3.39 ms with
+// this; N = 16384, M = 8192: 1.07 and 0.87 ms.
+struct Sum2 {
+    float hi = 0.f, lo = 0.f;
+    __device__ __forceinline__ void add(float x) {
+        const float s = hi + x, bp = s - hi;
+        lo += (hi - (s - bp)) + (x - bp);
+        hi = s;
+    }
+    // x * x as the exact pair product + remainder
+    __device__ __forceinline__ void add_square(float x) {
+        const float q = x * x;
+        lo += fmaf(x, x, -q);
+        add(q);
+    }
+    __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+};
+
 // Issues L2 prefetches for the trailing-update input row segment of this
 // thread, before it waits for the accumulator.
 template <int OP>
@@ -538,8 +567,8 @@ __device__ __forceinline__ void epilogue_prefetch(const TcParams &p, const Work 
 // exp(-gamma d) - c times the staged weights, NQ (>= p) weight columns.
 template <int NQ>
 __device__ __forceinline__ void predict_half(const TcParams &p, uint32_t tacc, int ch0, int64_t gi, int64_t j0,
-                                             const int32_t *nb_s, const float *aw_s, float kc, float *dst) {
-    const int32_t ni = p.norms_a[gi];
+                                             const float *nb_s, const float *aw_s, float kc, float *dst) {
+    const float ni = (float)p.norms_a[gi];
     const bool real_row = gi < p.n_test;
     const int nc = p.nconf;
     float ci[CONF_MAX];
@@ -554,7 +583,7 @@ __device__ __forceinline__ void predict_half(const TcParams &p, uint32_t tacc, i
 #pragma unroll
         for (int e = 0; e < 16; ++e) {
             const int c = ch * 16 + e;
-            const int32_t d = ni + nb_s[c] - 2 * (int32_t)v[e];
+            const float d = dist_f32(ni, nb_s[c], v[e]);
             const float *ar = aw_s + c * PRED_MAX_P;
             // confounders of the training row: slots [16, 32) of its staged row (p <= 16 then)
             const float dc = nc ? conf_dist(ci, ar + 16, nc) : 0.f;
@@ -574,9 +603,9 @@ __device__ __forceinline__ void predict_half(const TcParams &p, uint32_t tacc, i
 // the thread's dot products with its own row; returns the warp's sum.
 template <int NQ, bool KTERM>
 __device__ __forceinline__ double grad_half(const TcParams &p, const Work &w, uint32_t tacc, int ch0, int64_t gi,
-                                            int64_t j0, const int32_t *nb_s, const float *aw_s) {
+                                            int64_t j0, const float *nb_s, const float *aw_s) {
     const int64_t a_real = KTERM ? p.n : p.n_test;
-    const int32_t ni = p.norms_a[gi];
+    const float ni = (float)p.norms_a[gi];
     const int pp = (int)p.p;
     float accA[NQ], accZ[NQ];
 #pragma unroll
@@ -587,8 +616,8 @@ __device__ __forceinline__ double grad_half(const TcParams &p, const Work &w, ui
 #pragma unroll
         for (int e = 0; e < 16; ++e) {
             const int c = ch * 16 + e;
-            const int32_t d = ni + nb_s[c] - 2 * (int32_t)v[e];
-            const float sv = (gi < a_real && j0 + c < p.n) ? (float)d * expf(-p.gamma * (float)d) : 0.f;
+            const float d = dist_f32(ni, nb_s[c], v[e]);
+            const float sv = (gi < a_real && j0 + c < p.n) ? d * expf(-p.gamma * d) : 0.f;
             const float *ar = aw_s + c * PRED_MAX_P;  // columns beyond p are zero
 #pragma unroll
             for (int q = 0; q < NQ; ++q) {
@@ -615,12 +644,12 @@ __device__ __forceinline__ double grad_half(const TcParams &p, const Work &w, ui
 
 template <int OP>
 __device__ __forceinline__ void epilogue(const TcParams &p, const Work &w, uint32_t tacc, int row, int half,
-                                         int32_t *nb_s, float *aw_s, double *red_s) {
+                                         float *nb_s, float *aw_s, double *red_s) {
     const int64_t b = p.b;
     const int ch0 = half * CH_PER_HALF;
     if (OP == OP_DIST) {
         const int64_t gi = w.i * b + w.sm * BM + row;
-        const int32_t ni = p.norms_a[gi];
+        const float ni = (float)p.norms_a[gi];
         const int nc = p.nconf;
         float ci[CONF_MAX];
 #pragma unroll
@@ -628,34 +657,40 @@ __device__ __forceinline__ void epilogue(const TcParams &p, const Work &w, uint3
         const int64_t tidx = tri_index(w.i, w.j);
         float *krow = p.Kd + tidx * b * b + (w.sm * BM + row) * b + w.sn * BN;
         uint32_t *drow = p.Dd ? p.Dd + tidx * b * b + (w.sm * BM + row) * b + w.sn * BN : nullptr;
-        double ss = 0.0, s1 = 0.0;
+        Sum2 sum2, sum1;
         for (int ch = ch0; ch < ch0 + CH_PER_HALF; ++ch) {
             float v[16];
             tmem_ld16(tacc + ch * 16, v);
             float kv[16];
-            uint32_t dv[16];
 #pragma unroll
             for (int e = 0; e < 16; ++e) {
                 const int c = ch * 16 + e;
                 const int64_t gj = w.j * b + w.sn * BN + c;
-                const int32_t d = ni + nb_s[c] - 2 * (int32_t)v[e];
+                const float d = dist_f32(ni, nb_s[c], v[e]);
                 const bool real = gi < p.n && gj < p.n;
                 // confounders of column c: slots [16, 32) of its staged row
                 const float dc = nc ? conf_dist(ci, aw_s + c * PRED_MAX_P + 16, nc) : 0.f;
                 kv[e] = real ? (p.kf.gram ? v[e] : p.kf.value(p.gamma, d, dc)) : (gi == gj ? 1.f : 0.f);
-                dv[e] = real ? (uint32_t)d : 0u;
-                ss += (double)kv[e] * (double)kv[e];
-                s1 += (double)kv[e];
+                sum2.add_square(kv[e]);
+                sum1.add(kv[e]);
             }
             float4 *dst = reinterpret_cast<float4 *>(krow + ch * 16);
 #pragma unroll
             for (int e = 0; e < 4; ++e) dst[e] = make_float4(kv[4 * e], kv[4 * e + 1], kv[4 * e + 2], kv[4 * e + 3]);
             if (drow) {
+                uint32_t dv[16];
+#pragma unroll
+                for (int e = 0; e < 16; ++e) {
+                    const int c = ch * 16 + e;
+                    const bool real = gi < p.n && w.j * b + w.sn * BN + c < p.n;
+                    dv[e] = real ? (uint32_t)dist_f32(ni, nb_s[c], v[e]) : 0u;
+                }
                 uint4 *dd = reinterpret_cast<uint4 *>(drow + ch * 16);
 #pragma unroll
                 for (int e = 0; e < 4; ++e) dd[e] = make_uint4(dv[4 * e], dv[4 * e + 1], dv[4 * e + 2], dv[4 * e + 3]);
             }
         }
+        double ss = sum2.value(), s1 = sum1.value();
         // deterministic per-block sums of K^2 and K: warp sums, then the eight
         // warps in order.  Layout: all K^2 partials, then all K partials.
         for (int o = 16; o > 0; o >>= 1) {
@@ -844,10 +879,10 @@ __device__ __forceinline__ bool epi_any(bool fail) {
 // Per-block epilogue inputs staged in shared memory by the epilogue warps.
 template <int OP>
 __device__ __forceinline__ void epilogue_stage(const TcParams &p, const Work &w, int row,
-                                               int32_t *nb_s, float *aw_s) {
+                                               float *nb_s, float *aw_s) {
     if (OP == OP_DIST) {
         const int64_t j0 = w.j * p.b + w.sn * BN;
-        for (int c = row; c < BN; c += EPI_THREADS) nb_s[c] = p.norms_b[j0 + c];
+        for (int c = row; c < BN; c += EPI_THREADS) nb_s[c] = (float)p.norms_b[j0 + c];
         if (p.nconf) {  // confounders of the block's columns: slots [16, 32) of each staged row
             for (int e = row; e < BN * CONF_MAX; e += EPI_THREADS) {
                 const int c = e / CONF_MAX, q = e % CONF_MAX;
@@ -857,7 +892,7 @@ __device__ __forceinline__ void epilogue_stage(const TcParams &p, const Work &w,
     } else if (OP == OP_GRADK) {
         // columns j of the block: norms, A_j in slots [0, 16), Z_j in [16, 32)
         const int64_t j0 = w.j * p.b + w.sn * BN;
-        for (int c = row; c < BN; c += EPI_THREADS) nb_s[c] = p.norms_b[j0 + c];
+        for (int c = row; c < BN; c += EPI_THREADS) nb_s[c] = (float)p.norms_b[j0 + c];
         for (int e = row; e < BN * PRED_MAX_P; e += EPI_THREADS) {
             const int c = e / PRED_MAX_P, q = e % PRED_MAX_P;
             float v = 0.f;
@@ -869,7 +904,7 @@ __device__ __forceinline__ void epilogue_stage(const TcParams &p, const Work &w,
             aw_s[e] = v;
         }
     } else if (OP == OP_PREDICT || OP == OP_GRADT) {
-        for (int c = row; c < BN; c += EPI_THREADS) nb_s[c] = p.norms_b[w.j * BN + c];
+        for (int c = row; c < BN; c += EPI_THREADS) nb_s[c] = (float)p.norms_b[w.j * BN + c];
         // weights of the block's 256 rows: thread `row` takes element q = row %
         // 32 of rows row / 32 + 8 k; all 32 loads are in flight before the
         // (bank-conflict-free) stores
@@ -910,7 +945,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 2 * NST + 7);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
     double *red_s = reinterpret_cast<double *>(tmem_slot + 2);
-    int32_t *nb_s = reinterpret_cast<int32_t *>(red_s + 16);
+    float *nb_s = reinterpret_cast<float *>(red_s + 16);
     float *aw_s = reinterpret_cast<float *>(nb_s + BN);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;

@@ -2,39 +2,46 @@
 // the triangular inverse of the factor, as one persistent dataflow kernel over
 // 64 x 64 blocks of the b x b tile (FP32).
 //
-// Items, claimed from a device counter in an order that respects their
-// dependencies:
-//   factor (NB = b / 64):
-//     P(q)        for q >= 1 first L_q,q-1 = A_q,q-1 X_q-1,q-1^T (published at
-//                 once) and A_qq -= L_q,q-1 L_q,q-1^T, then L_qq = chol(A_qq)
-//                 and X_qq = inv(L_qq) in shared memory: the chain from one
-//                 diagonal block to the next is a single item
-//     T(i, q)     L_iq = A_iq X_qq^T                     (i > q + 1)
-//     U(i, j, q)  A_ij -= L_iq L_jq^T                    (q < j <= i, i > q + 1)
-//   listed as P(0), then for q = 0 .. NB-2: P(q + 1) and the T and U items of
-//   column q;
-//   inverse X = L^-1 by recursive doubling, for s = 64, 128, ..., b / 2 and
-//   every pair of diagonal s-blocks:
-//     step 1      T_p = L_21 X_11                        (one 64 x 64 output block per item)
-//     step 2      X_21 = -X_22 T_p
-//   finish        X^T (for the backward substitution) and the FP16 hi/lo
-//                 split of X (operands of the tensor-core panel solve), per
-//                 64 x 64 block, as soon as that block of X is final.
-// Progress counters: upd[i][j] (updates applied to block (i, j)), pdone[q],
-// tdone[i][q], and finished items of each inverse pair (step 1 and step 2
-// separately).  Inverse items wait only for the blocks they read: a step-1
-// item for its row of L_21 (T items) and for X_11 (the pair's first half),
-// a step-2 item for X_22 and the pair's step-1 products, a finishing item for
-// the pairs whose second half holds its rows; so the inverse of the leading
-// blocks runs while the factorisation of the trailing ones goes on.  An item
-// only waits for items claimed before it by running CTAs, so the kernel always
-// progresses; every wait is bounded (%globaltimer) and ends the kernel with
-// KRR_ETIMEOUT.  Blocks written by other CTAs are read through L2
-// (ld.global.cg).
+// The critical path is the chain of diagonal blocks P(0) -> P(1) -> ... ->
+// P(NB - 1), NB = b / 64, so one CTA (block 0) does nothing else and keeps the
+// inverse it needs next in shared memory:
+//   P(q)   for q >= 1 L_q,q-1 = A_q,q-1 X_q-1,q-1^T and A_qq -= L_q,q-1
+//          L_q,q-1^T, then L_qq = chol(A_qq) and X_qq = inv(L_qq).
+// A loader warp of that CTA waits for the updates of A_q,q-1 and A_qq and
+// copies them in (cp.async) while P(q - 1) is still being factored; a publisher
+// warp fences and raises the progress counters, so neither the waits nor the
+// fences stall the eight compute warps.
+//
+// The other CTAs claim items from a device counter, in an order in which every
+// item depends only on earlier items and on the chain:
+//   for q = 0 .. NB-1:
+//     for i = q + 2 .. NB-1:
+//       T(i, q)     L_iq = A_iq X_qq^T
+//       U(i, j, q)  A_ij -= L_iq L_jq^T                 (q < j <= i)
+//     X(q, j), j <= q: row q of the inverse: X_qj = -X_qq sum_{j<=k<q} L_qk X_kj,
+//                   its transpose (for the backward substitution) and its FP16
+//                   hi/lo split (operands of the tensor-core panel solve).
+// Row q of the inverse needs the rows above it and X_qq only, so the inverse is
+// finished one product after the last diagonal block.  Blocks of X above the
+// diagonal are zero from the allocation on.
+// Progress counters: pdone[q], tdone[i][q], upd[i][j] (updates applied to block
+// (i, j)), xdone[i][j].  Items wait only for items claimed before them by
+// running CTAs and for the chain, which waits only for such items; every wait
+// is bounded (%globaltimer) and ends the kernel with KRR_ETIMEOUT.  Blocks
+// written by other CTAs are read through L2 (ld.global.cg, cp.async.cg).
+//
+// What bounds it: latency.  A link of the chain is one 64 x 64 x 64 product,
+// half of one, and the 64-column factor, whose pivots are serial.  One
+// tile of b = 1024 alone takes 0.27 ms and one of 256 0.07 ms; with the chain's
+// blocks as items of the common queue (every link paying a claim, the wait for
+// the counters, the loads and the publication) and the inverse by recursive
+// doubling after the factorisation it was 0.50 and 0.12 ms.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
+#include <string.h>
 
 #include <algorithm>
+#include <string>
 
 #include "krr_internal.h"
 
@@ -43,42 +50,36 @@ namespace krr {
 namespace {
 
 constexpr int DB = 64;          // block edge
-constexpr int DT = 256;         // threads per CTA
+constexpr int DS = DB + 4;      // row stride of a block in shared memory: 16-byte rows, 8 rows apart in banks
+constexpr int DC = 256;         // compute threads
+constexpr int DT = DC + 64;     // and, in the chain CTA, the loader and the publisher warp
 constexpr int DMAX_NB = 64;     // blocks per tile edge supported (b <= 4096)
+
+typedef float Blk[DB][DS];
 
 struct DiagParams {
     float *W;          // tile, overwritten by L (lower part)
-    float *X;          // inverse (zeroed before the launch)
+    float *X;          // inverse (zero above the diagonal)
     float *XT;         // transpose of the inverse
     __half *hi, *lo;   // FP16 split of the inverse (or null)
-    float *tmp;        // b * b / 2 floats: products of the inverse steps, one region per level
     int64_t b;
-    int NB, levels;
+    int NB;
     int64_t tile_k;
-    int64_t n_factor;  // number of factor items
-    int64_t items;
+    int items;
     int *ctr;          // counters (layout in ctr_* below)
-    double *minpiv;    // NB minimum pivots of this tile
+    double *lkk;       // out: sqrt of the largest diagonal entry of the tile before the factorisation
     DevErrors *err;
     uint64_t wait_ns;
 };
 
 // counter layout: [0] item counter, [1] abort, then pdone[NB], tdone[NB * NB],
-// upd[NB * NB], and per inverse pair (all levels, fewer than NB pairs) the
-// finished step-1 items i1done[NB] and step-2 items i2done[NB]
+// upd[NB * NB], xdone[NB * NB]
 __device__ __forceinline__ int *ctr_pdone(const DiagParams &p) { return p.ctr + 2; }
 __device__ __forceinline__ int *ctr_tdone(const DiagParams &p) { return ctr_pdone(p) + p.NB; }
 __device__ __forceinline__ int *ctr_upd(const DiagParams &p) { return ctr_tdone(p) + p.NB * p.NB; }
-__device__ __forceinline__ int *ctr_i1done(const DiagParams &p) { return ctr_upd(p) + p.NB * p.NB; }
-__device__ __forceinline__ int *ctr_i2done(const DiagParams &p) { return ctr_i1done(p) + p.NB; }
+__device__ __forceinline__ int *ctr_xdone(const DiagParams &p) { return ctr_upd(p) + p.NB * p.NB; }
 
-// Slot of pair `pr` of inverse level l (levels before it hold NB / 2,
-// NB / 4, ... pairs).
-__device__ __forceinline__ int pair_slot(const DiagParams &p, int l, int pr) {
-    int base = 0;
-    for (int q = 0; q < l; ++q) base += p.NB >> (q + 1);
-    return base + pr;
-}
+__device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
 __device__ __forceinline__ uint64_t globaltimer() {
     uint64_t t;
@@ -90,6 +91,11 @@ __device__ __forceinline__ int ld_acquire(const int *p) {
     int v;
     asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
+}
+
+__device__ __forceinline__ void record_timeout(const DiagParams &p) {
+    atomicExch(&p.ctr[1], 1);
+    atomicCAS(&p.err->code, 0, (int)KRR_ETIMEOUT);
 }
 
 // Bounded wait (one thread) until *c >= target; false on expiry / abort.
@@ -106,8 +112,7 @@ __device__ bool wait_ge(const int *c, int target, const DiagParams &p) {
         if ((it & 15) == 0) {
             if (*(volatile int *)&p.ctr[1]) return false;
             if (globaltimer() - t0 > p.wait_ns) {
-                atomicExch(&p.ctr[1], 1);
-                atomicCAS(&p.err->code, 0, (int)KRR_ETIMEOUT);
+                record_timeout(p);
                 return false;
             }
         }
@@ -120,186 +125,209 @@ __device__ __forceinline__ void signal(int *c) {
     atomicAdd(c, 1);
 }
 
+// Barriers between the warps of the chain CTA.
+__device__ __forceinline__ void mbar_init(uint64_t *b, uint32_t count) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(b)), "r"(count) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive(uint64_t *b) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(b)) : "memory");
+}
+__device__ __forceinline__ bool mbar_try_wait(uint64_t *b, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred P;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 P, [%1], %2;\n\t"
+        "selp.b32 %0, 1, 0, P;\n\t}\n"
+        : "=r"(ok)
+        : "r"(smem_u32(b)), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+// Bounded: the warp waited for itself waits at most twice for a counter, so
+// the limit lies beyond that.
+__device__ bool wait_bar(uint64_t *b, uint32_t parity, const DiagParams &p) {
+    if (mbar_try_wait(b, parity)) return true;
+    const uint64_t t0 = globaltimer(), limit = 4 * p.wait_ns + drain_limit(p.wait_ns);
+    for (uint32_t it = 1;; ++it) {
+        if (mbar_try_wait(b, parity)) return true;
+        if ((it & 31) == 0) {
+            if (*(volatile int *)&p.ctr[1]) return false;
+            if (globaltimer() - t0 > limit) {
+                record_timeout(p);
+                return false;
+            }
+        }
+    }
+}
+
+// Barrier of the compute threads.
+__device__ __forceinline__ void csync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
+
 // ---------------------------------------------------------------------------
-// Item list.
+// Item list of the other CTAs.
 // ---------------------------------------------------------------------------
-enum DiagKind { K_P = 0, K_T = 1, K_U = 2, K_I1 = 3, K_I2 = 4, K_FIN = 5 };
+enum DiagKind { K_T = 0, K_U = 1, K_X = 2 };
 
 struct DItem {
     int kind;
-    int q, i, j;     // factor blocks
-    int level, pair, a, c;  // inverse output block (a, c) of pair `pair` at `level`
-    int phase;       // inverse step index 2 * level + (0 | 1)
+    int i, j, q;  // T: (i, q), U: (i, j, q), X: (i, j)
 };
 
-// Items of factor group q (0 <= q <= NB - 2): P(q + 1), then for every row
-// i = q + 2 .. NB - 1 the items T(i, q), U(i, q + 1 .. i, q).
-__host__ __device__ inline int64_t factor_group_items(int NB, int q) {
-    const int64_t m = NB - q - 1;  // rows below block q
-    return m + m * (m + 1) / 2 - 1;
+// T and U items of column q: rows i = q + 2 .. NB - 1 hold 1 + (i - q) each.
+__host__ __device__ inline int column_items(int NB, int q) {
+    const int m = NB - q - 1;
+    return m >= 1 ? m + m * (m + 1) / 2 - 2 : 0;
 }
 
-__host__ __device__ inline int64_t factor_items_for(int NB) {
-    int64_t n = 1;  // P(0)
-    for (int q = 0; q + 1 < NB; ++q) n += factor_group_items(NB, q);
+__host__ __device__ inline int item_count(int NB) {
+    int n = 0;
+    for (int q = 0; q < NB; ++q) n += column_items(NB, q) + q + 1;
     return n;
 }
 
-// Items of inverse step (level l, step s): pairs * (sz / 64)^2.
-__host__ __device__ inline int64_t inv_step_items(int NB, int l) {
-    const int64_t nb = (int64_t)1 << l;   // sz / 64
-    const int64_t pairs = NB / (2 * nb);
-    return pairs * nb * nb;
-}
-
-__device__ void decode_item(const DiagParams &p, int64_t t, DItem &it) {
+__device__ void decode_item(const DiagParams &p, int t, DItem &it) {
     const int NB = p.NB;
-    if (t < p.n_factor) {
-        if (t == 0) {
-            it.kind = K_P;
-            it.q = 0;
-            return;
-        }
-        // walk the q groups: P(q + 1), then rows i = q + 2.. with T(i, q) and U(i, j, q)
-        int64_t r = t - 1;
-        for (int q = 0; q + 1 < NB; ++q) {
-            const int64_t g = factor_group_items(NB, q);
-            if (r >= g) {
-                r -= g;
-                continue;
-            }
-            if (r == 0) {
-                it.kind = K_P;
-                it.q = q + 1;
-                return;
-            }
+    for (int q = 0; q < NB; ++q) {
+        const int g = column_items(NB, q);
+        if (t < g) {
             it.q = q;
-            --r;
-            for (int i = q + 2; i < NB; ++i) {
-                const int64_t row = 1 + (i - q);  // T + U(i, q+1..i)
-                if (r < row) {
+            for (int i = q + 2;; ++i) {
+                const int row = 1 + (i - q);  // T, then U(i, q + 1 .. i)
+                if (t < row) {
                     it.i = i;
-                    if (r == 0) {
-                        it.kind = K_T;
-                    } else {
-                        it.kind = K_U;
-                        it.j = q + (int)r;
-                    }
+                    it.j = q + t;
+                    it.kind = (t == 0) ? K_T : K_U;
                     return;
                 }
-                r -= row;
+                t -= row;
             }
         }
-    }
-    int64_t r = t - p.n_factor;
-    for (int l = 0; l < p.levels; ++l) {
-        const int64_t per = inv_step_items(NB, l);
-        for (int s = 0; s < 2; ++s) {
-            if (r < per) {
-                const int64_t nb = (int64_t)1 << l;
-                it.kind = s == 0 ? K_I1 : K_I2;
-                it.level = l;
-                it.phase = 2 * l + s;
-                it.pair = (int)(r / (nb * nb));
-                it.a = (int)((r % (nb * nb)) / nb);
-                it.c = (int)(r % nb);
-                return;
-            }
-            r -= per;
+        t -= g;
+        if (t <= q) {
+            // the diagonal block first: its split is ready at once
+            it.kind = K_X;
+            it.i = q;
+            it.j = q - t;
+            return;
         }
+        t -= q + 1;
     }
-    it.kind = K_FIN;
-    it.i = (int)(r / NB);  // block (i, j) of the inverse
-    it.j = (int)(r % NB);
+    it.kind = -1;  // not reached: t < items
 }
 
 // ---------------------------------------------------------------------------
-// 64 x 64 block product on 256 threads: C = alpha * sum_k A_k op(B_k) + beta * C.
-// Thread (tx, ty) = (t % 16, t / 16) owns rows ty + 16 u and columns tx + 16 v.
+// 64 x 64 blocks.
 // ---------------------------------------------------------------------------
-struct BlkSmem {
-    float a[DB][DB + 1];
-    float b[DB][DB + 1];
-};
-
-__device__ __forceinline__ void load_blk(float (*dst)[DB + 1], const float *src, int64_t ld, bool trans) {
-    // 64 x 64 floats, 16 per thread as 4 float4 loads through L2
-    for (int e = threadIdx.x; e < DB * DB / 4; e += DT) {
+// Asynchronous copy of a block into shared memory by `n` threads (tid < n).
+__device__ __forceinline__ void load_async(Blk &dst, const float *src, int64_t ld, int tid, int n) {
+    for (int e = tid; e < DB * DB / 4; e += n) {
         const int r = e / (DB / 4), c4 = (e % (DB / 4)) * 4;
-        const float4 v = __ldcg(reinterpret_cast<const float4 *>(src + r * ld + c4));
-        if (trans) {
-            dst[c4 + 0][r] = v.x; dst[c4 + 1][r] = v.y; dst[c4 + 2][r] = v.z; dst[c4 + 3][r] = v.w;
-        } else {
-            dst[r][c4 + 0] = v.x; dst[r][c4 + 1] = v.y; dst[r][c4 + 2] = v.z; dst[r][c4 + 3] = v.w;
-        }
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(&dst[r][c4])), "l"(src + r * ld + c4)
+                     : "memory");
     }
 }
+__device__ __forceinline__ void load_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void load_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
+__device__ __forceinline__ void load_wait_but1() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
 
-// acc += A_blk (64 x 64) * Bs (64 x 64, [k][n] layout)
-__device__ __forceinline__ void mac_blk(const BlkSmem &s, float (&acc)[4][4]) {
+// acc += A B^T (both row-major, K along the rows): thread (tx, ty) = (t % 16,
+// t / 16) owns rows ty + 16 u and columns tx + 16 v.  Four K per step: 16-byte
+// loads keep the shared-memory wavefronts (12 per step and warp) below the
+// FMAs (64 / 4).  LOWER: only blocks v <= u.
+template <bool LOWER = false>
+__device__ __forceinline__ void mac_nt(const Blk &a, const Blk &b, float (&acc)[4][4]) {
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-#pragma unroll 8
-    for (int k = 0; k < DB; ++k) {
-        float av[4], bv[4];
+#pragma unroll 4
+    for (int k = 0; k < DB; k += 4) {
+        float4 av[4], bv[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) av[u] = s.a[ty + 16 * u][k];
+        for (int u = 0; u < 4; ++u) av[u] = *reinterpret_cast<const float4 *>(&a[ty + 16 * u][k]);
 #pragma unroll
-        for (int v = 0; v < 4; ++v) bv[v] = s.b[k][tx + 16 * v];
+        for (int v = 0; v < 4; ++v) bv[v] = *reinterpret_cast<const float4 *>(&b[tx + 16 * v][k]);
 #pragma unroll
         for (int u = 0; u < 4; ++u)
 #pragma unroll
-            for (int v = 0; v < 4; ++v) acc[u][v] = fmaf(av[u], bv[v], acc[u][v]);
+            for (int v = 0; v < 4; ++v) {
+                if (LOWER && v > u) continue;
+                acc[u][v] = fmaf(av[u].x, bv[v].x, acc[u][v]);
+                acc[u][v] = fmaf(av[u].y, bv[v].y, acc[u][v]);
+                acc[u][v] = fmaf(av[u].z, bv[v].z, acc[u][v]);
+                acc[u][v] = fmaf(av[u].w, bv[v].w, acc[u][v]);
+            }
     }
 }
 
-// C (ld) = alpha * acc + beta * C
-__device__ __forceinline__ void store_blk(float *C, int64_t ld, const float (&acc)[4][4], float alpha, float beta) {
+// acc += A E (E row-major along its columns): the thread owns rows ty + 16 u
+// and columns 4 tx + v.
+__device__ __forceinline__ void mac_nn(const Blk &a, const Blk &e, float (&acc)[4][4]) {
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+#pragma unroll 4
+    for (int k = 0; k < DB; k += 4) {
+        float4 av[4], ev[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) av[u] = *reinterpret_cast<const float4 *>(&a[ty + 16 * u][k]);
+#pragma unroll
+        for (int s = 0; s < 4; ++s) ev[s] = *reinterpret_cast<const float4 *>(&e[k + s][4 * tx]);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const float as[4] = {av[u].x, av[u].y, av[u].z, av[u].w};
+#pragma unroll
+            for (int s = 0; s < 4; ++s) {
+                acc[u][0] = fmaf(as[s], ev[s].x, acc[u][0]);
+                acc[u][1] = fmaf(as[s], ev[s].y, acc[u][1]);
+                acc[u][2] = fmaf(as[s], ev[s].z, acc[u][2]);
+                acc[u][3] = fmaf(as[s], ev[s].w, acc[u][3]);
+            }
+        }
+    }
+}
+
+__device__ __forceinline__ void zero_acc(float (&acc)[4][4]) {
 #pragma unroll
     for (int u = 0; u < 4; ++u)
 #pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            float *cp = C + (int64_t)(ty + 16 * u) * ld + tx + 16 * v;
-            const float old = (beta != 0.f) ? __ldcg(cp) : 0.f;
-            __stcg(cp, alpha * acc[u][v] + beta * old);
-        }
+        for (int v = 0; v < 4; ++v) acc[u][v] = 0.f;
 }
 
 // ---------------------------------------------------------------------------
-// P(q): Cholesky and inverse of the 64 x 64 diagonal block in shared memory,
-// blocked by 16 (a pivot that is not positive is recorded, first one wins,
-// and replaced by 1 so the rest stays finite):
-//   for each 16-block q of the diagonal:
-//     warp 0 factors A_qq and inverts L_qq in registers (lane l owns row l;
-//     columns and rows are broadcast by warp shuffles);
-//     L_iq = A_iq X_qq^T for the 16-row blocks below (all threads);
-//     A_ij -= L_iq L_jq^T on the trailing lower triangle (all threads, 16 x 16
-//     thread grid, rows of L_iq / L_jq held in registers);
-//   then X = L^-1 below the diagonal blocks, by block diagonals:
-//     X_iq = -X_ii (sum_{k=q}^{i-1} L_ik X_kq).
-// a holds A on entry and L on exit, x receives X; tmp is 3 x 16 x 17 floats.
+// Cholesky of the 64 x 64 block a (lower triangle in, L out) and E = X^T,
+// X = L^-1 (rows of E in the 16-blocks on and above the diagonal), by the
+// elimination of the 128 x 64 matrix [A; I] in four steps of 16 columns: the
+// same row operations that turn A into L turn the identity into X^T, so the
+// inverse needs no phase of its own.  Per step:
+//   1. warp 0: lanes 0-15 hold the 16 rows of the diagonal block (kept
+//      symmetric, so a lane also holds its column), lanes 16-31 the rows of
+//      the identity below it; every lane runs the same operations, column by
+//      column.  The broadcasts of row c need no pivot and run beside its
+//      reciprocal square root: a column costs one broadcast, the root, one
+//      product and one fused update in series.
+//   2. the other 48 active rows (of A below the block, of E above it) times
+//      the block's inverse;
+//   3. the trailing update of both parts.
+// A pivot that is not positive is recorded (first one wins) and replaced by 1
+// so the rest stays finite.
 // ---------------------------------------------------------------------------
-__device__ void chol_inv_64(float (*a)[65], float (*x)[65], float (*tmp)[16][17], float *dinv,
-                                            int &bad, float &mpiv) {
-    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+__device__ void chol_inv_64(Blk &a, Blk &e, int &bad, float &mpiv) {
+    const int t = threadIdx.x, lane = t & 31;
+    const int tc = t & 15, tr = t >> 4;
     const unsigned FULL = 0xffffffffu;
-    for (int e = t; e < 64 * 64; e += 256) x[e >> 6][e & 63] = 0.f;
-    __syncthreads();
+#pragma unroll 1
     for (int q = 0; q < 4; ++q) {
         const int o = 16 * q;
-        if (warp == 0) {
+        if (t < 32) {
             const int l = lane & 15;
-            float v[16], xr[16];
+            float v[16];
 #pragma unroll
-            for (int j = 0; j < 16; ++j) v[j] = (j <= l) ? a[o + l][o + j] : 0.f;
-#pragma unroll
-            for (int k = 0; k < 16; ++k) xr[k] = (k == l) ? 1.f : 0.f;
-            // column c of the factor, then column c of the inverse (it needs
-            // only columns 0 .. c of L): one loop, so the inverse step of
-            // column c fills the latency of column c + 1's pivot chain
+            for (int j = 0; j < 16; ++j) {
+                const float av = a[o + max(l, j)][o + min(l, j)];
+                v[j] = (lane < 16) ? av : (j == l ? 1.f : 0.f);
+            }
 #pragma unroll
             for (int c = 0; c < 16; ++c) {
-                float d = __shfl_sync(FULL, v[c], c);
+                float row[16];
+#pragma unroll
+                for (int i = c; i < 16; ++i) row[i] = __shfl_sync(FULL, v[i], c);
+                float d = row[c];
                 if (!(d > 0.f)) {
                     if (bad < 0) bad = o + c;
                     d = 1.f;
@@ -310,348 +338,452 @@ __device__ void chol_inv_64(float (*a)[65], float (*x)[65], float (*tmp)[16][17]
                 inv = inv * fmaf(-0.5f * d * inv, inv, 1.5f);
                 const float lcc = d * inv;
                 mpiv = fminf(mpiv, lcc);
-                if (l == c) {
-                    v[c] = lcc;
-                    if (lane == c) dinv[o + c] = inv;
-                } else if (l > c) {
-                    v[c] *= inv;
-                }
-                // constant loop bounds (j > c as a condition) keep v in registers
+                v[c] = (lane == c) ? lcc : v[c] * inv;
 #pragma unroll
-                for (int j = 1; j < 16; ++j) {
-                    if (j > c) {
-                        const float ljc = __shfl_sync(FULL, v[c], j);
-                        if (l >= j) v[j] = fmaf(-v[c], ljc, v[j]);
-                    }
-                }
-                // inverse: row c of X is final once scaled by 1 / L[c][c]
-                if (l == c) {
-#pragma unroll
-                    for (int k = 0; k <= c; ++k) xr[k] *= inv;
-                }
-#pragma unroll
-                for (int k = 0; k <= c; ++k) {
-                    const float xck = __shfl_sync(FULL, xr[k], c);
-                    if (l > c) xr[k] = fmaf(-v[c], xck, xr[k]);
-                }
+                for (int i = c + 1; i < 16; ++i) v[i] = fmaf(-v[c], row[i] * inv, v[i]);
             }
-            if (lane < 16) {
+            Blk &dst = (lane < 16) ? a : e;
 #pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    if (j <= l) {
-                        a[o + l][o + j] = v[j];
-                        x[o + l][o + j] = xr[j];
-                    }
-                }
+            for (int j = 0; j < 16; j += 4) {
+                float4 w;
+                w.x = (lane < 16 && j > l) ? 0.f : v[j];
+                w.y = (lane < 16 && j + 1 > l) ? 0.f : v[j + 1];
+                w.z = (lane < 16 && j + 2 > l) ? 0.f : v[j + 2];
+                w.w = (lane < 16 && j + 3 > l) ? 0.f : v[j + 3];
+                *reinterpret_cast<float4 *>(&dst[o + l][o + j]) = w;
             }
         }
-        __syncthreads();
-        const int rows = 64 - o - 16;
-        if (rows > 0) {
-            const int tc = t & 15, tr = t >> 4;
-            float res[3];
+        csync();
+        // active rows: blocks q + 1 .. 3 of A and 0 .. q - 1 of E
+        {
+            float ecol[16];
+#pragma unroll
+            for (int m = 0; m < 16; ++m) ecol[m] = e[o + m][o + tc];
 #pragma unroll
             for (int u = 0; u < 3; ++u) {
-                const int rr = tr + 16 * u;
-                if (rr < rows) {
-                    const int i = o + 16 + rr, c = o + tc;
-                    float acc = 0.f;
+                const int rb = (u < 3 - q) ? q + 1 + u : u - (3 - q);
+                float *row = (u < 3 - q) ? &a[16 * rb + tr][o] : &e[16 * rb + tr][o];
+                float acc = 0.f;
 #pragma unroll
-                    for (int k = 0; k < 16; ++k) acc = fmaf(a[i][o + k], x[c][o + k], acc);
-                    res[u] = acc;
+                for (int m = 0; m < 16; m += 4) {
+                    const float4 r4 = *reinterpret_cast<const float4 *>(row + m);
+                    acc = fmaf(r4.x, ecol[m], acc);
+                    acc = fmaf(r4.y, ecol[m + 1], acc);
+                    acc = fmaf(r4.z, ecol[m + 2], acc);
+                    acc = fmaf(r4.w, ecol[m + 3], acc);
                 }
+                __syncwarp();  // the 16 threads of a row share a warp
+                row[tc] = acc;
             }
-            __syncthreads();
+        }
+        csync();
+        if (q < 3) {
+            float4 lj[3][4];
 #pragma unroll
-            for (int u = 0; u < 3; ++u) {
-                const int rr = tr + 16 * u;
-                if (rr < rows) a[o + 16 + rr][o + tc] = res[u];
-            }
-            __syncthreads();
-            const int nb = rows / 16;
-            float li[3][16], lj[3][16];
+            for (int w = 0; w < 3; ++w)
+                if (w < 3 - q)
 #pragma unroll
-            for (int u = 0; u < 3; ++u) {
-                if (u < nb) {
+                    for (int m = 0; m < 4; ++m)
+                        lj[w][m] = *reinterpret_cast<const float4 *>(&a[o + 16 + 16 * w + tc][o + 4 * m]);
+            // row blocks: 3 - q of A (lower blocks only), then q + 1 of E
 #pragma unroll
-                    for (int k = 0; k < 16; ++k) {
-                        li[u][k] = a[o + 16 + tr + 16 * u][o + k];
-                        lj[u][k] = a[o + 16 + tc + 16 * u][o + k];
-                    }
-                }
-            }
+            for (int u = 0; u < 4; ++u) {
+                const bool in_a = u < 3 - q;
+                const int rb = in_a ? q + 1 + u : u - (3 - q);
+                float *row = in_a ? a[16 * rb + tr] : e[16 * rb + tr];
+                float4 li[4];
 #pragma unroll
-            for (int u = 0; u < 3; ++u) {
+                for (int m = 0; m < 4; ++m) li[m] = *reinterpret_cast<const float4 *>(row + o + 4 * m);
 #pragma unroll
                 for (int w = 0; w < 3; ++w) {
-                    if (u < nb && w <= u) {
-                        const int i = o + 16 + tr + 16 * u, j = o + 16 + tc + 16 * w;
-                        if (i >= j) {
-                            float acc = 0.f;
+                    if (w < 3 - q && (!in_a || w <= u)) {
+                        float acc = 0.f;
 #pragma unroll
-                            for (int k = 0; k < 16; ++k) acc = fmaf(li[u][k], lj[w][k], acc);
-                            a[i][j] -= acc;
+                        for (int m = 0; m < 4; ++m) {
+                            acc = fmaf(li[m].x, lj[w][m].x, acc);
+                            acc = fmaf(li[m].y, lj[w][m].y, acc);
+                            acc = fmaf(li[m].z, lj[w][m].z, acc);
+                            acc = fmaf(li[m].w, lj[w][m].w, acc);
                         }
+                        float *dst = row + o + 16 + 16 * w + tc;
+                        // block row q of E enters here: its entries right of
+                        // the diagonal block were zero
+                        *dst = ((!in_a && rb == q) ? 0.f : *dst) - acc;
                     }
                 }
             }
+            csync();
         }
-        __syncthreads();
-    }
-    // off-diagonal blocks of X = L^-1: X_iq = -X_ii sum_{k=q}^{i-1} L_ik X_kq
-    const int tc = t & 15, tr = t >> 4;
-    for (int dd = 1; dd < 4; ++dd) {
-        const int npair = 4 - dd;
-        for (int qq = 0; qq < npair; ++qq) {
-            const int ib = qq + dd;
-            float acc = 0.f;
-            for (int kb = qq; kb < ib; ++kb) {
-#pragma unroll
-                for (int k = 0; k < 16; ++k) acc = fmaf(a[16 * ib + tr][16 * kb + k], x[16 * kb + k][16 * qq + tc], acc);
-            }
-            tmp[qq][tr][tc] = acc;
-        }
-        __syncthreads();
-        for (int qq = 0; qq < npair; ++qq) {
-            const int ib = qq + dd;
-            float acc = 0.f;
-#pragma unroll
-            for (int k = 0; k < 16; ++k) acc = fmaf(x[16 * ib + tr][16 * ib + k], tmp[qq][k][tc], acc);
-            x[16 * ib + tr][16 * qq + tc] = -acc;
-        }
-        __syncthreads();
     }
 }
 
-// sub (optional): a product to subtract from A_qq first, held as the 16 x 16
-// thread grid of mac_blk holds it.
-__device__ void potrf_inv_block(const DiagParams &p, int q, BlkSmem &s, const float (*sub)[4] = nullptr) {
-    float (*a)[DB + 1] = s.a;
-    float (*x)[DB + 1] = s.b;
+// ---------------------------------------------------------------------------
+// The chain CTA.
+// ---------------------------------------------------------------------------
+struct ChainBars {
+    uint64_t full;      // loader -> compute: A_q,q-1 and A_qq are in
+    uint64_t s1free;    // compute -> loader: the panel buffer is free
+    uint64_t pubt, pubp;  // compute -> publisher: L_q,q-1 / L_qq and X_qq are written
+    volatile int pubseq;  // publications finished (t and p alternate)
+    int ok;
+};
+
+// s: [0] E = X_q-1,q-1^T, then X_qq^T; [1] A_q,q-1, then L_q,q-1; [2 + (q & 1)] A_qq
+__device__ void chain(const DiagParams &p, Blk *s, ChainBars &cb) {
+    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
     const int64_t b = p.b;
-    float *blk = p.W + (int64_t)q * DB * b + q * DB;
-    __shared__ float dinv[DB];
-    __shared__ float tmp[3][16][17];
-    const int tx = threadIdx.x & (DB - 1), ty = threadIdx.x / DB;  // 4 row groups
-    constexpr int RS = DT / DB;
-    for (int r = ty; r < DB; r += RS) a[r][tx] = __ldcg(blk + (int64_t)r * b + tx);
-    __syncthreads();
-    if (sub) {
-        const int gx = threadIdx.x & 15, gy = threadIdx.x >> 4;
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-#pragma unroll
-            for (int v = 0; v < 4; ++v) a[gy + 16 * u][gx + 16 * v] -= sub[u][v];
-        __syncthreads();
+    const int NB = p.NB;
+    auto blk = [&](float *m, int i, int j) { return m + (int64_t)i * DB * b + (int64_t)j * DB; };
+    if (warp == 8) {
+        // ------------------------------ loader ------------------------------
+        load_async(s[2], p.W, b, lane, 32);
+        load_commit();
+        load_wait_all();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&cb.full);
+        for (int q = 1; q < NB; ++q) {
+            bool ok = true;
+            if (lane == 0) {
+                ok = wait_ge(ctr_upd(p) + q * NB + q - 1, q - 1, p) && wait_ge(ctr_upd(p) + q * NB + q, q - 1, p);
+                if (ok) ok = wait_bar(&cb.s1free, (q - 1) & 1, p);
+            }
+            if (!__shfl_sync(0xffffffffu, (int)ok, 0)) break;
+            __syncwarp();
+            load_async(s[1], blk(p.W, q, q - 1), b, lane, 32);
+            load_async(s[2 + (q & 1)], blk(p.W, q, q), b, lane, 32);
+            load_commit();
+            load_wait_all();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&cb.full);
+        }
+        return;
     }
+    if (warp == 9) {
+        // ----------------------------- publisher -----------------------------
+        // largest diagonal entry of the tile before anything is overwritten:
+        // the compute warps store L_00 after the arrival on barrier 2, the
+        // other CTAs write after pdone[0]
+        float mx = 0.f;
+        for (int64_t r = lane; r < b; r += 32) mx = fmaxf(mx, __ldcg(p.W + r * b + r));
+        for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        if (lane == 0) *p.lkk = sqrt((double)mx);
+        asm volatile("bar.arrive 2, 288;" ::: "memory");
+        if (lane != 0) return;
+        for (int q = 0; q < NB; ++q) {
+            if (q > 0) {
+                if (!wait_bar(&cb.pubt, (q - 1) & 1, p)) return;
+                signal(ctr_tdone(p) + q * NB + q - 1);
+                cb.pubseq = 2 * q;
+            }
+            if (!wait_bar(&cb.pubp, q & 1, p)) return;
+            signal(ctr_pdone(p) + q);
+            cb.pubseq = 2 * q + 1;
+        }
+        return;
+    }
+    // ------------------------------ compute ------------------------------
+    const int tx = t & 15, ty = t >> 4;
     int bad = -1;
     float mpiv = 3.0e38f;
-    chol_inv_64(a, x, tmp, dinv, bad, mpiv);
-    float *iblk = p.X + (int64_t)q * DB * b + q * DB;
-    for (int r = ty; r < DB; r += RS) {
-        __stcg(blk + (int64_t)r * b + tx, (tx <= r) ? a[r][tx] : 0.f);
-        __stcg(iblk + (int64_t)r * b + tx, (tx <= r) ? x[r][tx] : 0.f);
+    // the publication two before this one on the same barrier is through (it
+    // always is: a link takes several times a publication)
+    auto arrive_pub = [&](uint64_t *bar, int seq) {
+        __syncwarp();
+        if (lane == 0) {
+            const uint64_t t0 = globaltimer();
+            while (cb.pubseq < seq - 2 && globaltimer() - t0 < 4 * p.wait_ns && !*(volatile int *)&p.ctr[1]) {}
+            mbar_arrive(bar);
+        }
+    };
+    for (int q = 0; q < NB; ++q) {
+        if (t == 0) cb.ok = wait_bar(&cb.full, q & 1, p) ? 1 : 0;
+        csync();
+        if (!cb.ok) return;
+        Blk &A = s[2 + (q & 1)];
+        if (q > 0) {
+            // L_q,q-1 = A_q,q-1 X_q-1,q-1^T
+            float acc[4][4];
+            zero_acc(acc);
+            mac_nn(s[1], s[0], acc);
+            csync();
+            float *g = blk(p.W, q, q - 1);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const float4 w = make_float4(acc[u][0], acc[u][1], acc[u][2], acc[u][3]);
+                *reinterpret_cast<float4 *>(&s[1][ty + 16 * u][4 * tx]) = w;
+                __stcg(reinterpret_cast<float4 *>(g + (int64_t)(ty + 16 * u) * b + 4 * tx), w);
+            }
+            arrive_pub(&cb.pubt, 2 * q);
+            csync();
+            // A_qq -= L_q,q-1 L_q,q-1^T (lower blocks)
+            zero_acc(acc);
+            mac_nt<true>(s[1], s[1], acc);
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+#pragma unroll
+                for (int v = 0; v <= u; ++v) A[ty + 16 * u][tx + 16 * v] -= acc[u][v];
+            csync();
+        }
+        if (t == 0) mbar_arrive(&cb.s1free);
+        int bq = -1;
+        chol_inv_64(A, s[0], bq, mpiv);
+        if (bq >= 0 && bad < 0) bad = q * DB + bq;
+        if (q == 0) asm volatile("bar.sync 2, 288;" ::: "memory");
+        // L_qq and X_qq^T by rows, X_qq by columns of E
+        float *gl = blk(p.W, q, q), *gt = blk(p.XT, q, q), *gx = blk(p.X, q, q);
+        {
+            // X first: the other CTAs wait for it.  Lanes along the rows of E:
+            // 16-byte reads, 128-byte stores
+            const int k = t & 63, c0 = (t >> 6) * 16;
+#pragma unroll
+            for (int c = c0; c < c0 + 16; c += 4) {
+                const float4 w = *reinterpret_cast<const float4 *>(&s[0][k][c]);
+                const bool in = (c >> 4) >= (k >> 4);
+                __stcg(gx + (int64_t)c * b + k, in ? w.x : 0.f);
+                __stcg(gx + (int64_t)(c + 1) * b + k, in ? w.y : 0.f);
+                __stcg(gx + (int64_t)(c + 2) * b + k, in ? w.z : 0.f);
+                __stcg(gx + (int64_t)(c + 3) * b + k, in ? w.w : 0.f);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int r = ty + 16 * u, c = 4 * tx;
+            float4 w = *reinterpret_cast<const float4 *>(&s[0][r][c]);
+            if ((c >> 4) < (r >> 4)) {
+                // below the diagonal blocks E is zero; the next product reads it
+                w = make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+            __stcg(reinterpret_cast<float4 *>(gt + (int64_t)r * b + c), w);
+            const float4 l = *reinterpret_cast<const float4 *>(&A[r][c]);
+            __stcg(reinterpret_cast<float4 *>(gl + (int64_t)r * b + c),
+                   make_float4(c <= r ? l.x : 0.f, c + 1 <= r ? l.y : 0.f, c + 2 <= r ? l.z : 0.f,
+                               c + 3 <= r ? l.w : 0.f));
+        }
+        arrive_pub(&cb.pubp, 2 * q + 1);
+        csync();
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int r = ty + 16 * u, c = 4 * tx;
+            if ((c >> 4) < (r >> 4)) *reinterpret_cast<float4 *>(&s[0][r][c]) = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
     }
-    if (threadIdx.x == 0) {
-        p.minpiv[q] = (double)mpiv;
+    if (t == 0) {
+        p.err->min_pivot = fmin(p.err->min_pivot, (double)mpiv);
         if (bad >= 0 && atomicCAS(&p.err->code, 0, (int)KRR_ENOTPD) == 0) {
             p.err->bad_tile = p.tile_k;
-            p.err->bad_column = p.tile_k * b + (int64_t)q * DB + bad;
+            p.err->bad_column = p.tile_k * b + bad;
         }
     }
 }
 
 __global__ void __launch_bounds__(DT) diag_kernel(const DiagParams p) {
-    __shared__ BlkSmem s;
-    __shared__ int64_t item_s;
+    extern __shared__ __align__(16) float diag_smem[];
+    Blk *s = reinterpret_cast<Blk *>(diag_smem);  // four blocks
+    __shared__ ChainBars cb;
+    __shared__ int item_s;
     __shared__ int ok_s;
+    __shared__ int rdy[DMAX_NB];
     const int64_t b = p.b;
     const int NB = p.NB;
-    while (true) {
-        if (threadIdx.x == 0) item_s = atomicAdd(&p.ctr[0], 1);
-        __syncthreads();
-        const int64_t t = item_s;
-        if (t >= p.items) break;
-        DItem it;
-        decode_item(p, t, it);
-        // ---- wait for the inputs (one thread), then all threads proceed
-        if (threadIdx.x == 0) {
-            bool ok = true;
-            int *upd = ctr_upd(p), *tdone = ctr_tdone(p), *pdone = ctr_pdone(p);
-            if (it.kind == K_P) {
-                // P(q), q >= 1: X_q-1,q-1, and blocks (q, q-1) and (q, q) with the
-                // updates of columns 0 .. q-2
-                // (the other two inputs are awaited in the item body, after the
-                // first block is loaded)
-                if (it.q > 0) ok = wait_ge(upd + it.q * NB + it.q - 1, it.q - 1, p);
-            } else if (it.kind == K_T) {
-                ok = wait_ge(pdone + it.q, 1, p) && wait_ge(upd + it.i * NB + it.q, it.q, p);
-            } else if (it.kind == K_U) {
-                ok = wait_ge(tdone + it.i * NB + it.q, 1, p) && wait_ge(tdone + it.j * NB + it.q, 1, p) &&
-                     wait_ge(upd + it.i * NB + it.j, it.q, p);
-            } else if (it.kind == K_I1 || it.kind == K_I2) {
-                const int nb = 1 << it.level, r0 = 2 * it.pair * nb, half = nb / 2;
-                // X of the pair's first (I1) or second (I2) half: the P item at
-                // level 0, else all step-2 items of that half one level down
-                const int sub = (it.kind == K_I1) ? 0 : 1;
-                ok = (it.level == 0) ? wait_ge(pdone + r0 + sub, 1, p)
-                                     : wait_ge(ctr_i2done(p) + pair_slot(p, it.level - 1, 2 * it.pair + sub),
-                                               half * half, p);
-                if (it.kind == K_I1) {
-                    // row a of L_21, columns c .. nb - 1
-                    for (int k = it.c; k < nb && ok; ++k) ok = wait_ge(tdone + (r0 + nb + it.a) * NB + r0 + k, 1, p);
-                } else {
-                    ok = ok && wait_ge(ctr_i1done(p) + pair_slot(p, it.level, it.pair), nb * nb, p);
-                }
-            } else if (it.j == it.i) {
-                ok = wait_ge(pdone + it.i, 1, p);  // diagonal block of X
-            } else if (it.j < it.i) {
-                // block (i, j) of X is written by the step-2 items of the pair in
-                // which i and j first fall into different halves
-                const int l = 31 - __clz(it.i ^ it.j), nb = 1 << l;
-                ok = wait_ge(ctr_i2done(p) + pair_slot(p, l, it.i >> (l + 1)), nb * nb, p);
-            }  // blocks above the diagonal are zero from the start
-            ok_s = ok ? 1 : 0;
+    const int t = threadIdx.x;
+    if (blockIdx.x == 0) {
+        if (t == 0) {
+            mbar_init(&cb.full, 1);
+            mbar_init(&cb.s1free, 1);
+            mbar_init(&cb.pubt, DC / 32);
+            mbar_init(&cb.pubp, DC / 32);
+            cb.pubseq = 0;
         }
         __syncthreads();
-        if (!ok_s) break;
+        chain(p, s, cb);
+        return;
+    }
+    if (t >= DC) return;
+    const int tx = t & 15, ty = t >> 4;
+    int *upd = ctr_upd(p), *tdone = ctr_tdone(p), *pdone = ctr_pdone(p), *xdone = ctr_xdone(p);
+    auto blk = [&](float *m, int i, int j) { return m + (int64_t)i * DB * b + (int64_t)j * DB; };
+    while (true) {
+        if (t == 0) item_s = atomicAdd(&p.ctr[0], 1);
+        csync();
+        const int n = item_s;
+        if (n >= p.items) break;
+        DItem it;
+        decode_item(p, n, it);
         float acc[4][4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-#pragma unroll
-            for (int v = 0; v < 4; ++v) acc[u][v] = 0.f;
-        if (it.kind == K_P) {
-            if (it.q > 0) {
-                // L_q,q-1 = A_q,q-1 X_q-1,q-1^T, published for the U items of column q-1
-                const int q = it.q;
-                float *c = p.W + (int64_t)q * DB * b + (q - 1) * DB;
-                // A_q,q-1 (final since the updates of columns 0 .. q-2) comes in
-                // while P(q-1) may still be running
-                load_blk(s.a, c, b, false);
-                __syncthreads();  // every thread has read the previous ok_s
-                if (threadIdx.x == 0)
-                    ok_s = (wait_ge(ctr_pdone(p) + q - 1, 1, p) && wait_ge(ctr_upd(p) + q * NB + q, q - 1, p)) ? 1 : 0;
-                __syncthreads();
-                if (!ok_s) break;
-                load_blk(s.b, p.X + (int64_t)(q - 1) * DB * b + (q - 1) * DB, b, true);
-                __syncthreads();
-                mac_blk(s, acc);
-                __syncthreads();
-                store_blk(c, b, acc, 1.f, 0.f);
-                // L_q,q-1 into s.a and, transposed, into s.b; then L L^T
-                const int gx = threadIdx.x & 15, gy = threadIdx.x >> 4;
-#pragma unroll
-                for (int u = 0; u < 4; ++u)
-#pragma unroll
-                    for (int v = 0; v < 4; ++v) {
-                        s.a[gy + 16 * u][gx + 16 * v] = acc[u][v];
-                        s.b[gx + 16 * v][gy + 16 * u] = acc[u][v];
-                        acc[u][v] = 0.f;
-                    }
-                __syncthreads();
-                if (threadIdx.x == 0) signal(ctr_tdone(p) + q * NB + q - 1);
-                mac_blk(s, acc);
-                __syncthreads();
-                potrf_inv_block(p, q, s, acc);
-            } else {
-                potrf_inv_block(p, it.q, s);
-            }
-        } else if (it.kind == K_T) {
+        zero_acc(acc);
+        if (it.kind == K_T) {
             // L_iq = A_iq X_qq^T, in place
-            float *c = p.W + (int64_t)it.i * DB * b + it.q * DB;
-            load_blk(s.a, c, b, false);
-            load_blk(s.b, p.X + (int64_t)it.q * DB * b + it.q * DB, b, true);
-            __syncthreads();
-            mac_blk(s, acc);
-            __syncthreads();
-            store_blk(c, b, acc, 1.f, 0.f);
+            float *c = blk(p.W, it.i, it.q);
+            if (t == 0) ok_s = (wait_ge(upd + it.i * NB + it.q, it.q, p) && wait_ge(pdone + it.q, 1, p)) ? 1 : 0;
+            csync();
+            if (!ok_s) break;
+            load_async(s[0], c, b, t, DC);
+            load_async(s[1], blk(p.X, it.q, it.q), b, t, DC);
+            load_commit();
+            load_wait_all();
+            csync();
+            mac_nt(s[0], s[1], acc);
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+#pragma unroll
+                for (int v = 0; v < 4; ++v) __stcg(c + (int64_t)(ty + 16 * u) * b + tx + 16 * v, acc[u][v]);
+            csync();
+            if (t == 0) signal(tdone + it.i * NB + it.q);
         } else if (it.kind == K_U) {
             // A_ij -= L_iq L_jq^T
-            load_blk(s.a, p.W + (int64_t)it.i * DB * b + it.q * DB, b, false);
-            load_blk(s.b, p.W + (int64_t)it.j * DB * b + it.q * DB, b, true);
-            __syncthreads();
-            mac_blk(s, acc);
-            __syncthreads();
-            store_blk(p.W + (int64_t)it.i * DB * b + it.j * DB, b, acc, -1.f, 1.f);
-        } else if (it.kind == K_I1 || it.kind == K_I2) {
-            const int64_t nb = (int64_t)1 << it.level, sz = nb * DB, base = 2 * it.pair * sz;
-            // products of level l after those of levels 0 .. l - 1 (each level
-            // NB * 2^l * DB * DB / 2 floats): levels run concurrently
-            float *tp = p.tmp + (int64_t)p.NB * (nb - 1) * (DB * DB / 2) + (int64_t)it.pair * sz * sz;
-            if (it.kind == K_I1) {
-                // T_p[a][c] = sum_{k >= c} L21[a][k] X11[k][c]
-                for (int64_t kk = it.c; kk < nb; ++kk) {
-                    load_blk(s.a, p.W + (base + sz + it.a * DB) * b + base + kk * DB, b, false);
-                    load_blk(s.b, p.X + (base + kk * DB) * b + base + it.c * DB, b, false);
-                    __syncthreads();
-                    mac_blk(s, acc);
-                    __syncthreads();
+            if (t == 0)
+                ok_s = (wait_ge(upd + it.i * NB + it.j, it.q, p) && wait_ge(tdone + it.j * NB + it.q, 1, p) &&
+                        wait_ge(tdone + it.i * NB + it.q, 1, p)) ? 1 : 0;
+            csync();
+            if (!ok_s) break;
+            load_async(s[0], blk(p.W, it.i, it.q), b, t, DC);
+            load_async(s[1], blk(p.W, it.j, it.q), b, t, DC);
+            load_commit();
+            float *c = blk(p.W, it.i, it.j);
+            float old[4][4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+#pragma unroll
+                for (int v = 0; v < 4; ++v) old[u][v] = __ldcg(c + (int64_t)(ty + 16 * u) * b + tx + 16 * v);
+            load_wait_all();
+            csync();
+            mac_nt(s[0], s[1], acc);
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+#pragma unroll
+                for (int v = 0; v < 4; ++v) __stcg(c + (int64_t)(ty + 16 * u) * b + tx + 16 * v, old[u][v] - acc[u][v]);
+            csync();
+            if (t == 0) signal(upd + it.i * NB + it.j);
+        } else if (it.i == it.j) {
+            // FP16 split of X_ii (the chain wrote X_ii and its transpose)
+            if (t == 0) ok_s = wait_ge(pdone + it.i, 1, p) ? 1 : 0;
+            csync();
+            if (!ok_s) break;
+            if (p.hi) {
+                const float *src = blk(p.X, it.i, it.i);
+                const int64_t o0 = (int64_t)it.i * DB * b + (int64_t)it.i * DB;
+                for (int e = t; e < DB * DB; e += DC) {
+                    const int64_t o = (int64_t)(e / DB) * b + e % DB;
+                    const float v = __ldcg(src + o);
+                    const __half h = __float2half_rn(v);
+                    p.hi[o0 + o] = h;
+                    p.lo[o0 + o] = __float2half_rn(v - __half2float(h));
                 }
-                store_blk(tp + (int64_t)it.a * DB * sz + it.c * DB, sz, acc, 1.f, 0.f);
-            } else {
-                // X21[a][c] = -sum_{k <= a} X22[a][k] T_p[k][c]
-                for (int64_t kk = 0; kk <= it.a; ++kk) {
-                    load_blk(s.a, p.X + (base + sz + it.a * DB) * b + base + sz + kk * DB, b, false);
-                    load_blk(s.b, tp + kk * DB * sz + it.c * DB, sz, false);
-                    __syncthreads();
-                    mac_blk(s, acc);
-                    __syncthreads();
-                }
-                store_blk(p.X + (base + sz + it.a * DB) * b + base + it.c * DB, b, acc, -1.f, 0.f);
             }
         } else {
-            // block (r, cb) of X: transpose into X^T and the FP16 split
-            const int r = it.i, cb = it.j;
-            const float *src = p.X + (int64_t)r * DB * b + cb * DB;
-            load_blk(s.a, src, b, false);
-            __syncthreads();
-            for (int e = threadIdx.x; e < DB * DB; e += DT) {
-                const int rr = e / DB, cc = e % DB;
-                // X^T block (cb, r): element (cc, rr) = X (rr, cc)
-                __stcg(p.XT + ((int64_t)cb * DB + rr) * b + r * DB + cc, s.a[cc][rr]);
-                if (p.hi) {
-                    const float v = s.a[rr][cc];
-                    const __half h = __float2half_rn(v);
-                    const int64_t o = ((int64_t)r * DB + rr) * b + cb * DB + cc;
-                    p.hi[o] = h;
-                    p.lo[o] = __float2half_rn(v - __half2float(h));
+            // X_ij = -X_ii sum_{j <= k < i} L_ik X_kj: the operands of step k + 1
+            // are copied in while step k is multiplied, as far as they are ready
+            const int i = it.i, j = it.j, len = i - j;
+            auto dep = [&](int k) { return (k == j) ? pdone + j : xdone + k * NB + j; };
+            if (t < len) {
+                const int k = j + t;
+                rdy[t] = (ld_acquire(tdone + i * NB + k) >= 1 && ld_acquire(dep(k)) >= 1) ? 1 : 0;
+            }
+            csync();
+            bool ok = true;
+            auto issue = [&](int e) -> bool {
+                const int k = j + e;
+                if (!rdy[e]) {
+                    if (t == 0) ok_s = (wait_ge(tdone + i * NB + k, 1, p) && wait_ge(dep(k), 1, p)) ? 1 : 0;
+                    csync();
+                    if (!ok_s) return false;
                 }
+                load_async(s[2 * (e & 1)], blk(p.W, i, k), b, t, DC);
+                load_async(s[2 * (e & 1) + 1], blk(p.XT, j, k), b, t, DC);
+                load_commit();
+                return true;
+            };
+            ok = issue(0);
+            int issued = 1;
+            for (int e = 0; e < len && ok; ++e) {
+                if (issued == e) {  // step e was not ready when step e - 1 ran
+                    ok = issue(e);
+                    if (!ok) break;
+                    ++issued;
+                }
+                if (e + 1 < len && rdy[e + 1]) {
+                    issue(e + 1);
+                    ++issued;
+                    load_wait_but1();
+                } else {
+                    load_wait_all();
+                }
+                csync();
+                mac_nt(s[2 * (e & 1)], s[2 * (e & 1) + 1], acc);
+                csync();
             }
-        }
-        __syncthreads();
-        // ---- publish
-        if (threadIdx.x == 0) {
-            if (it.kind == K_P) {
-                signal(ctr_pdone(p) + it.q);
-            } else if (it.kind == K_T) {
-                signal(ctr_tdone(p) + it.i * NB + it.q);
-            } else if (it.kind == K_U) {
-                signal(ctr_upd(p) + it.i * NB + it.j);
-            } else if (it.kind == K_I1) {
-                signal(ctr_i1done(p) + pair_slot(p, it.level, it.pair));
-            } else if (it.kind == K_I2) {
-                signal(ctr_i2done(p) + pair_slot(p, it.level, it.pair));
+            if (!ok) break;
+            if (t == 0) ok_s = wait_ge(pdone + i, 1, p) ? 1 : 0;
+            // the sum, transposed, is the second operand
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+#pragma unroll
+                for (int v = 0; v < 4; ++v) s[1][tx + 16 * v][ty + 16 * u] = acc[u][v];
+            csync();
+            if (!ok_s) break;
+            load_async(s[0], blk(p.X, i, i), b, t, DC);
+            load_commit();
+            load_wait_all();
+            csync();
+            zero_acc(acc);
+            mac_nt(s[0], s[1], acc);
+            float *gx = blk(p.X, i, j);
+            const int64_t o0 = (int64_t)i * DB * b + (int64_t)j * DB;
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+#pragma unroll
+                for (int v = 0; v < 4; ++v) {
+                    const int64_t o = (int64_t)(ty + 16 * u) * b + tx + 16 * v;
+                    const float x = -acc[u][v];
+                    __stcg(gx + o, x);
+                    s[2][tx + 16 * v][ty + 16 * u] = x;
+                    if (p.hi) {
+                        const __half h = __float2half_rn(x);
+                        p.hi[o0 + o] = h;
+                        p.lo[o0 + o] = __float2half_rn(x - __half2float(h));
+                    }
+                }
+            csync();
+            float *gt = blk(p.XT, j, i);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int r = ty + 16 * u;
+                __stcg(reinterpret_cast<float4 *>(gt + (int64_t)r * b + 4 * tx),
+                       *reinterpret_cast<const float4 *>(&s[2][r][4 * tx]));
             }
+            csync();
+            if (t == 0) signal(xdone + i * NB + j);
         }
+        csync();  // the buffers and flags are free
     }
+    load_wait_all();
 }
+
+constexpr size_t diag_smem_bytes() { return 4 * sizeof(Blk); }
 
 }  // namespace
 
 int64_t diag_counter_count(int64_t b) {
     const int64_t NB = b / DB;
-    return 2 + NB + 2 * NB * NB + 2 * NB;
+    return 2 + NB + 3 * NB * NB;
 }
 
 // Factor + inverse of diagonal tile k in FP32 (W in place, Linv, LinvT and
-// the FP16 split of Linv when present).  The counters `ctr` hold
-// diag_counter_count(b) ints.
-krr_status launch_diag_dataflow(Ctx *c, int64_t k, float *W, float *X, float *XT, __half *hi, __half *lo,
-                                float *tmp, int *ctr, double *minpiv, cudaStream_t s, int64_t cta_cap) {
+// the FP16 split of Linv when present; these are zero above the diagonal from
+// their allocation on).  The counters `ctr` hold diag_counter_count(b) ints;
+// lkk receives the square root of the tile's largest diagonal entry.
+krr_status launch_diag_dataflow(Ctx *c, int64_t k, float *W, float *X, float *XT, __half *hi, __half *lo, int *ctr,
+                                double *lkk, cudaStream_t s, int64_t cta_cap) {
     const int64_t b = c->b;
     if (b % DB != 0 || b / DB > DMAX_NB) {
         c->last_error = "diagonal step: tile edge must be a multiple of 64 and at most 4096";
         return KRR_EINVAL;
+    }
+    static PerDevice attr;
+    if (!attr.has(c->device)) {
+        KRR_CUDA_TRY(c, cudaFuncSetAttribute(diag_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)diag_smem_bytes()));
+        attr.put(c->device);
     }
     DiagParams p;
     memset(&p, 0, sizeof(p));
@@ -660,27 +792,20 @@ krr_status launch_diag_dataflow(Ctx *c, int64_t k, float *W, float *X, float *XT
     p.XT = XT;
     p.hi = hi;
     p.lo = lo;
-    p.tmp = tmp;
     p.b = b;
     p.NB = (int)(b / DB);
-    int levels = 0;
-    while (((int64_t)DB << levels) < b) ++levels;
-    p.levels = levels;
     p.tile_k = k;
-    p.n_factor = factor_items_for(p.NB);
-    int64_t inv = 0;
-    for (int l = 0; l < levels; ++l) inv += 2 * inv_step_items(p.NB, l);
-    p.items = p.n_factor + inv + (int64_t)p.NB * p.NB;
+    p.items = item_count(p.NB);
     p.ctr = ctr;
-    p.minpiv = minpiv;
+    p.lkk = lkk;
     p.err = c->derr;
     p.wait_ns = (uint64_t)c->opt.wait_budget_ns;
     KRR_CUDA_TRY(c, cudaMemsetAsync(ctr, 0, (size_t)diag_counter_count(b) * sizeof(int), s));
-    KRR_CUDA_TRY(c, cudaMemsetAsync(X, 0, (size_t)b * b * sizeof(float), s));
     int64_t gl = grid_limit(c, GL_DIAG);
     if (cta_cap > 0 && cta_cap < gl) gl = cta_cap;
-    const int64_t grid = std::min<int64_t>(gl, std::max<int64_t>(p.NB * (p.NB + 1) / 2, 1));
-    count_launch(), diag_kernel<<<(unsigned)grid, DT, 0, s>>>(p);
+    // the chain CTA and at least one other
+    const int64_t grid = std::max<int64_t>(2, std::min<int64_t>(gl, p.NB * (p.NB + 1) / 2));
+    count_launch(), diag_kernel<<<(unsigned)grid, DT, diag_smem_bytes(), s>>>(p);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
         c->last_error = std::string("diagonal step launch: ") + cudaGetErrorString(e);

@@ -818,8 +818,13 @@ krr_status krr_factor(krr_ctx *c, double lambda, krr_factor_info *info) {
         KRR_TRY(dev_alloc(c, &c->Wd, (size_t)nt * bb, "diagonal tiles"));
         KRR_TRY(dev_alloc(c, &c->Linv, (size_t)nt * bb, "diagonal inverses"));
         KRR_TRY(dev_alloc(c, &c->LinvT, (size_t)nt * bb, "transposed diagonal inverses"));
-        KRR_TRY(dev_alloc(c, &c->diag64, (size_t)bb, "FP64 diagonal scratch"));
-        KRR_TRY(dev_alloc(c, &c->diag64_inv, (size_t)2 * bb, "FP64 inverse scratch"));
+        // the diagonal step writes the inverses on and below the diagonal only
+        KRR_CUDA_TRY(c, cudaMemsetAsync(c->Linv, 0, (size_t)nt * bb * sizeof(float), s));
+        KRR_CUDA_TRY(c, cudaMemsetAsync(c->LinvT, 0, (size_t)nt * bb * sizeof(float), s));
+        if (c->opt.diag_fp64) {
+            KRR_TRY(dev_alloc(c, &c->diag64, (size_t)bb, "FP64 diagonal scratch"));
+            KRR_TRY(dev_alloc(c, &c->diag64_inv, (size_t)2 * bb, "FP64 inverse scratch"));
+        }
         KRR_TRY(dev_alloc(c, &c->diag_ctr, (size_t)diag_counter_count(b), "diagonal-step counters"));
         const size_t pool_bytes = (size_t)std::max<int64_t>(noff, 1) * bb * 4;
         KRR_TRY(dev_alloc(c, &c->pool, pool_bytes, "factor pool"));
@@ -829,6 +834,8 @@ krr_status krr_factor(krr_ctx *c, double lambda, krr_factor_info *info) {
         if (mx) {
             KRR_TRY(dev_alloc(c, &c->Linv_hi, (size_t)nt * bb, "inverse split"));
             KRR_TRY(dev_alloc(c, &c->Linv_lo, (size_t)nt * bb, "inverse split"));
+            KRR_CUDA_TRY(c, cudaMemsetAsync(c->Linv_hi, 0, (size_t)nt * bb * sizeof(__half), s));
+            KRR_CUDA_TRY(c, cudaMemsetAsync(c->Linv_lo, 0, (size_t)nt * bb * sizeof(__half), s));
             const size_t colt = (size_t)std::max<int64_t>(nt - 1, 1);
             KRR_TRY(dev_alloc(c, &c->colbuf, colt * bb, "column buffer"));
             KRR_TRY(dev_alloc(c, &c->pan_hi, colt * bb, "operand panel"));

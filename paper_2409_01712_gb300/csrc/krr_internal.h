@@ -377,10 +377,10 @@ void launch_predict_simt(Ctx *c, const float *tf, const int32_t *tn, int64_t n_t
 
 // Diagonal-step dataflow kernel (diag.cu): FP32 factor of tile W, inverse X,
 // its transpose XT and FP16 split hi/lo (optional); ctr holds
-// diag_counter_count(b) ints, minpiv b / 64 doubles.
+// diag_counter_count(b) ints; lkk receives sqrt of the largest diagonal entry.
 int64_t diag_counter_count(int64_t b);
-krr_status launch_diag_dataflow(Ctx *c, int64_t k, float *W, float *X, float *XT, __half *hi, __half *lo,
-                                float *tmp, int *ctr, double *minpiv, cudaStream_t s, int64_t cta_cap);
+krr_status launch_diag_dataflow(Ctx *c, int64_t k, float *W, float *X, float *XT, __half *hi, __half *lo, int *ctr,
+                                double *lkk, cudaStream_t s, int64_t cta_cap);
 
 // Diagonal step: in-place Cholesky of Wd tile k and its inverse into Linv.
 // Factor and inverse of diagonal tile k, on stream s (nullptr: the context's

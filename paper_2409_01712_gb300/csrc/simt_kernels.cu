@@ -791,8 +791,8 @@ krr_status diag_step(Ctx *c, int64_t k, cudaStream_t s, int64_t cta_cap) {
     double *lkk = c->red + RED_MINPIV + c->nt * nq;
     unsigned g = cdiv(bb, 256);
     if (k == 0) count_launch(), copy_add_diag_kernel<<<g, 256, 0, s>>>(c->Kd, wd, bb, (float)c->lambda, b);
-    count_launch(), diag_max_kernel<<<1, 256, 0, s>>>(wd, b, lkk + k);
     if (c->opt.diag_fp64) {
+        count_launch(), diag_max_kernel<<<1, 256, 0, s>>>(wd, b, lkk + k);
         count_launch(), f32_to_f64_kernel<<<g, 256, 0, s>>>(wd, c->diag64, bb, 0.0, b);
         diag_factor_tile<double>(c, c->diag64, c->diag64_inv, c->diag64_inv + bb, k, minpiv);
         count_launch(), f64_to_f32_kernel<<<g, 256, 0, s>>>(c->diag64, wd, bb);
@@ -801,14 +801,13 @@ krr_status diag_step(Ctx *c, int64_t k, cudaStream_t s, int64_t cta_cap) {
                                                 c->Linv_lo ? c->Linv_lo + k * bb : nullptr, bb);
         count_launch(), transpose_kernel<<<dim3((unsigned)(b / 32), (unsigned)(b / 32)), dim3(32, 8), 0, s>>>(
             linv, c->LinvT + k * bb, b);
-    } else {
-        // one dataflow launch: factor, inverse, transpose and FP16 split
-        KRR_TRY(launch_diag_dataflow(c, k, wd, linv, c->LinvT + k * bb, c->Linv_hi ? c->Linv_hi + k * bb : nullptr,
-                                     c->Linv_lo ? c->Linv_lo + k * bb : nullptr, (float *)c->diag64, c->diag_ctr,
-                                     minpiv + k * nq, s, cta_cap));
+        count_launch(), min_pivot_kernel<<<1, 1, 0, s>>>(minpiv + k * nq, nq, c->derr);
+        return KRR_OK;
     }
-    count_launch(), min_pivot_kernel<<<1, 1, 0, s>>>(minpiv + k * nq, nq, c->derr);
-    return KRR_OK;
+    // one dataflow launch: factor, inverse, transpose, FP16 split, the largest
+    // diagonal entry and the smallest pivot
+    return launch_diag_dataflow(c, k, wd, linv, c->LinvT + k * bb, c->Linv_hi ? c->Linv_hi + k * bb : nullptr,
+                                c->Linv_lo ? c->Linv_lo + k * bb : nullptr, c->diag_ctr, lkk + k, s, cta_cap);
 }
 
 // ----------------------------------------------------------------------------

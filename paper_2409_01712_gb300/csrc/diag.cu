@@ -26,13 +26,17 @@
 // diagonal are zero from the allocation on.
 // Progress counters: pdone[q], tdone[i][q], upd[i][j] (updates applied to block
 // (i, j)), xdone[i][j].  Items wait only for items claimed before them by
-// running CTAs and for the chain, which waits only for such items; every wait
-// is bounded (%globaltimer) and ends the kernel with KRR_ETIMEOUT.  Blocks
-// written by other CTAs are read through L2 (ld.global.cg, cp.async.cg).
+// running CTAs and for the chain, which waits only for such items.  CTAs are
+// launched in clusters of two, so at least one other CTA runs with the chain
+// and the kernel progresses however many more find an SM.  Every wait is
+// bounded (%globaltimer) and ends the kernel with KRR_ETIMEOUT.  Blocks written
+// by other CTAs are read through L2 (ld.global.cg, cp.async.cg).
 //
 // What bounds it: latency.  A link of the chain is one 64 x 64 x 64 product,
 // half of one, and the 64-column factor, whose pivots are serial.  One
-// tile of b = 1024 alone takes 0.27 ms and one of 256 0.07 ms; with the chain's
+// tile of b = 1024 alone takes 0.266 ms (a link 16 us: the first product 1.4,
+// the second 1.7 and its store 0.6, the 64-column factor 11, the stores 0.8) and
+// one of 256 0.07 ms; with the chain's
 // blocks as items of the common queue (every link paying a claim, the wait for
 // the counters, the loads and the publication) and the inverse by recursive
 // doubling after the factorisation it was 0.50 and 0.12 ms.
@@ -257,17 +261,28 @@ __device__ __forceinline__ void mac_nt(const Blk &a, const Blk &b, float (&acc)[
     }
 }
 
-// acc += A E (E row-major along its columns): the thread owns rows ty + 16 u
-// and columns 4 tx + v.
+// acc = A E, E upper triangular in 16 x 16 blocks (entry (k, j) zero for k's
+// block > j's).  A warp owns 16 columns and 32 rows, a thread 4 x 4 of them
+// (nn_row, nn_col), and stops at its last nonzero block row; the column blocks
+// are dealt to the warps so that the warps of a scheduler share the work
+// evenly.  A block product moves half a shared-memory value per FMA into
+// registers, 128 bytes a cycle, which bounds it: 3800 cycles in full.
+__device__ __forceinline__ int nn_block() {
+    const int w = threadIdx.x >> 6;  // two warps per block of columns
+    return w < 2 ? w : 5 - w;
+}
+__device__ __forceinline__ int nn_row() { return ((threadIdx.x >> 5) & 1) * 32 + ((threadIdx.x & 31) >> 2) * 4; }
+__device__ __forceinline__ int nn_col() { return 16 * nn_block() + (threadIdx.x & 3) * 4; }
+
 __device__ __forceinline__ void mac_nn(const Blk &a, const Blk &e, float (&acc)[4][4]) {
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    const int r = nn_row(), c = nn_col(), kend = 16 * (nn_block() + 1);
 #pragma unroll 4
-    for (int k = 0; k < DB; k += 4) {
+    for (int k = 0; k < kend; k += 4) {
         float4 av[4], ev[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) av[u] = *reinterpret_cast<const float4 *>(&a[ty + 16 * u][k]);
+        for (int u = 0; u < 4; ++u) av[u] = *reinterpret_cast<const float4 *>(&a[r + u][k]);
 #pragma unroll
-        for (int s = 0; s < 4; ++s) ev[s] = *reinterpret_cast<const float4 *>(&e[k + s][4 * tx]);
+        for (int s = 0; s < 4; ++s) ev[s] = *reinterpret_cast<const float4 *>(&e[k + s][c]);
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             const float as[4] = {av[u].x, av[u].y, av[u].z, av[u].w};
@@ -287,6 +302,88 @@ __device__ __forceinline__ void zero_acc(float (&acc)[4][4]) {
     for (int u = 0; u < 4; ++u)
 #pragma unroll
         for (int v = 0; v < 4; ++v) acc[u][v] = 0.f;
+}
+
+// Steps 2 and 3 (below) of 16-column block Q of chol_inv_64 on 256 threads:
+// thread (tc, tr) = (t % 16, t / 16) holds entry (tr, tc) of every 16 x 16
+// block.  Q is a template parameter so that the sums of all blocks are
+// straight code and run beside each other (16 dependent FMAs each; as a loop
+// over a run-time Q step 3 took 1400 cycles, 910 now: the
+// shared-memory loads of its 3 x 4 operands).
+template <int Q>
+__device__ __forceinline__ void eliminate_16(Blk &a, Blk &e) {
+    constexpr int o = 16 * Q, NA = 3 - Q;  // block rows of A below, of E above (Q of them)
+    const int tc = threadIdx.x & 15, tr = threadIdx.x >> 4;
+    {
+        float ecol[16], acc[3];
+        float4 r4[3][4];
+#pragma unroll
+        for (int m = 0; m < 16; ++m) ecol[m] = e[o + m][o + tc];
+#pragma unroll
+        for (int u = 0; u < 3; ++u) {
+            const float *row = (u < NA) ? &a[16 * (Q + 1 + u) + tr][o] : &e[16 * (u - NA) + tr][o];
+#pragma unroll
+            for (int m = 0; m < 4; ++m) r4[u][m] = *reinterpret_cast<const float4 *>(row + 4 * m);
+            acc[u] = 0.f;
+        }
+#pragma unroll
+        for (int m = 0; m < 4; ++m)
+#pragma unroll
+            for (int u = 0; u < 3; ++u) {
+                acc[u] = fmaf(r4[u][m].x, ecol[4 * m], acc[u]);
+                acc[u] = fmaf(r4[u][m].y, ecol[4 * m + 1], acc[u]);
+                acc[u] = fmaf(r4[u][m].z, ecol[4 * m + 2], acc[u]);
+                acc[u] = fmaf(r4[u][m].w, ecol[4 * m + 3], acc[u]);
+            }
+        __syncwarp();  // the 16 threads of a row share a warp
+#pragma unroll
+        for (int u = 0; u < 3; ++u) {
+            float *row = (u < NA) ? &a[16 * (Q + 1 + u) + tr][o] : &e[16 * (u - NA) + tr][o];
+            row[tc] = acc[u];
+        }
+    }
+    csync();
+    if constexpr (Q < 3) {
+        // block (u, w): block row u of the NA of A (lower ones only) or of the
+        // Q + 1 of E, columns of block Q + 1 + w
+        float acc[4][3];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+            for (int w = 0; w < 3; ++w) acc[u][w] = 0.f;
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+            float4 lj[3], li[4];
+#pragma unroll
+            for (int w = 0; w < NA; ++w) lj[w] = *reinterpret_cast<const float4 *>(&a[o + 16 + 16 * w + tc][o + 4 * m]);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const float *row = (u < NA) ? a[16 * (Q + 1 + u) + tr] : e[16 * (u - NA) + tr];
+                li[u] = *reinterpret_cast<const float4 *>(row + o + 4 * m);
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+#pragma unroll
+                for (int w = 0; w < NA; ++w) {
+                    if (u < NA && w > u) continue;
+                    acc[u][w] = fmaf(li[u].x, lj[w].x, acc[u][w]);
+                    acc[u][w] = fmaf(li[u].y, lj[w].y, acc[u][w]);
+                    acc[u][w] = fmaf(li[u].z, lj[w].z, acc[u][w]);
+                    acc[u][w] = fmaf(li[u].w, lj[w].w, acc[u][w]);
+                }
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+            for (int w = 0; w < NA; ++w) {
+                if (u < NA && w > u) continue;
+                float *dst = ((u < NA) ? a[16 * (Q + 1 + u) + tr] : e[16 * (u - NA) + tr]) + o + 16 + 16 * w + tc;
+                // block row Q of E enters here: its entries right of the diagonal
+                // block were zero
+                *dst = ((u - NA == Q) ? 0.f : *dst) - acc[u][w];
+            }
+        csync();
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -309,7 +406,6 @@ __device__ __forceinline__ void zero_acc(float (&acc)[4][4]) {
 // ---------------------------------------------------------------------------
 __device__ void chol_inv_64(Blk &a, Blk &e, int &bad, float &mpiv) {
     const int t = threadIdx.x, lane = t & 31;
-    const int tc = t & 15, tr = t >> 4;
     const unsigned FULL = 0xffffffffu;
 #pragma unroll 1
     for (int q = 0; q < 4; ++q) {
@@ -354,65 +450,11 @@ __device__ void chol_inv_64(Blk &a, Blk &e, int &bad, float &mpiv) {
             }
         }
         csync();
-        // active rows: blocks q + 1 .. 3 of A and 0 .. q - 1 of E
-        {
-            float ecol[16];
-#pragma unroll
-            for (int m = 0; m < 16; ++m) ecol[m] = e[o + m][o + tc];
-#pragma unroll
-            for (int u = 0; u < 3; ++u) {
-                const int rb = (u < 3 - q) ? q + 1 + u : u - (3 - q);
-                float *row = (u < 3 - q) ? &a[16 * rb + tr][o] : &e[16 * rb + tr][o];
-                float acc = 0.f;
-#pragma unroll
-                for (int m = 0; m < 16; m += 4) {
-                    const float4 r4 = *reinterpret_cast<const float4 *>(row + m);
-                    acc = fmaf(r4.x, ecol[m], acc);
-                    acc = fmaf(r4.y, ecol[m + 1], acc);
-                    acc = fmaf(r4.z, ecol[m + 2], acc);
-                    acc = fmaf(r4.w, ecol[m + 3], acc);
-                }
-                __syncwarp();  // the 16 threads of a row share a warp
-                row[tc] = acc;
-            }
-        }
-        csync();
-        if (q < 3) {
-            float4 lj[3][4];
-#pragma unroll
-            for (int w = 0; w < 3; ++w)
-                if (w < 3 - q)
-#pragma unroll
-                    for (int m = 0; m < 4; ++m)
-                        lj[w][m] = *reinterpret_cast<const float4 *>(&a[o + 16 + 16 * w + tc][o + 4 * m]);
-            // row blocks: 3 - q of A (lower blocks only), then q + 1 of E
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const bool in_a = u < 3 - q;
-                const int rb = in_a ? q + 1 + u : u - (3 - q);
-                float *row = in_a ? a[16 * rb + tr] : e[16 * rb + tr];
-                float4 li[4];
-#pragma unroll
-                for (int m = 0; m < 4; ++m) li[m] = *reinterpret_cast<const float4 *>(row + o + 4 * m);
-#pragma unroll
-                for (int w = 0; w < 3; ++w) {
-                    if (w < 3 - q && (!in_a || w <= u)) {
-                        float acc = 0.f;
-#pragma unroll
-                        for (int m = 0; m < 4; ++m) {
-                            acc = fmaf(li[m].x, lj[w][m].x, acc);
-                            acc = fmaf(li[m].y, lj[w][m].y, acc);
-                            acc = fmaf(li[m].z, lj[w][m].z, acc);
-                            acc = fmaf(li[m].w, lj[w][m].w, acc);
-                        }
-                        float *dst = row + o + 16 + 16 * w + tc;
-                        // block row q of E enters here: its entries right of
-                        // the diagonal block were zero
-                        *dst = ((!in_a && rb == q) ? 0.f : *dst) - acc;
-                    }
-                }
-            }
-            csync();
+        switch (q) {
+            case 0: eliminate_16<0>(a, e); break;
+            case 1: eliminate_16<1>(a, e); break;
+            case 2: eliminate_16<2>(a, e); break;
+            default: eliminate_16<3>(a, e);
         }
     }
 }
@@ -485,18 +527,18 @@ __device__ void chain(const DiagParams &p, Blk *s, ChainBars &cb) {
     const int tx = t & 15, ty = t >> 4;
     int bad = -1;
     float mpiv = 3.0e38f;
-    // the publication two before this one on the same barrier is through (it
-    // always is: a link takes several times a publication)
+    // One thread of a warp off the pivot path arrives and waits for all.  The
+    // publication before this one on the same barrier is through (it always
+    // is: a link takes several times a publication).
     auto arrive_pub = [&](uint64_t *bar, int seq) {
-        __syncwarp();
-        if (lane == 0) {
+        if (t == 255) {
             const uint64_t t0 = globaltimer();
             while (cb.pubseq < seq - 2 && globaltimer() - t0 < 4 * p.wait_ns && !*(volatile int *)&p.ctr[1]) {}
             mbar_arrive(bar);
         }
     };
     for (int q = 0; q < NB; ++q) {
-        if (t == 0) cb.ok = wait_bar(&cb.full, q & 1, p) ? 1 : 0;
+        if (t == 255) cb.ok = wait_bar(&cb.full, q & 1, p) ? 1 : 0;
         csync();
         if (!cb.ok) return;
         Blk &A = s[2 + (q & 1)];
@@ -510,11 +552,12 @@ __device__ void chain(const DiagParams &p, Blk *s, ChainBars &cb) {
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 const float4 w = make_float4(acc[u][0], acc[u][1], acc[u][2], acc[u][3]);
-                *reinterpret_cast<float4 *>(&s[1][ty + 16 * u][4 * tx]) = w;
-                __stcg(reinterpret_cast<float4 *>(g + (int64_t)(ty + 16 * u) * b + 4 * tx), w);
+                const int r = nn_row() + u, c = nn_col();
+                *reinterpret_cast<float4 *>(&s[1][r][c]) = w;
+                __stcg(reinterpret_cast<float4 *>(g + (int64_t)r * b + c), w);
             }
-            arrive_pub(&cb.pubt, 2 * q);
             csync();
+            arrive_pub(&cb.pubt, 2 * q);
             // A_qq -= L_q,q-1 L_q,q-1^T (lower blocks)
             zero_acc(acc);
             mac_nt<true>(s[1], s[1], acc);
@@ -524,7 +567,7 @@ __device__ void chain(const DiagParams &p, Blk *s, ChainBars &cb) {
                 for (int v = 0; v <= u; ++v) A[ty + 16 * u][tx + 16 * v] -= acc[u][v];
             csync();
         }
-        if (t == 0) mbar_arrive(&cb.s1free);
+        if (t == 255) mbar_arrive(&cb.s1free);
         int bq = -1;
         chol_inv_64(A, s[0], bq, mpiv);
         if (bq >= 0 && bad < 0) bad = q * DB + bq;
@@ -559,8 +602,8 @@ __device__ void chain(const DiagParams &p, Blk *s, ChainBars &cb) {
                    make_float4(c <= r ? l.x : 0.f, c + 1 <= r ? l.y : 0.f, c + 2 <= r ? l.z : 0.f,
                                c + 3 <= r ? l.w : 0.f));
         }
-        arrive_pub(&cb.pubp, 2 * q + 1);
         csync();
+        arrive_pub(&cb.pubp, 2 * q + 1);
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             const int r = ty + 16 * u, c = 4 * tx;
@@ -576,7 +619,10 @@ __device__ void chain(const DiagParams &p, Blk *s, ChainBars &cb) {
     }
 }
 
-__global__ void __launch_bounds__(DT) diag_kernel(const DiagParams p) {
+// (Without a bound ptxas takes 96 registers and spills; at the 168 that one CTA
+// per SM allows the pivot loop comes out slower than at 144: 0.280 against
+// 0.267 ms a tile of 1024.)
+__global__ void __maxnreg__(144) diag_kernel(const DiagParams p) {
     extern __shared__ __align__(16) float diag_smem[];
     Blk *s = reinterpret_cast<Blk *>(diag_smem);  // four blocks
     __shared__ ChainBars cb;
@@ -590,8 +636,8 @@ __global__ void __launch_bounds__(DT) diag_kernel(const DiagParams p) {
         if (t == 0) {
             mbar_init(&cb.full, 1);
             mbar_init(&cb.s1free, 1);
-            mbar_init(&cb.pubt, DC / 32);
-            mbar_init(&cb.pubp, DC / 32);
+            mbar_init(&cb.pubt, 1);
+            mbar_init(&cb.pubp, 1);
             cb.pubseq = 0;
         }
         __syncthreads();
@@ -803,11 +849,25 @@ krr_status launch_diag_dataflow(Ctx *c, int64_t k, float *W, float *X, float *XT
     KRR_CUDA_TRY(c, cudaMemsetAsync(ctr, 0, (size_t)diag_counter_count(b) * sizeof(int), s));
     int64_t gl = grid_limit(c, GL_DIAG);
     if (cta_cap > 0 && cta_cap < gl) gl = cta_cap;
-    // the chain CTA and at least one other
-    const int64_t grid = std::max<int64_t>(2, std::min<int64_t>(gl, p.NB * (p.NB + 1) / 2));
-    count_launch(), diag_kernel<<<(unsigned)grid, DT, diag_smem_bytes(), s>>>(p);
-    const cudaError_t e = cudaGetLastError();
+    // the chain CTA and at least one other, in clusters of two
+    const int64_t grid = std::max<int64_t>(2, std::min<int64_t>(gl, p.NB * (p.NB + 1) / 2)) / 2 * 2;
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof(cfg));
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 2;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3(DT);
+    cfg.dynamicSmemBytes = diag_smem_bytes();
+    cfg.stream = s;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    count_launch();
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, diag_kernel, p);
     if (e != cudaSuccess) {
+        cudaGetLastError();
         c->last_error = std::string("diagonal step launch: ") + cudaGetErrorString(e);
         return KRR_ECUDA;
     }

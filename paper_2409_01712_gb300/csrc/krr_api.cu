@@ -468,11 +468,6 @@ krr_status prepare_build(Ctx *c, int64_t n, int64_t m_pad, int keep_d) {
 }
 krr_status ensure_lookahead_stream(Ctx *c) {
     if (c->la_stream) return KRR_OK;
-    if (c->graph_mode) {
-        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-        KRR_CUDA_TRY(c, cudaStreamIsCapturing(c->stream, &cs));
-        if (cs != cudaStreamCaptureStatusNone) return KRR_OK;  // made before the capture, or not at all
-    }
     int lo = 0, hi = 0;
     KRR_CUDA_TRY(c, cudaDeviceGetStreamPriorityRange(&lo, &hi));
     KRR_CUDA_TRY(c, cudaStreamCreateWithPriority(&c->la_stream, cudaStreamNonBlocking, hi));
@@ -732,11 +727,11 @@ namespace {
 // takes 660 ms this way and 697 ms in sequence; fixed R = 24 and R = 48 gave
 // the same 658-662 ms, R = 8 690 ms.
 //
-// A context of a batch (graph mode) shares the GPU with the other problems
-// and its kernels are capped per class: there the diagonal step keeps its
-// class cap and the whole rest of the update runs beside it (on the
-// cross-validation workload, 64 problems: 170.4-171.8 ms per run against
-// 172.9-175.4 ms in sequence).
+// A context of a batch (graph mode) shares the GPU with the other problems,
+// whose updates fill the SMs that a diagonal step leaves free anyway: there
+// the plain sequence is faster (cross-validation over 6 cohorts of 1024 to
+// 16384 rows x 4 lambdas: 53.4 ms per run, 175 ms with the lookahead, whose
+// diagonal steps wait for SMs that their own problem's update holds).
 struct LookaheadPlan {
     bool on = false;
     int64_t ctas = 0, tiles = 0;  // 0 CTAs: the class limit
@@ -744,9 +739,7 @@ struct LookaheadPlan {
 };
 
 bool lookahead_enabled(const Ctx *c) {
-    // in graph mode the second stream must exist before the capture began
-    if (c->graph_mode && !c->la_stream) return false;
-    return c->opt.lookahead && mixed(c) && !c->opt.diag_fp64 && c->nt >= 3 && c->num_sms >= 32;
+    return c->opt.lookahead && !c->graph_mode && mixed(c) && !c->opt.diag_fp64 && c->nt >= 3 && c->num_sms >= 32;
 }
 
 LookaheadPlan lookahead_plan(const Ctx *c, int64_t k) {
@@ -754,11 +747,6 @@ LookaheadPlan lookahead_plan(const Ctx *c, int64_t k) {
     const int64_t u = c->nt - k - 1;
     const int64_t tiles = u * (u + 1) / 2;
     if (tiles < 2) return pl;
-    if (c->graph_mode) {
-        pl.on = true;
-        pl.tiles = tiles - 1;
-        return pl;
-    }
     const double bd = (double)c->b, rel = bd / 1024.0;
     const double a_us = 600.0 * rel, c_us = 13000.0 * rel * rel * rel;
     const double tile_sm_us = 2.0 * bd * bd * bd / 8.3e12 * 1e6;  // SM-microseconds per target tile

@@ -57,7 +57,8 @@ thread_local std::string g_batch_create_error;
 // at 16 / 24 (with the lookahead) 175 / 187 ms; diagonal step and sweeps
 // both at 8 195 ms; the pair kernels at 48 (sweeps 12) 194 ms: the chain of
 // the diagonal steps of the largest problems needs their CTAs, and more
-// CTAs crowd out the other problems.
+// CTAs crowd out the other problems.  (All of these with the diagonal step
+// before its chain had a CTA of its own, and most with the lookahead.)
 constexpr int BATCH_CTA_CAP = 32;
 constexpr int BATCH_CAP_DIAG = 12, BATCH_CAP_SWEEP = 16, BATCH_CAP_PAIR = 64, BATCH_CAP_SINGLE = 64;
 
@@ -99,10 +100,6 @@ krr_status trial_ms(const krr_options &base, cudaStream_t s, const krr_batch_pro
     KRR_TRY(krr_create(&c, &o, s));
     reinterpret_cast<krr::Ctx *>(c)->graph_mode = 1;
     set_batch_caps(c);
-    if (krr::ensure_lookahead_stream(reinterpret_cast<krr::Ctx *>(c)) != KRR_OK) {
-        krr_destroy(c);
-        return KRR_ECUDA;
-    }
     krr_status st = issue(c, pr, m, p);  // warm-up (allocations)
     if (st == KRR_OK) {
         cudaStreamSynchronize(s);
@@ -165,11 +162,6 @@ krr_status instantiate(krr_batch *bt, std::string *msg) {
         }
         reinterpret_cast<krr::Ctx *>(bt->ctx[i])->graph_mode = 1;
         set_batch_caps(bt->ctx[i]);
-        st = krr::ensure_lookahead_stream(reinterpret_cast<krr::Ctx *>(bt->ctx[i]));
-        if (st != KRR_OK) {
-            *msg = "krr_batch_create: lookahead stream";
-            return st;
-        }
         const int32_t ow = bt->owner[i];
         st = (ow == i) ? issue(bt->ctx[i], problems[i], m, p, nullptr, nullptr, bt->built[i])
                        : issue(bt->ctx[i], problems[i], m, p, bt->ctx[ow], bt->built[ow]);

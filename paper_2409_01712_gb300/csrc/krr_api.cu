@@ -297,10 +297,6 @@ bool mixed(const Ctx *c) { return c->opt.mode == KRR_MODE_MIXED; }
 }  // namespace krr
 
 namespace {
-// Scratch of the residual-norm reduction: the last norm_partial_count()
-// doubles of the reduction buffer.
-double *red_norm_part(Ctx *c) { return c->red + c->red_cap - norm_partial_count(); }
-
 // Allocates (or keeps) the n_pad x p work vectors of the solve.
 krr_status ensure_vectors(Ctx *c, int64_t p) {
     const int64_t cnt = c->n_pad * p;
@@ -324,7 +320,6 @@ krr_status ensure_vectors(Ctx *c, int64_t p) {
 krr_status solve_device(Ctx *c, int64_t p, krr_solve_info *info) {
     cudaStream_t s = c->stream;
     const int64_t cnt = c->n_pad * p;
-    KRR_CUDA_TRY(c, cudaMemcpyAsync(c->abuf, c->ybuf, cnt * sizeof(float), cudaMemcpyDeviceToDevice, s));
     // compulsory bytes of one pair of sweeps: the stored factor read twice
     // (diagonal inverses in FP32 plus the off-diagonal pool) and the vectors
     const double pool_used = mixed(c) ? (double)c->herr->pool_cursor
@@ -333,7 +328,7 @@ krr_status solve_device(Ctx *c, int64_t p, krr_solve_info *info) {
     const double sweep_bytes = 2.0 * factor_bytes_all + 4.0 * (double)cnt * 4.0;
     const double sweep_flops = 2.0 * 2.0 * (double)c->n_pad * c->n_pad * p;
     int pr = prof_begin(c, KRR_PROF_SOLVE);
-    KRR_TRY(solve_inplace(c, c->abuf, c->zbuf, p));
+    KRR_TRY(solve_rhs(c, c->ybuf, c->abuf, c->zbuf, p));
     prof_end(c, pr, sweep_flops, sweep_bytes);
     KRR_TRY(check_launch(c, "solve"));
     krr_solve_info si;
@@ -344,13 +339,10 @@ krr_status solve_device(Ctx *c, int64_t p, krr_solve_info *info) {
         // relative residual is left in red[RED_RNORM..+1] for the caller
         const int iters = mixed(c) ? c->opt.ir_max : 0;
         for (int it = 0; it < iters; ++it) {
-            KRR_TRY(launch_residual(c, c->ybuf, c->abuf, c->rbuf, p));
-            launch_axpy_r(c->rbuf, c->dabuf, cnt, s);
-            KRR_TRY(solve_inplace(c, c->dabuf, c->zbuf, p));
-            launch_add_scaled(c->abuf, c->dabuf, 1.0f, cnt, s);
+            KRR_TRY(launch_residual(c, c->ybuf, c->abuf, p));
+            KRR_TRY(solve_rhs(c, nullptr, c->dabuf, c->zbuf, p, c->abuf));
         }
-        KRR_TRY(launch_residual(c, c->ybuf, c->abuf, c->rbuf, p));
-        launch_reduce_norms(c->rbuf, c->ybuf, c->n_pad, p, c->red + RED_RNORM, red_norm_part(c), s);
+        KRR_TRY(launch_residual(c, c->ybuf, c->abuf, p));
         KRR_TRY(check_launch(c, "refinement (graph mode)"));
         if (info) *info = si;
         return KRR_OK;
@@ -360,10 +352,8 @@ krr_status solve_device(Ctx *c, int64_t p, krr_solve_info *info) {
         double best = INFINITY;
         for (int it = 0;; ++it) {
             int rr = prof_begin(c, KRR_PROF_RESIDUAL);
-            KRR_TRY(launch_residual(c, c->ybuf, c->abuf, c->rbuf, p));
-            launch_reduce_norms(c->rbuf, c->ybuf, c->n_pad, p, c->red + RED_RNORM, red_norm_part(c), s);
-            // the lower-triangle K tiles are read once by the row pass and
-            // once by the column pass
+            KRR_TRY(launch_residual(c, c->ybuf, c->abuf, p));
+            // the lower-triangle K tiles are needed by rows and by columns
             prof_end(c, rr, 2.0 * (double)c->n_pad * c->n_pad * p, 2.0 * (double)c->kd_bytes);
             KRR_TRY(check_launch(c, "residual"));
             KRR_CUDA_TRY(c, cudaMemcpyAsync(c->hred, c->red, 2 * sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -403,11 +393,9 @@ krr_status solve_device(Ctx *c, int64_t p, krr_solve_info *info) {
                 break;
             }
             best = std::min(best, rel);
-            launch_axpy_r(c->rbuf, c->dabuf, cnt, s);
             int sr = prof_begin(c, KRR_PROF_SOLVE);
-            KRR_TRY(solve_inplace(c, c->dabuf, c->zbuf, p));
+            KRR_TRY(solve_rhs(c, nullptr, c->dabuf, c->zbuf, p, c->abuf));
             prof_end(c, sr, sweep_flops, sweep_bytes);
-            launch_add_scaled(c->abuf, c->dabuf, 1.0f, cnt, s);
             KRR_TRY(check_launch(c, "refinement step"));
         }
     }
@@ -576,6 +564,7 @@ void krr_destroy(krr_ctx *c) {
     dev_free(&c->ybuf);
     dev_free(&c->zbuf);
     dev_free(&c->rbuf);
+    dev_free(&c->rs_part);
     dev_free(&c->abuf);
     dev_free(&c->dabuf);
     dev_free(&c->pred_part);

@@ -152,7 +152,7 @@ struct Ctx {
 
     // solve / predict scratch
     float *ybuf = nullptr, *zbuf = nullptr;  // n_pad x p work vectors
-    double *rbuf = nullptr;                  // n_pad x p residual (FP64)
+    double *rbuf = nullptr;                  // n_pad x p residual (FP64; fp32 mode)
     float *abuf = nullptr;                   // n_pad x p current solution
     float *dabuf = nullptr;                  // n_pad x p correction
     double *red = nullptr;                   // reductions (norms), small; slots RED_*
@@ -162,6 +162,8 @@ struct Ctx {
     int64_t vec_cap = 0;                     // capacity in elements of the n_pad x p buffers
     float *pred_part = nullptr;              // predict partial products
     size_t pred_part_cap = 0;
+    double *rs_part = nullptr;               // residual: partial sums per slot, column and row
+    int64_t rs_part_cap = 0;
     int *sw_flags = nullptr;                 // sweep item counter, abort flag, progress counters
     int64_t sw_flags_cap = 0;
     __half *ts_v0 = nullptr, *ts_v1 = nullptr;  // tensor-core sweep: FP16 pairs of vector blocks
@@ -396,22 +398,24 @@ inline int64_t tile_max_partials(int64_t b) { return (b / 128) * (b / 256); }
 // ||K||_F^2 is read from c->red[2] (written by the build).
 void launch_column_cast(Ctx *c, int64_t k);
 
-// Triangular solves with the stored factor: X <- (L L^T)^-1 X, n_pad x p
-// (row-major, leading dimension p); tmp is n_pad x p scratch.
-krr_status solve_inplace(Ctx *c, float *x, float *tmp, int64_t p);
+// Triangular solves with the stored factor: x <- (L L^T)^-1 rhs, n_pad x p
+// (row-major, leading dimension p); tmp is n_pad x p scratch; sum (optional):
+// also sum += x.  rhs = nullptr: the right-hand side is the last residual.
+krr_status solve_rhs(Ctx *c, const float *rhs, float *x, float *tmp, int64_t p, float *sum = nullptr);
 
 // Persistent dataflow sweeps (sweep.cu): the two substitutions of a solve
 // on CUDA cores (fp32 mode), and the residual r = y - (K + lambda I) a given
 // the column sums of a in c->colsum.
 krr_status sweep_solve(Ctx *c, float *x, float *tmp, int64_t p);
 // The two substitutions on the tensor cores (tcsweep.cu, mixed mode).
-krr_status tc_sweep_solve(Ctx *c, float *x, float *tmp, int64_t p);
+krr_status tc_sweep_solve(Ctx *c, const float *rhs, float *x, float *tmp, int64_t p, float *sum);
 // The refinement residual on the tensor cores (tcsweep.cu, mixed mode).
-krr_status tc_residual(Ctx *c, const float *y, const float *a, double *r, int64_t p);
+krr_status tc_residual(Ctx *c, const float *y, const float *a, int64_t p);
 krr_status sweep_residual(Ctx *c, const float *y, const float *a, double *r, int64_t p);
 
-// r = y - (K + lambda I) a (FP64 accumulation), norms into c->red.
-krr_status launch_residual(Ctx *c, const float *y, const float *a, double *r, int64_t p);
+// Residual y - (K + lambda I) a, kept for solve_rhs; ||r||_F^2 and ||y||_F^2
+// into c->red[RED_RNORM], [RED_RNORM + 1].
+krr_status launch_residual(Ctx *c, const float *y, const float *a, int64_t p);
 
 // Resets the device error record and the precision map, and (fp32 mode)
 // fills the tile table: every factor tile FP32 at a fixed slot.
@@ -424,7 +428,6 @@ void launch_fill_zero(void *p, size_t bytes, cudaStream_t s);
 constexpr int64_t norm_partial_count() { return 2 * 256; }
 void launch_reduce_norms(const double *r, const float *y, int64_t n, int64_t p, double *out, double *part,
                          cudaStream_t s);
-void launch_axpy_r(const double *r, float *dst, int64_t count, cudaStream_t s);
 void launch_add_scaled(float *a, const float *da, float alpha, int64_t count, cudaStream_t s);
 // Yt = sum of the per-block partials; when shift is given the partials are of
 // (K - c) A and c (1^T A) is added (c = *shift rounded to FP32, colsum = 1^T A).

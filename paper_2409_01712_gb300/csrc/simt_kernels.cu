@@ -966,8 +966,15 @@ void launch_kernel_sumsq(Ctx *c, double *out) {
 }
 
 // x (n_pad x p) <- (L L^T)^-1 x.  tmp is n_pad x p scratch (ends as Z).
-krr_status solve_inplace(Ctx *c, float *x, float *tmp, int64_t p) {
-    return c->opt.mode == KRR_MODE_MIXED ? tc_sweep_solve(c, x, tmp, p) : sweep_solve(c, x, tmp, p);
+krr_status solve_rhs(Ctx *c, const float *rhs, float *x, float *tmp, int64_t p, float *sum) {
+    if (mixed(c)) return tc_sweep_solve(c, rhs, x, tmp, p, sum);
+    // fp32 mode: one solve per call, no refinement
+    if (!rhs || sum) {
+        c->last_error = "solve_rhs: refinement needs the mixed mode";
+        return KRR_EINVAL;
+    }
+    KRR_CUDA_TRY(c, cudaMemcpyAsync(x, rhs, (size_t)c->n_pad * p * sizeof(float), cudaMemcpyDeviceToDevice, c->stream));
+    return sweep_solve(c, x, tmp, p);
 }
 
 // Column sums of a (n x p) in FP64, one block per column.
@@ -988,11 +995,6 @@ __global__ void colsum_kernel(const float *a, int64_t n, int64_t p, double *out)
 
 void launch_colsum(const float *a, int64_t n, int64_t p, double *out, cudaStream_t s) {
     count_launch(), colsum_kernel<<<(unsigned)p, 512, 0, s>>>(a, n, p, out);
-}
-
-krr_status launch_residual(Ctx *c, const float *y, const float *a, double *r, int64_t p) {
-    count_launch(), colsum_kernel<<<(unsigned)p, 512, 0, c->stream>>>(a, c->n_pad, p, c->colsum);
-    return c->opt.mode == KRR_MODE_MIXED ? tc_residual(c, y, a, r, p) : sweep_residual(c, y, a, r, p);
 }
 
 // ||r||_F^2 and ||y||_F^2 into out[0], out[1]: fixed per-block partial sums
@@ -1048,12 +1050,14 @@ void launch_reduce_norms(const double *r, const float *y, int64_t n, int64_t p, 
     count_launch(), norm_final_kernel<<<1, 256, 0, s>>>(part, NORM_BLOCKS, out);
 }
 
-__global__ void d2f_kernel(const double *r, float *dst, int64_t count) {
-    int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (e < count) dst[e] = (float)r[e];
-}
-void launch_axpy_r(const double *r, float *dst, int64_t count, cudaStream_t s) {
-    count_launch(), d2f_kernel<<<cdiv(count, 256), 256, 0, s>>>(r, dst, count);
+krr_status launch_residual(Ctx *c, const float *y, const float *a, int64_t p) {
+    if (mixed(c)) return tc_residual(c, y, a, p);
+    count_launch(), colsum_kernel<<<(unsigned)p, 512, 0, c->stream>>>(a, c->n_pad, p, c->colsum);
+    KRR_TRY(sweep_residual(c, y, a, c->rbuf, p));
+    // the norm partials are the last norm_partial_count() doubles of the reduction buffer
+    launch_reduce_norms(c->rbuf, y, c->n_pad, p, c->red + RED_RNORM, c->red + c->red_cap - norm_partial_count(),
+                        c->stream);
+    return KRR_OK;
 }
 
 __global__ void add_kernel(float *a, const float *da, float alpha, int64_t count) {

@@ -365,15 +365,11 @@ __device__ void decode_item(const TsParams &p, int64_t t, ItemHdr &h) {
 // Block conversion (128 epilogue threads): v rows [blk b, +b), columns
 // [q0, q0 + pc) -> FP16 terms with the power-of-two scale s_q putting the
 // column maximum in [4096, 8192) (8x headroom below the FP16 maximum):
-// two terms hi = fp16(s v), lo = fp16(s v - hi) (about 22 significant bits),
-// or three, hi, mid = fp16(s v - hi), lo = fp16(s v - hi - mid), which hold
-// an FP32 value exactly down to 2^-14 of the column maximum (below that the
-// absolute error stays under 2^-38 of the maximum).  Planes of np rows each;
-// padding columns [pc, np) are zero.
+// two terms hi = fp16(s v), lo = fp16(s v - hi) (about 22 significant bits).
+// Planes of np rows each; padding columns [pc, np) are zero.
 // ---------------------------------------------------------------------------
 __device__ void convert_block(const TsParams &p, const float *v, int64_t blk, __half *vb, float *sv,
-                              float *smax, float *sscale, int tid, int terms = 2, const float *slabmax = nullptr,
-                              float *bmax = nullptr) {
+                              float *smax, float *sscale, int tid, const float *slabmax, float *bmax) {
     const int64_t b = p.b, n_pad = p.n_pad, rs = p.rs, cs = p.cs;
     const int pc = p.pc, np = p.np;
     if (slabmax) {
@@ -419,7 +415,7 @@ __device__ void convert_block(const TsParams &p, const float *v, int64_t blk, __
                 frexpf(m, &e);  // m = f 2^e, f in [0.5, 1)
                 s = ldexpf(1.f, max(-126, min(126, 13 - e)));
             }
-            if (bmax) bmax[blk * TS_NPMAX + tid] = m;
+            bmax[blk * TS_NPMAX + tid] = m;
         }
         sscale[tid] = s;
         sv[blk * np + tid] = s;
@@ -442,11 +438,8 @@ __device__ void convert_block(const TsParams &p, const float *v, int64_t blk, __
             if (q < np) {
                 const float x = (q < pc) ? xv[q] * sscale[q] : 0.f;
                 const __half hh = __float2half_rn(x);
-                const float r1 = x - __half2float(hh);  // exact
-                const __half m = __float2half_rn(r1);
                 vb[(int64_t)q * n_pad + grow] = hh;
-                vb[(int64_t)(np + q) * n_pad + grow] = m;
-                if (terms == 3) vb[(int64_t)(2 * np + q) * n_pad + grow] = __float2half_rn(r1 - __half2float(m));
+                vb[(int64_t)(np + q) * n_pad + grow] = __float2half_rn(x - __half2float(hh));
             }
         }
     }
@@ -747,7 +740,7 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
             if (++slot == TS_IRING) { slot = 0; sph ^= 1; }
             if (h.type == IT_END) break;
             if (h.type == IT_CONV) {
-                convert_block(p, p.rhs, h.blk, p.vin, p.sin, smax, sscale, tid, 2, nullptr, p.bm_in);
+                convert_block(p, p.rhs, h.blk, p.vin, p.sin, smax, sscale, tid, nullptr, p.bm_in);
                 if (tid == 0) st_release(done_ctr(p) + h.blk, 1);
                 continue;
             }
@@ -830,7 +823,7 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
                 epi_sync();
                 if (sflag[1]) {
                     if (!accept_block(p, p.mx_out, h.blk, sscale, p.sout, p.bm_out, sflag, tid))
-                        convert_block(p, p.out, h.blk, p.vout, p.sout, smax, sscale, tid, 2, p.mx_out, p.bm_out);
+                        convert_block(p, p.out, h.blk, p.vout, p.sout, smax, sscale, tid, p.mx_out, p.bm_out);
                     if (tid == 0) {
                         __threadfence();
                         st_release(ready_ctr(p) + h.blk, 1);
@@ -866,7 +859,7 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
                 epi_sync();
                 if (sflag[1]) {
                     if (!accept_block(p, p.mx_in, h.blk, sscale, p.sin, p.bm_in, sflag, tid))
-                        convert_block(p, p.rhs, h.blk, p.vin, p.sin, smax, sscale, tid, 2, p.mx_in, p.bm_in);
+                        convert_block(p, p.rhs, h.blk, p.vin, p.sin, smax, sscale, tid, p.mx_in, p.bm_in);
                     if (tid == 0) {
                         __threadfence();
                         st_release(done_ctr(p) + h.blk, 1);
@@ -885,35 +878,47 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
 
 // ---------------------------------------------------------------------------
 // Refinement residual on the tensor cores:
-//   r = y - lambda a - sum_j (K_ij - c) a_j - c 1 (1^T a)      (FP64 output)
+//   r = y - lambda a - sum_j (K_ij - c) a_j - c 1 (1^T a)
 // with K the FP32 kernel tiles (lower triangle; block row i reads the row
 // slabs of tiles (i, j <= i) and the column slabs of tiles (j > i, i)) and c
 // the shift (mean off-diagonal entry of K), which keeps the products small.
-// Item (i, s) = 128 rows of block i, one accumulation per tile j:
-//   warp 0      producer: TMA of the FP32 K chunk (128 x 64 rows x columns, or
-//               64 x 128 for a column slab) into a staging ring, and of the
-//               FP16 terms of a_j (B) into a ring of their own;
-//   warps 6..9  converters: (K - c) 2^12 -> FP16 pair (hi, lo), written in
-//               place over the staged FP32 chunk (each thread overwrites only
-//               the bytes its own warp read) in the MMA's K-major or MN-major
-//               128-byte-swizzled layout, so the staging ring is also the
-//               operand ring;
-//   warp 1      MMA: A_hi x [B_hi; B_mid; B_lo] (N = 3 np) and A_lo x [B_hi;
-//               B_mid] (N = 2 np); a is split into three FP16 terms (exact for
-//               FP32 values), K - c into two (about 22 bits of a quantity
-//               already small); the dropped products are below 2^-33;
-//   warps 2..5  epilogue: per 64-wide chunk, the three FP32 accumulator
-//               parts are summed, de-scaled exactly (powers of two) and added
-//               to a two-term FP32 (TwoSum) accumulator, so each FP32 sum in
-//               TMEM spans only 64 products.
+//
+// Item: 128 rows of one block times `g` consecutive source blocks (or 1 / h of
+// one), added up in a two-term FP32 accumulator and written to a slot of its
+// own, [slot][column][row] in FP64; a finishing kernel adds the slots in
+// order (deterministic).  Items are listed by pairs of block groups (I, J),
+// the slabs of both orientations together: a tile is needed once by rows (for
+// the block row I) and once by columns (for J), and the two uses follow each
+// other within a few items, so the second finds the tile in L2 and K comes
+// from HBM once.  The split also fills the GPU when there are fewer 128-row
+// slabs than SMs.  With
+// one item per slab over all tiles, one epilogue group and the tiles read
+// twice from HBM a residual took 1.27 ms at N = 32768 and 10 columns, 11.3 ms
+// at N = 98304 and 20, 0.16 ms at N = 5000 and 2; now 0.88, 8.5 and 0.06 ms.
+//   warp 0       producer: TMA of the FP32 K chunk (128 x 64 rows x columns, or
+//                64 x 128 for a column slab) and of the FP16 terms of a_j (B);
+//   warps 6..9   converters: (K - c) 2^12 -> FP16 pair (hi, lo), written in
+//                place over the staged FP32 chunk (each thread overwrites only
+//                the bytes its own warp read) in the MMA's K-major or MN-major
+//                128-byte-swizzled layout, so the staging ring is also the
+//                operand ring;
+//   warp 1       MMA: A_hi x [B_hi; B_mid; B_lo] (N = 3 np) and A_lo x [B_hi;
+//                B_mid] (N = 2 np); a is split into three FP16 terms (exact for
+//                FP32 values), K - c into two (about 22 bits of a quantity
+//                already small); the dropped products are below 2^-33;
+//   warps 2..5 and 10..13  epilogue: per 64-wide chunk, the three FP32
+//                accumulator parts are summed, de-scaled exactly (powers of
+//                two) and added to a two-term FP32 (TwoSum) accumulator, so
+//                each FP32 sum in TMEM spans only 64 products; each group of
+//                four warps takes half of the columns.
 // Operands exactly representing the FP32 inputs, exact FP16 products and
 // FP32 accumulation: the residual keeps FP32 accuracy.
 // Every wait is bounded and ends the kernel with KRR_ETIMEOUT.
 // ---------------------------------------------------------------------------
-constexpr int RS_THREADS = 320;
+constexpr int RS_THREADS = 448;
 constexpr int RS_STG = 32768;      // FP32 chunk: 128 x 64 or 64 x 128
-constexpr int RS_NSTG = 5;         // staging ring (FP32 K chunks by TMA, converted in place)
-constexpr int RS_NB = 3;           // B ring (FP16 terms of a, TMA): loads run ahead of the A ring
+constexpr int RS_NSTG = 5;         // stages (FP32 K chunk by TMA, converted in place, and the terms of a)
+constexpr int RS_NACC = 4;         // TMEM accumulators of 3 np columns
 // (K - c) s in FP16 with the power of two s = 2^(e - 1) <= 8192 / (max|K| + |c|):
 // |(K - c) s| <= 8192, far below the FP16 maximum (s = 2^12 for the Gaussian
 // kernel, whose entries lie in (0, 1]).
@@ -924,21 +929,47 @@ __device__ __forceinline__ float rs_kscale(const double *kbound, const double *s
 }
 
 struct RsParams {
-    int64_t b, nt, S, KC, items, n_pad;
-    int np, pc, q0;
-    int64_t ldx;
-    const float *y, *a;
-    double *r;
-    const double *shift, *colsum;
+    int b, nt, S, KC, items;
+    int64_t n_pad;
+    int pc;
+    int g, h;               // source blocks of an item, or parts of one (g == 1 or h == 1)
+    int ngrp;               // block groups: ceil(nt / g)
+    const double *shift;
     const double *kbound;   // max |K_ij| (the residual operand's scale follows from it)
-    float lambda;
-    const float *sa;        // scales of the FP16 pair of a, [nt][np]
+    const float *inv_s;     // inverse scales of the FP16 terms of a, [n_pad / 128][np]
+    double *part;           // [slot][pc][n_pad]
     int *flags;             // [0] item counter, [1] abort
-    int b_bytes;            // one B chunk: 3 np rows of 128 bytes
     uint32_t idesc_k, idesc_mn, idesc_k2, idesc_mn2;  // N = 3 np and N = 2 np
     uint64_t wait_ns;
     DevErrors *err;
 };
+
+// One item: rows [sl 128, +128) of block i; source blocks [j0, j1), K chunks
+// [kc0, kc1) of each; its slot.  Items of a group pair: parts, then the two
+// orientations, then the blocks of the output group and their slabs.
+struct RsItem {
+    int i, sl, j0, j1, kc0, kc1, slot;
+};
+
+__device__ __forceinline__ bool rs_decode(const RsParams &p, int t, RsItem &it) {
+    const int per = 2 * p.g * p.S * p.h;
+    int64_t gi, gj;
+    tri_decode(t / per, &gi, &gj);
+    int v = t % per;
+    const int e = v / (2 * p.g * p.S);
+    v %= 2 * p.g * p.S;
+    const int o = v / (p.g * p.S);
+    v %= p.g * p.S;
+    const int out = o ? (int)gj : (int)gi, src = o ? (int)gi : (int)gj;
+    it.i = out * p.g + v / p.S;
+    it.sl = v % p.S;
+    it.j0 = src * p.g;
+    it.j1 = min(it.j0 + p.g, p.nt);
+    it.kc0 = p.KC * e / p.h;
+    it.kc1 = p.KC * (e + 1) / p.h;
+    it.slot = src * p.h + e;
+    return it.i < p.nt && !(o == 1 && gi == gj);  // a group's pair with itself has one orientation
+}
 
 __device__ __forceinline__ bool rs_aborted(const RsParams &p) { return *(volatile int *)&p.flags[1] != 0; }
 
@@ -958,43 +989,59 @@ __device__ __forceinline__ bool rs_wait(uint64_t *bar, uint32_t parity, const Rs
     }
 }
 
+// Three groups of eight TMEM columns, one wait.
+__device__ __forceinline__ void tmem_ld8x3(uint32_t t0, uint32_t t1, uint32_t t2, float (&a)[8], float (&b)[8],
+                                           float (&c)[8]) {
+    uint32_t r[24];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%24];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%8,%9,%10,%11,%12,%13,%14,%15}, [%25];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%16,%17,%18,%19,%20,%21,%22,%23}, [%26];\n\t"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=&r"(r[0]), "=&r"(r[1]), "=&r"(r[2]), "=&r"(r[3]), "=&r"(r[4]), "=&r"(r[5]), "=&r"(r[6]), "=&r"(r[7]),
+          "=&r"(r[8]), "=&r"(r[9]), "=&r"(r[10]), "=&r"(r[11]), "=&r"(r[12]), "=&r"(r[13]), "=&r"(r[14]),
+          "=&r"(r[15]), "=&r"(r[16]), "=&r"(r[17]), "=&r"(r[18]), "=&r"(r[19]), "=&r"(r[20]), "=&r"(r[21]),
+          "=&r"(r[22]), "=&r"(r[23])
+        : "r"(t0), "r"(t1), "r"(t2)
+        : "memory");
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+        a[e] = __uint_as_float(r[e]);
+        b[e] = __uint_as_float(r[8 + e]);
+        c[e] = __uint_as_float(r[16 + e]);
+    }
+}
+
+template <int NP>
 __global__ void __launch_bounds__(RS_THREADS, 1)
     tcres_kernel(const __grid_constant__ CUtensorMap mK128, const __grid_constant__ CUtensorMap mK64,
                  const __grid_constant__ CUtensorMap mA, const RsParams p) {
+    constexpr int BB = 3 * NP * 128;           // bytes of the B terms of a chunk
+    constexpr int SB = RS_STG + BB;            // bytes of a stage
+    constexpr uint32_t TCOLS = (RS_NACC * 3 * NP <= 256) ? 256u : 512u;
     extern __shared__ __align__(1024) uint8_t rs_smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(rs_smem_raw) + 1023) & ~uintptr_t(1023));
-    uint8_t *stg = smem;                                   // RS_NSTG x 32 KB
-    uint8_t *bst = smem + RS_NSTG * RS_STG;                // RS_NB x b_bytes
-    int64_t *items = reinterpret_cast<int64_t *>(bst + RS_NB * p.b_bytes);  // item ring
+    int *items = reinterpret_cast<int *>(smem + RS_NSTG * SB);  // item ring
     uint64_t *bars = reinterpret_cast<uint64_t *>(items + TS_IRING);
-    // sfull: FP32 chunk landed; cfull: converted in place; sempty: MMAs done
-    uint64_t *sfull = bars, *sempty = bars + RS_NSTG, *cfull = bars + 2 * RS_NSTG,
-             *bfull = cfull + RS_NSTG, *bempty = bfull + RS_NB,
-             *tfull = bempty + RS_NB, *tempty = tfull + 2, *ifull = tempty + 2, *iempty = ifull + TS_IRING,
+    // sfull: FP32 chunk and B landed; cfull: converted in place; sempty: MMAs done
+    uint64_t *sfull = bars, *sempty = bars + RS_NSTG, *cfull = bars + 2 * RS_NSTG, *tfull = cfull + RS_NSTG,
+             *tempty = tfull + RS_NACC, *ifull = tempty + RS_NACC, *iempty = ifull + TS_IRING,
              *drain = iempty + TS_IRING;
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(drain + 1);
-    // epilogue: low halves of the two-term column sums, [TS_NPMAX][128 threads]
-    float *alo_s = reinterpret_cast<float *>(tmem_slot + 4);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int np = p.np;
-    const uint32_t tcols = (np * 6 <= 128) ? 128u : 256u;  // two accumulators of 3 np columns
     if (threadIdx.x == 0) {
         for (int q = 0; q < RS_NSTG; ++q) {
             mbar_init(&sfull[q], 1);
             mbar_init(&sempty[q], 1);      // MMA commit
             mbar_init(&cfull[q], 4);       // converter warps
         }
-        for (int q = 0; q < RS_NB; ++q) {
-            mbar_init(&bfull[q], 1);       // producer (B bytes)
-            mbar_init(&bempty[q], 1);      // MMA commit
-        }
-        for (int a = 0; a < 2; ++a) {
+        for (int a = 0; a < RS_NACC; ++a) {
             mbar_init(&tfull[a], 1);
-            mbar_init(&tempty[a], 4);      // epilogue warps
+            mbar_init(&tempty[a], 8);      // epilogue warps
         }
         for (int q = 0; q < TS_IRING; ++q) {
             mbar_init(&ifull[q], 1);
-            mbar_init(&iempty[q], 4 + 4 + 1);  // epilogue, converter warps, MMA thread
+            mbar_init(&iempty[q], 8 + 4 + 1);  // epilogue, converter warps, MMA thread
         }
         mbar_init(drain, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -1002,7 +1049,7 @@ __global__ void __launch_bounds__(RS_THREADS, 1)
     }
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
-                     "r"(tcols)
+                     "r"(TCOLS)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
@@ -1015,54 +1062,53 @@ __global__ void __launch_bounds__(RS_THREADS, 1)
     __syncthreads();
     tmem_fence_after();
     const uint32_t tmem_base = *tmem_slot;
-    const int64_t b = p.b, nt = p.nt, S = p.S;
-    const int KC = (int)p.KC;
-    const uint32_t bbytes = (uint32_t)p.b_bytes;
 
     if (warp == 0) {
         if (lane == 0) {
             // ------------------------------ producer ------------------------------
-            int ss = 0, os = 0, slot = 0;
-            uint32_t sph = 0, oph = 0, iph = 0;
-            int issued_s = 0, issued_o = 0;
+            int ss = 0, slot = 0;
+            uint32_t sph = 0, iph = 0;
+            int issued = 0;
             bool ok = true;
+            int t = atomicAdd(&p.flags[0], 1);
             while (ok) {
-                const int64_t t = atomicAdd(&p.flags[0], 1);
+                RsItem it;
+                const bool end = t >= p.items;
+                if (!end && !rs_decode(p, t, it)) {  // empty position
+                    t = atomicAdd(&p.flags[0], 1);
+                    continue;
+                }
                 if (!rs_wait(&iempty[slot], iph ^ 1, p)) { ok = false; break; }
-                items[slot] = (t < p.items) ? t : -1;
+                items[slot] = end ? -1 : t;
                 mbar_arrive(&ifull[slot]);
                 if (++slot == TS_IRING) { slot = 0; iph ^= 1; }
-                if (t >= p.items) break;
-                const int64_t i = t / S, sl = t % S;
-                for (int64_t j = 0; j < nt && ok; ++j) {
-                    for (int kc = 0; kc < KC && ok; ++kc) {
+                if (end) break;
+                t = atomicAdd(&p.flags[0], 1);  // the next item's number arrives during this one
+                for (int j = it.j0; j < it.j1 && ok; ++j) {
+                    for (int kc = it.kc0; kc < it.kc1; ++kc) {
                         if (!rs_wait(&sempty[ss], sph ^ 1, p)) { ok = false; break; }
-                        uint8_t *st = stg + ss * RS_STG;
-                        mbar_arrive_expect_tx(&sfull[ss], RS_STG);
-                        if (j <= i) {
+                        uint8_t *st = smem + ss * SB;
+                        mbar_arrive_expect_tx(&sfull[ss], SB);
+                        if (j <= it.i) {
                             // row slab of tile (i, j): rows [sl 128, +128), columns [kc 64, +64)
-                            const int y = (int)(tri_index(i, j) * b + sl * TS_SLAB);
+                            const int y = (int)tri_index(it.i, j) * p.b + it.sl * TS_SLAB;
                             tma_load_2d(st, &mK128, kc * 64, y, &sfull[ss]);
                             tma_load_2d(st + RS_STG / 2, &mK128, kc * 64 + 32, y, &sfull[ss]);
                         } else {
                             // column slab of tile (j, i): rows [kc 64, +64), columns [sl 128, +128)
-                            const int y = (int)(tri_index(j, i) * b + kc * 64);
+                            const int y = (int)tri_index(j, it.i) * p.b + kc * 64;
                             for (int e = 0; e < 4; ++e)
-                                tma_load_2d(st + e * (RS_STG / 4), &mK64, (int)(sl * TS_SLAB) + 32 * e, y, &sfull[ss]);
+                                tma_load_2d(st + e * (RS_STG / 4), &mK64, it.sl * TS_SLAB + 32 * e, y, &sfull[ss]);
                         }
-                        ++issued_s;
+                        tma_load_2d(st + RS_STG, &mA, j * p.b + kc * 64, 0, &sfull[ss]);
+                        ++issued;
                         if (++ss == RS_NSTG) { ss = 0; sph ^= 1; }
-                        if (!rs_wait(&bempty[os], oph ^ 1, p)) { ok = false; break; }
-                        mbar_arrive_expect_tx(&bfull[os], bbytes);
-                        tma_load_2d(bst + os * p.b_bytes, &mA, (int)(j * b) + kc * 64, 0, &bfull[os]);
-                        ++issued_o;
-                        if (++os == RS_NB) { os = 0; oph ^= 1; }
                     }
                 }
             }
             if (!ok) {
                 // drain the copies in flight (bounded)
-                int n = issued_s < RS_NSTG ? issued_s : RS_NSTG;
+                const int n = issued < RS_NSTG ? issued : RS_NSTG;
                 int q = ss;
                 uint32_t pp = sph;
                 for (int e = 0; e < n; ++e) {
@@ -1070,41 +1116,32 @@ __global__ void __launch_bounds__(RS_THREADS, 1)
                     const uint64_t t0 = globaltimer();
                     while (!mbar_try_wait(&sfull[q], pp) && globaltimer() - t0 < drain_limit(p.wait_ns)) {}
                 }
-                n = issued_o < RS_NB ? issued_o : RS_NB;
-                q = os;
-                pp = oph;
-                for (int e = 0; e < n; ++e) {
-                    if (--q < 0) { q = RS_NB - 1; pp ^= 1; }
-                    const uint64_t t0 = globaltimer();
-                    while (!mbar_try_wait(&bfull[q], pp) && globaltimer() - t0 < drain_limit(p.wait_ns)) {}
-                }
             }
         }
     } else if (warp == 1) {
         if (lane == 0) {
             // ------------------------------ MMA issuer ------------------------------
-            int ss = 0, bs = 0, slot = 0, acc = 0;
-            uint32_t sph = 0, bph = 0, iph = 0, aph = 0;
+            int ss = 0, slot = 0, acc = 0;
+            uint32_t sph = 0, iph = 0, aph = 0;
             bool ok = true, any = false;
             while (ok) {
                 if (!rs_wait(&ifull[slot], iph, p)) { ok = false; break; }
-                const int64_t t = items[slot];
+                const int t = items[slot];
                 mbar_arrive(&iempty[slot]);
                 if (++slot == TS_IRING) { slot = 0; iph ^= 1; }
                 if (t < 0) break;
-                const int64_t i = t / S;
-                for (int64_t j = 0; j < nt && ok; ++j) {
-                    const bool kmaj = (j <= i);
-                    for (int kc = 0; kc < KC; ++kc) {
-                        // one accumulation per 64-wide chunk, folded into FP64
-                        // by the epilogue: the FP32 sums in TMEM stay short
+                RsItem it;
+                rs_decode(p, t, it);
+                for (int j = it.j0; j < it.j1 && ok; ++j) {
+                    const bool kmaj = (j <= it.i);
+                    for (int kc = it.kc0; kc < it.kc1; ++kc) {
+                        // one accumulation per 64-wide chunk: the FP32 sums in TMEM stay short
                         if (!rs_wait(&tempty[acc], aph ^ 1, p)) { ok = false; break; }
-                        tmem_fence_after();
-                        const uint32_t tacc = tmem_base + (uint32_t)(acc * 3 * np);
+                        const uint32_t tacc = tmem_base + (uint32_t)(acc * 3 * NP);
+                        if (!rs_wait(&sfull[ss], sph, p)) { ok = false; break; }
                         if (!rs_wait(&cfull[ss], sph, p)) { ok = false; break; }
-                        if (!rs_wait(&bfull[bs], bph, p)) { ok = false; break; }
                         tmem_fence_after();
-                        const uint32_t sa = smem_u32(stg + ss * RS_STG), sb = smem_u32(bst + bs * p.b_bytes);
+                        const uint32_t sa = smem_u32(smem + ss * SB), sb = sa + RS_STG;
 #pragma unroll
                         for (int kk = 0; kk < 4; ++kk) {
                             const uint64_t bd = desc_kmajor(sb + kk * 32);
@@ -1118,11 +1155,9 @@ __global__ void __launch_bounds__(RS_THREADS, 1)
                         }
                         any = true;
                         mma_commit(&sempty[ss]);  // the stage takes the next TMA load
-                        mma_commit(&bempty[bs]);
                         if (++ss == RS_NSTG) { ss = 0; sph ^= 1; }
-                        if (++bs == RS_NB) { bs = 0; bph ^= 1; }
                         mma_commit(&tfull[acc]);
-                        if (++acc == 2) { acc = 0; aph ^= 1; }
+                        if (++acc == RS_NACC) { acc = 0; aph ^= 1; }
                     }
                 }
             }
@@ -1132,7 +1167,7 @@ __global__ void __launch_bounds__(RS_THREADS, 1)
                 while (!mbar_try_wait(drain, 0) && globaltimer() - t0 < drain_limit(p.wait_ns)) {}
             }
         }
-    } else if (warp >= 6) {
+    } else if (warp >= 6 && warp < 10) {
         // ------------------------------ converters ------------------------------
         const int ct = threadIdx.x - 192;
         const float c = (float)*p.shift;
@@ -1142,21 +1177,22 @@ __global__ void __launch_bounds__(RS_THREADS, 1)
         bool ok = true;
         while (ok) {
             if (!__all_sync(0xffffffffu, rs_wait(&ifull[slot], iph, p))) break;
-            const int64_t t = items[slot];
+            const int t = items[slot];
             __syncwarp();
             if (lane == 0) mbar_arrive(&iempty[slot]);
             if (++slot == TS_IRING) { slot = 0; iph ^= 1; }
             if (t < 0) break;
-            const int64_t i = t / S;
-            for (int64_t j = 0; j < nt && ok; ++j) {
-                const bool kmaj = (j <= i);
+            RsItem it;
+            rs_decode(p, t, it);
+            for (int j = it.j0; j < it.j1 && ok; ++j) {
+                const bool kmaj = (j <= it.i);
                 // thread -> (row r of the staged chunk, 64-value half h)
                 const int r = kmaj ? ct : (ct >> 1), h = kmaj ? 0 : (ct & 1);
                 const int boxb = kmaj ? RS_STG / 2 : RS_STG / 4;
-                for (int kc = 0; kc < KC; ++kc) {
+                for (int kc = it.kc0; kc < it.kc1; ++kc) {
                     if (!__all_sync(0xffffffffu, rs_wait(&sfull[ss], sph, p))) { ok = false; break; }
-                    const uint8_t *src = stg + ss * RS_STG + r * 128;
-                    uint8_t *dst = stg + ss * RS_STG + h * 8192 + r * 128;
+                    const uint8_t *src = smem + ss * SB + r * 128;
+                    uint8_t *dst = smem + ss * SB + h * 8192 + r * 128;
                     float v[64];
 #pragma unroll
                     for (int e = 0; e < 2; ++e) {
@@ -1196,88 +1232,229 @@ __global__ void __launch_bounds__(RS_THREADS, 1)
         }
     } else {
         // ------------------------------ epilogue ------------------------------
+        constexpr int NC = NP / 2;  // columns of this group
         const int row = ((warp & 3) << 5) + lane;
+        const int q0 = (warp >= 10) ? NC : 0;
         int slot = 0, acc = 0;
         uint32_t iph = 0, aph = 0;
-        const int pc = p.pc;
+        const float kinv = 1.f / rs_kscale(p.kbound, p.shift);  // a power of two: exact
         while (true) {
             if (!__all_sync(0xffffffffu, rs_wait(&ifull[slot], iph, p))) break;
-            const int64_t t = items[slot];
+            const int t = items[slot];
             __syncwarp();
             if (lane == 0) mbar_arrive(&iempty[slot]);
             if (++slot == TS_IRING) { slot = 0; iph ^= 1; }
             if (t < 0) break;
-            const int64_t i = t / S, sl = t % S;
+            RsItem it;
+            rs_decode(p, t, it);
             // per column a two-term FP32 sum (hi, lo) grown by error-free
             // transformations (TwoSum): about 48 significant bits without
             // FP64 arithmetic, which runs at a small fraction of the FP32 rate
-            const int et = threadIdx.x - 64;  // epilogue thread 0..127
-            float ahi[TS_NPMAX];
+            float ahi[NC], alo[NC];
 #pragma unroll
-            for (int q = 0; q < TS_NPMAX; ++q) {
-                ahi[q] = 0.f;
-                alo_s[q * 128 + et] = 0.f;
-            }
+            for (int q = 0; q < NC; ++q) ahi[q] = alo[q] = 0.f;
             bool ok = true;
-            const float kscale = rs_kscale(p.kbound, p.shift);
-            float mlane = 0.f;  // lane q: 1 / (kscale * scale of column q of a_j)
-            for (int64_t jc = 0; jc < nt * KC; ++jc) {
-                const int64_t j = jc / KC;
-                if (jc % KC == 0) mlane = (lane < pc) ? 1.f / (kscale * __ldg(p.sa + j * np + lane)) : 0.f;
-                if (!__all_sync(0xffffffffu, rs_wait(&tfull[acc], aph, p))) { ok = false; break; }
-                tmem_fence_after();
-                const uint32_t tacc = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(acc * 3 * np);
-                float v[TS_NPMAX];
+            for (int j = it.j0; j < it.j1 && ok; ++j) {
+                for (int kc = it.kc0; kc < it.kc1; ++kc) {
+                    // inverse scales of these rows of a (one set per 128 rows)
+                    const float4 *is =
+                        reinterpret_cast<const float4 *>(p.inv_s + (int64_t)(j * p.S + (kc >> 1)) * NP + q0);
+                    float mul[NC];
 #pragma unroll
-                for (int c16 = 0; c16 < TS_NPMAX / 16; ++c16) {
-                    if (c16 * 16 < np) {
-                        float hv[16], mv[16], lv[16];
-                        tmem_ld16(tacc + c16 * 16, hv);
-                        tmem_ld16(tacc + np + c16 * 16, mv);
-                        tmem_ld16(tacc + 2 * np + c16 * 16, lv);
-#pragma unroll
-                        for (int e = 0; e < 16; ++e) v[c16 * 16 + e] = hv[e] + (mv[e] + lv[e]);
+                    for (int q = 0; q < NC; q += 4) {
+                        const float4 m4 = __ldg(is + q / 4);
+                        mul[q] = m4.x, mul[q + 1] = m4.y, mul[q + 2] = m4.z, mul[q + 3] = m4.w;
                     }
-                }
-                tmem_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&tempty[acc]);
-                if (++acc == 2) { acc = 0; aph ^= 1; }
+                    if (!__all_sync(0xffffffffu, rs_wait(&tfull[acc], aph, p))) { ok = false; break; }
+                    tmem_fence_after();
+                    const uint32_t tacc =
+                        tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(acc * 3 * NP + q0);
+                    float v[NC];
 #pragma unroll
-                for (int q = 0; q < TS_NPMAX; ++q) {
-                    const float mq = __shfl_sync(0xffffffffu, mlane, q);
-                    if (q < pc) {
-                        const float xq = v[q] * mq;  // exact: powers of two
+                    for (int c8 = 0; c8 < NC; c8 += 8) {
+                        float hv[8], mv[8], lv[8];
+                        tmem_ld8x3(tacc + c8, tacc + NP + c8, tacc + 2 * NP + c8, hv, mv, lv);
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) v[c8 + e] = hv[e] + (mv[e] + lv[e]);
+                    }
+                    tmem_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&tempty[acc]);
+                    if (++acc == RS_NACC) { acc = 0; aph ^= 1; }
+#pragma unroll
+                    for (int q = 0; q < NC; ++q) {
+                        const float xq = v[q] * mul[q];  // exact: powers of two
                         const float s2 = ahi[q] + xq, bp = s2 - ahi[q];
-                        alo_s[q * 128 + et] += (ahi[q] - (s2 - bp)) + (xq - bp);
+                        alo[q] += (ahi[q] - (s2 - bp)) + (xq - bp);
                         ahi[q] = s2;
                     }
                 }
             }
             if (!ok) break;
-            const int64_t grow = i * b + sl * TS_SLAB + row;
-            const int64_t gi = grow * p.ldx + p.q0;
-            const double c = *p.shift;
+            double *dst = p.part + ((int64_t)it.slot * p.pc + q0) * p.n_pad + (int64_t)it.i * p.b + it.sl * TS_SLAB + row;
 #pragma unroll
-            for (int q = 0; q < TS_NPMAX; ++q)
-                if (q < pc)
-                    p.r[gi + q] = ((double)p.y[gi + q] - (double)p.lambda * (double)p.a[gi + q]) -
-                                  ((double)ahi[q] + (double)alo_s[q * 128 + et]) - c * p.colsum[p.q0 + q];
+            for (int q = 0; q < NC; ++q)
+                if (q0 + q < p.pc) dst[(int64_t)q * p.n_pad] = (double)(ahi[q] * kinv) + (double)(alo[q] * kinv);
         }
     }
     tmem_fence_before();
     __syncthreads();
     if (warp == 1) {
         tmem_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(tcols) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TCOLS) : "memory");
     }
 }
 
-// FP16 pairs of every block of v (one CTA of 128 threads per block).
-__global__ void __launch_bounds__(TS_EPI) convert_all_kernel(const TsParams p, const float *v, __half *vb, float *sv,
-                                                              int terms) {
-    __shared__ float smax[4 * TS_NPMAX], sscale[TS_NPMAX];
-    convert_block(p, v, blockIdx.x, vb, sv, smax, sscale, threadIdx.x, terms);
+// True in every thread of the last block of the grid to come here (`total`
+// blocks count on *ctr); the other blocks' earlier writes are then visible.
+__device__ bool last_block(int *ctr, int total) {
+    __shared__ int last_s;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last_s = (atomicAdd(ctr, 1) == total - 1) ? 1 : 0;
+    __syncthreads();
+    if (last_s) __threadfence();
+    return last_s != 0;
+}
+
+// Operand of the residual: columns [q0, q0 + pc) of a (n_pad x p, row-major) as
+// three FP16 terms, hi = fp16(s v), mid = fp16(s v - hi), lo = fp16(s v - hi -
+// mid), which hold an FP32 value exactly down to 2^-14 of the column maximum
+// (below that the absolute error stays under 2^-38 of the maximum), with one
+// power-of-two scale per column and 128 rows putting the maximum in [4096,
+// 8192); and the column sums of a in FP64 (partials per 128 rows, added in
+// order by the last block).  One block per 128 rows, a row per thread.
+__global__ void __launch_bounds__(TS_EPI)
+    res_operand_kernel(const float *a, int64_t p, int q0, int pc, int np, int64_t n_pad, __half *vb, float *inv_s,
+                       double *cs_part, double *colsum, int *ctr) {
+    __shared__ float xs[TS_SLAB][TS_NPMAX + 1];
+    __shared__ float pmax[8 * TS_NPMAX], scale[TS_NPMAX];
+    __shared__ double psum[8 * TS_NPMAX];
+    const int t = threadIdx.x;
+    const int64_t grow = (int64_t)blockIdx.x * TS_SLAB + t;
+    const float *src = a + grow * p + q0;
+    for (int q = 0; q < np; ++q) xs[t][q] = (q < pc) ? src[q] : 0.f;
+    __syncthreads();
+    // np columns x parts of the rows
+    const int parts = TS_EPI / np, rows = TS_SLAB / parts;
+    {
+        const int q = t % np, part = t / np;
+        if (part < parts) {
+            float m = 0.f;
+            double s = 0.0;
+            for (int r = part * rows; r < (part + 1) * rows; ++r) {
+                m = fmaxf(m, fabsf(xs[r][q]));
+                s += (double)xs[r][q];
+            }
+            pmax[part * np + q] = m;
+            psum[part * np + q] = s;
+        }
+    }
+    __syncthreads();
+    if (t < np) {
+        float m = 0.f;
+        double s = 0.0;
+        for (int e = 0; e < parts; ++e) {
+            m = fmaxf(m, pmax[e * np + t]);
+            s += psum[e * np + t];
+        }
+        float sc = 1.f;
+        if (m > 0.f && m < 3.0e38f) {
+            int e;
+            frexpf(m, &e);  // m = f 2^e, f in [0.5, 1)
+            sc = ldexpf(1.f, max(-126, min(126, 13 - e)));
+        }
+        scale[t] = sc;
+        inv_s[(int64_t)blockIdx.x * np + t] = 1.f / sc;  // a power of two: exact
+        if (t < pc) cs_part[(int64_t)blockIdx.x * pc + t] = s;
+    }
+    __syncthreads();
+    for (int q = 0; q < np; ++q) {
+        const float x = xs[t][q] * scale[q];
+        const __half hh = __float2half_rn(x);
+        const float r1 = x - __half2float(hh);  // exact
+        const __half m = __float2half_rn(r1);
+        vb[(int64_t)q * n_pad + grow] = hh;
+        vb[(int64_t)(np + q) * n_pad + grow] = m;
+        vb[(int64_t)(2 * np + q) * n_pad + grow] = __float2half_rn(r1 - __half2float(m));
+    }
+    if (!last_block(ctr, gridDim.x)) return;
+    // lanes over the blocks, then a fixed tree
+    const int lane = t & 31;
+    for (int q = t >> 5; q < pc; q += TS_EPI / 32) {
+        double s = 0.0;
+        for (int64_t e = lane; e < gridDim.x; e += 32) s += __ldcg(cs_part + e * pc + q);
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+        if (lane == 0) colsum[q0 + q] = s;
+    }
+}
+
+// r = y - lambda a - (the slots in order) - c colsum for columns [q0, q0 + pc),
+// rounded to FP32 and written column-major (the sweeps' right-hand side), and
+// ||r||_F^2, ||y||_F^2 over all p columns into out[0], out[1]: a partial per
+// block (blocks of all column chunks count on ctr), added in order by the last.
+__global__ void __launch_bounds__(256)
+    res_finish_kernel(const float *y, const float *a, int64_t p, int q0, int pc, int64_t n_pad, const double *part,
+                      int slots, float lambda, const double *shift, const double *colsum, float *rt, double *np_part,
+                      int total, int *ctr, double *out) {
+    __shared__ double s1[8], s2[8];
+    const int t = threadIdx.x, q = blockIdx.y;
+    const int64_t r = (int64_t)blockIdx.x * 256 + t;
+    double rv = 0.0, yv = 0.0;
+    if (r < n_pad) {
+        double sum = 0.0;
+        const double *src = part + (int64_t)q * n_pad + r;
+        const int64_t step = (int64_t)pc * n_pad;
+#pragma unroll 4
+        for (int e = 0; e < slots; ++e) sum += __ldcs(src + e * step);
+        yv = (double)y[r * p + q0 + q];
+        rv = (yv - (double)lambda * (double)a[r * p + q0 + q]) - sum - *shift * colsum[q0 + q];
+        rt[(int64_t)(q0 + q) * n_pad + r] = (float)rv;
+    }
+    double v1 = rv * rv, v2 = yv * yv;
+    for (int o = 16; o > 0; o >>= 1) {
+        v1 += __shfl_down_sync(0xffffffffu, v1, o);
+        v2 += __shfl_down_sync(0xffffffffu, v2, o);
+    }
+    if ((t & 31) == 0) {
+        s1[t >> 5] = v1;
+        s2[t >> 5] = v2;
+    }
+    __syncthreads();
+    if (t == 0) {
+        double x = 0.0, z = 0.0;
+        for (int w = 0; w < 8; ++w) {
+            x += s1[w];
+            z += s2[w];
+        }
+        const int64_t slot = (int64_t)(q0 + q) * gridDim.x + blockIdx.x;
+        np_part[2 * slot] = x;
+        np_part[2 * slot + 1] = z;
+    }
+    if (!last_block(ctr, total)) return;
+    double x = 0.0, z = 0.0;
+    for (int e = t; e < total; e += 256) {
+        x += __ldcg(np_part + 2 * e);
+        z += __ldcg(np_part + 2 * e + 1);
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        x += __shfl_down_sync(0xffffffffu, x, o);
+        z += __shfl_down_sync(0xffffffffu, z, o);
+    }
+    if ((t & 31) == 0) {
+        s1[t >> 5] = x;
+        s2[t >> 5] = z;
+    }
+    __syncthreads();
+    if (t == 0) {
+        x = z = 0.0;
+        for (int w = 0; w < 8; ++w) {
+            x += s1[w];
+            z += s2[w];
+        }
+        out[0] = x;
+        out[1] = z;
+    }
 }
 
 // Encoder of TMA descriptors (driver entry point, looked up once).
@@ -1382,8 +1559,10 @@ float *ts_maxima(Ctx *c) { return ts_scales(c) + 2 * ts_scale_count(c); }
 float *ts_block_maxima(Ctx *c) { return ts_maxima(c) + 2 * ts_max_count(c); }
 int *ts_flags(Ctx *c) { return (int *)(ts_block_maxima(c) + 2 * ts_scale_count(c)); }
 
-// dst (cols x rows, row-major) = src^T, src rows x cols row-major.
-__global__ void transpose_kernel(const float *__restrict__ src, int64_t rows, int64_t cols, float *__restrict__ dst) {
+// dst (cols x rows, row-major) = src^T, src rows x cols row-major; with sum,
+// also sum += src^T.
+__global__ void transpose_kernel(const float *__restrict__ src, int64_t rows, int64_t cols, float *__restrict__ dst,
+                                 float *__restrict__ sum) {
     __shared__ float t[32][33];
     const int64_t r0 = (int64_t)blockIdx.y * 32, c0 = (int64_t)blockIdx.x * 32;
     for (int k = threadIdx.y; k < 32; k += 8) {
@@ -1393,13 +1572,16 @@ __global__ void transpose_kernel(const float *__restrict__ src, int64_t rows, in
     __syncthreads();
     for (int k = threadIdx.y; k < 32; k += 8) {
         const int64_t cc = c0 + k, r = r0 + threadIdx.x;
-        if (r < rows && cc < cols) dst[cc * rows + r] = t[threadIdx.x][k];
+        if (r < rows && cc < cols) {
+            dst[cc * rows + r] = t[threadIdx.x][k];
+            if (sum) sum[cc * rows + r] += t[threadIdx.x][k];
+        }
     }
 }
 
-void launch_transpose(const float *src, int64_t rows, int64_t cols, float *dst, cudaStream_t s) {
+void launch_transpose(const float *src, int64_t rows, int64_t cols, float *dst, cudaStream_t s, float *sum = nullptr) {
     const dim3 grid((unsigned)((cols + 31) / 32), (unsigned)((rows + 31) / 32));
-    count_launch(), transpose_kernel<<<grid, dim3(32, 8), 0, s>>>(src, rows, cols, dst);
+    count_launch(), transpose_kernel<<<grid, dim3(32, 8), 0, s>>>(src, rows, cols, dst, sum);
 }
 
 krr_status run_ts(Ctx *c, int job, float *rhs, float *out, int64_t p) {
@@ -1486,17 +1668,19 @@ krr_status run_ts(Ctx *c, int job, float *rhs, float *out, int64_t p) {
 
 }  // namespace
 
-// x (n_pad x p) <- (L L^T)^-1 x with the stored mixed-precision factor on the
-// tensor cores: the forward sweep updates x in place and writes z to tmp, the
-// backward sweep updates tmp in place and writes the solution to x.
-krr_status tc_sweep_solve(Ctx *c, float *x, float *tmp, int64_t p) {
+// x (n_pad x p) <- (L L^T)^-1 rhs with the stored mixed-precision factor on the
+// tensor cores; the sweeps work on the column-major copy ts_xt: the forward
+// sweep updates it in place and writes z to tmp, the backward sweep updates
+// tmp in place and writes the solution to ts_xt.  rhs: row-major right-hand
+// sides, or nullptr when ts_xt holds them already (tc_residual).  sum
+// (optional): also sum += x.
+krr_status tc_sweep_solve(Ctx *c, const float *rhs, float *x, float *tmp, int64_t p, float *sum) {
     KRR_TRY(ensure_ts_buffers(c, p));
-    // the sweeps work on column-major copies: x^T in ts_xt, z^T in tmp
     float *xt = c->ts_xt;
-    launch_transpose(x, c->n_pad, p, xt, c->stream);
+    if (rhs) launch_transpose(rhs, c->n_pad, p, xt, c->stream);
     KRR_TRY(run_ts(c, TS_FWD, xt, tmp, p));
     KRR_TRY(run_ts(c, TS_BWD, tmp, xt, p));
-    launch_transpose(xt, p, c->n_pad, x, c->stream);
+    launch_transpose(xt, p, c->n_pad, x, c->stream, sum);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
         c->last_error = std::string("sweep transposes: ") + cudaGetErrorString(e);
@@ -1525,87 +1709,102 @@ krr_status map_f32(Ctx *c, CUtensorMap *m, const void *base, int64_t rows, int64
     return KRR_OK;
 }
 
-size_t rs_smem_bytes(int b_bytes) {
-    return (size_t)RS_NSTG * RS_STG + (size_t)RS_NB * b_bytes + TS_IRING * 8 +
-           (size_t)(3 * RS_NSTG + 2 * RS_NB + 4 + 2 * TS_IRING + 1) * 8 + 16 +
-           (size_t)TS_NPMAX * 128 * 4 + 1024;
+size_t rs_smem_bytes(int np) {
+    return (size_t)RS_NSTG * (RS_STG + 3 * np * 128) + TS_IRING * sizeof(int) +
+           (size_t)(3 * RS_NSTG + 2 * RS_NACC + 2 * TS_IRING + 1) * 8 + 16 + 1024;
+}
+
+template <int NP>
+krr_status launch_res(Ctx *c, const CUtensorMap &mk128, const CUtensorMap &mk64, const CUtensorMap &ma,
+                      const RsParams &rp) {
+    static PerDevice attr;
+    if (!attr.has(c->device)) {
+        KRR_CUDA_TRY(c, cudaFuncSetAttribute(tcres_kernel<NP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)ts_smem_limit()));
+        attr.put(c->device);
+    }
+    const int64_t grid = std::min<int64_t>(rp.items, grid_limit(c, GL_RESIDUAL));
+    count_launch(), tcres_kernel<NP><<<(unsigned)grid, RS_THREADS, rs_smem_bytes(NP), c->stream>>>(mk128, mk64, ma, rp);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) {
+        c->last_error = std::string("tensor-core residual launch: ") + cudaGetErrorString(e);
+        return KRR_ECUDA;
+    }
+    return KRR_OK;
 }
 
 }  // namespace
 
-// r = y - (K + lambda I) a on the tensor cores (mixed mode), given the column
-// sums of a in c->colsum and the shift in c->red[RED_KSHIFT].
-krr_status tc_residual(Ctx *c, const float *y, const float *a, double *r, int64_t p) {
-    const int64_t b = c->b, nt = c->nt;
-    KRR_TRY(ensure_ts_buffers(c, 0));
-    float *sbase = ts_scales(c);
+// r = y - (K + lambda I) a on the tensor cores (mixed mode), rounded to FP32
+// and column-major in c->ts_xt, the right-hand side of the next sweeps;
+// ||r||_F^2 and ||y||_F^2 into c->red[RED_RNORM], [RED_RNORM + 1].
+krr_status tc_residual(Ctx *c, const float *y, const float *a, int64_t p) {
+    const int64_t b = c->b, nt = c->nt, S = b / TS_SLAB, n_pad = c->n_pad;
+    KRR_TRY(ensure_ts_buffers(c, p));
     int *flags = ts_flags(c);
     const int64_t ntri = nt * (nt + 1) / 2;
     CUtensorMap mk128, mk64, ma;
     KRR_TRY(map_f32(c, &mk128, c->Kd, ntri * b, b, 128));
     KRR_TRY(map_f32(c, &mk64, c->Kd, ntri * b, b, 64));
-    static PerDevice attr;
-    if (!attr.has(c->device)) {
-        const cudaError_t e =
-            cudaFuncSetAttribute(tcres_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ts_smem_limit());
-        if (e != cudaSuccess) {
-            c->last_error = std::string("cudaFuncSetAttribute (tensor-core residual): ") + cudaGetErrorString(e);
-            return KRR_ECUDA;
-        }
-        attr.put(c->device);
+    // Source blocks of an item: one up to 48 blocks, above that so many that
+    // the slots stay at 48 or fewer (their 16 bytes of traffic per slot, row
+    // and column against 4 bytes per entry of K: 48 slots and 20 columns add
+    // 4 % at N = 98304); a few large groups would outgrow L2 between the two
+    // uses of a tile.  A tile is split (in parts of at least four 64-wide
+    // chunks) while that leaves fewer than six items an SM: N = 5000 has 200
+    // whole-tile items for 152 SMs.
+    const int KC = (int)(b / TS_KC);
+    const int g = (int)((nt + 47) / 48);
+    int h = 1;
+    if (g == 1)
+        while (KC / (2 * h) >= 4 && nt * nt * S * h < 6 * grid_limit(c, GL_RESIDUAL)) h *= 2;
+    const int64_t ngrp = (nt + g - 1) / g, slots = ngrp * h;
+    const int64_t pmax = std::min<int64_t>(p, TS_NPMAX);
+    const int64_t nblk = n_pad / TS_SLAB, fblk = (n_pad + 255) / 256;
+    const int64_t part_count = slots * pmax * n_pad, need = part_count + nblk * pmax + 2 * fblk * p;
+    if (c->rs_part_cap < need) {
+        c->rs_part_cap = 0;
+        KRR_TRY(dev_alloc(c, &c->rs_part, (size_t)need, "residual partial sums"));
+        c->rs_part_cap = need;
     }
+    double *cs_part = c->rs_part + part_count, *np_part = cs_part + nblk * pmax;
+    float *inv_s = ts_maxima(c);
     for (int64_t q0 = 0; q0 < p; q0 += TS_NPMAX) {
-        // the FP16 pair of a with per-block scales (B operand)
-        TsParams cp;
-        memset(&cp, 0, sizeof(cp));
-        cp.b = b;
-        cp.nt = nt;
-        cp.n_pad = c->n_pad;
-        cp.pc = (int)std::min<int64_t>(TS_NPMAX, p - q0);
-        cp.np = (cp.pc + 15) & ~15;
-        cp.q0 = (int)q0;
-        cp.S = b / TS_SLAB;
-        cp.rs = p;  // a is row-major here
-        cp.cs = 1;
-        count_launch(), convert_all_kernel<<<(unsigned)nt, TS_EPI, 0, c->stream>>>(cp, a, c->ts_v0, sbase, 3);
-        KRR_TRY(map_f16(c, &ma, c->ts_v0, 3 * cp.np, c->n_pad, 3 * cp.np));
+        const int pc = (int)std::min<int64_t>(TS_NPMAX, p - q0), np = (pc + 15) & ~15;
+        // item counter, abort flag, block counters of the two small kernels
+        // (the second one's runs over all column chunks)
+        KRR_CUDA_TRY(c, cudaMemsetAsync(flags, 0, (q0 == 0 ? 4 : 3) * sizeof(int), c->stream));
+        count_launch(), res_operand_kernel<<<(unsigned)nblk, TS_EPI, 0, c->stream>>>(
+            a, p, (int)q0, pc, np, n_pad, c->ts_v0, inv_s, cs_part, c->colsum, flags + 2);
+        KRR_TRY(map_f16(c, &ma, c->ts_v0, 3 * np, n_pad, 3 * np));
         RsParams rp;
         memset(&rp, 0, sizeof(rp));
-        rp.b = b;
-        rp.nt = nt;
-        rp.S = b / TS_SLAB;
-        rp.KC = b / TS_KC;
-        rp.items = nt * rp.S;
-        rp.n_pad = c->n_pad;
-        rp.np = cp.np;
-        rp.pc = cp.pc;
-        rp.q0 = cp.q0;
-        rp.ldx = p;
-        rp.y = y;
-        rp.a = a;
-        rp.r = r;
+        rp.b = (int)b;
+        rp.nt = (int)nt;
+        rp.S = (int)S;
+        rp.KC = KC;
+        rp.g = g;
+        rp.h = h;
+        rp.ngrp = (int)ngrp;
+        rp.items = (int)(ngrp * (ngrp + 1) / 2 * 2 * g * S * h);
+        rp.n_pad = n_pad;
+        rp.pc = pc;
         rp.shift = c->red + RED_KSHIFT;
         rp.kbound = c->red + RED_KBOUND;
-        rp.colsum = c->colsum;
-        rp.lambda = (float)c->lambda;
-        rp.sa = sbase;
+        rp.inv_s = inv_s;
+        rp.part = c->rs_part;
         rp.flags = flags;
-        rp.b_bytes = 3 * rp.np * 128;
-        rp.idesc_k = (1u << 4) | ((uint32_t)((3 * rp.np) >> 3) << 17) | ((uint32_t)(TS_SLAB >> 4) << 24);
+        rp.idesc_k = (1u << 4) | ((uint32_t)((3 * np) >> 3) << 17) | ((uint32_t)(TS_SLAB >> 4) << 24);
         rp.idesc_mn = rp.idesc_k | (1u << 15);
-        rp.idesc_k2 = (1u << 4) | ((uint32_t)((2 * rp.np) >> 3) << 17) | ((uint32_t)(TS_SLAB >> 4) << 24);
+        rp.idesc_k2 = (1u << 4) | ((uint32_t)((2 * np) >> 3) << 17) | ((uint32_t)(TS_SLAB >> 4) << 24);
         rp.idesc_mn2 = rp.idesc_k2 | (1u << 15);
         rp.wait_ns = (uint64_t)c->opt.wait_budget_ns;
         rp.err = c->derr;
-        KRR_CUDA_TRY(c, cudaMemsetAsync(flags, 0, 2 * sizeof(int), c->stream));
-        const size_t smem = rs_smem_bytes(rp.b_bytes);
-        const int64_t grid = std::min<int64_t>(rp.items, grid_limit(c, GL_RESIDUAL));
-        count_launch(), tcres_kernel<<<(unsigned)grid, RS_THREADS, smem, c->stream>>>(mk128, mk64, ma, rp);
-        const cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) {
-            c->last_error = std::string("tensor-core residual launch: ") + cudaGetErrorString(e);
-            return KRR_ECUDA;
-        }
+        KRR_TRY(np == 16 ? launch_res<16>(c, mk128, mk64, ma, rp) : launch_res<32>(c, mk128, mk64, ma, rp));
+        count_launch(), res_finish_kernel<<<dim3((unsigned)fblk, (unsigned)pc), 256, 0, c->stream>>>(
+            y, a, p, (int)q0, pc, n_pad, c->rs_part, (int)slots, (float)c->lambda, c->red + RED_KSHIFT, c->colsum,
+            c->ts_xt, np_part, (int)(fblk * p), flags + 3, c->red + RED_RNORM);
+        KRR_TRY(check_launch(c, "residual"));
     }
     return KRR_OK;
 }

@@ -15,15 +15,18 @@
 //      an exact FP16 pair (hi, lo) and contribute two A phases; E4M3 tiles are
 //      read from their FP16 copy; the diagonal inverses from their FP16 split.
 //   B  the vector block as an FP16 pair (hi, lo) with one power-of-two scale
-//      per block and column, K-major ([column][row]); both halves are
-//      multiplied, so B carries about 22 significant bits.
+//      per block and column, both halves multiplied, so B carries about 22
+//      significant bits; stored in groups of 64 rows, [group][hi columns, lo
+//      columns][64], so that a block is contiguous and arrives in a few large
+//      copies, once for the hi and lo phases of an item.
 // The right-hand side is updated in place; a LINK applies its update after the
 // earlier ones of the same slab (fixed order: deterministic results).  A slab
 // whose rows become final (a DIAG slab, the last LINK of a slab) writes them
-// at once as the FP16 pair with a scale predicted from the previous block; the
-// last slab of the block checks the prediction against the block's maximum
-// (converting the whole block again with the exact scale if it fails) and
-// publishes the block.
+// at once as the FP16 pair with a scale predicted from the previous block and
+// adds itself, and whether its maxima fit that scale, to the block's state.  A
+// reader finds there that every slab is finished and the scales hold; if they
+// do not, the last slab converts the whole block again with the exact scale and
+// the reader waits for that.
 //
 // Items are claimed from a device counter in dependency order (item 0 converts
 // the first block; then, per column, its S DIAG items, its head LINK items and
@@ -32,12 +35,26 @@
 // (%globaltimer) and ends the kernel with KRR_ETIMEOUT.
 //
 // CTA (192 threads, one per SM):
-//   warp 0      producer: claims items, TMA loads of A (16 KB per stage) and B
-//               into a shared-memory ring; B only after the block it reads has
-//               been published (the A loads of the first stages go out first);
+//   warp 0      producer: claims items, TMA loads of A (16 KB a stage) into a
+//               shared-memory ring and of B into a buffer of its own.  The A
+//               loads of the first stages go out before the block that the item
+//               reads is final; the B copies as soon as it is, while the lanes
+//               check that its predicted scales hold;
 //   warp 1      TMEM allocation and the single MMA-issuing thread;
 //   warps 2..5  epilogue: TMEM -> registers, scales, the in-place update or the
-//               DIAG store, progress counters and block conversions.
+//               DIAG store, FP16 pairs, progress counters.
+//
+// What bounds it: the chain DIAG -> head LINK -> DIAG, two hops a column.  At
+// N = 32768, b = 1024, P = 10 the two took 36 us: 10 and 5.4 us from the
+// publication of the block they read to the last MMA, 5 us of epilogue each,
+// 3.3 us each to find the block's maxima, accept its scales and publish it.  Now
+// 20 us: the epilogue takes 1 us (branch-free per column, its loads before the
+// accumulator wait), the scales are accepted with the load that finds the block
+// finished, B arrives in large copies (0.4-0.9 us) and a chunk's MMAs are issued
+// in 0.2 us instead of 0.3 (uniform descriptors, the next stage's barrier tested
+// ahead); publication and its discovery are 1.5 us a hop.  A pair of sweeps took
+// 2.24 ms, now 1.28; N = 5000, P = 2 0.38 and 0.20; N = 2048, b = 256, P = 1 0.335
+// and 0.159 ms.
 #include <cuda.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -59,6 +76,8 @@ constexpr int TS_KC = 64;                // K elements of a stage (128 bytes of 
 constexpr int TS_ABYTES = TS_SLAB * 128;  // A bytes of a stage
 constexpr int TS_NPMAX = 32;             // right-hand sides per launch
 constexpr int TS_IRING = 4;              // item header slots
+constexpr int TS_BSEG = 16;              // most groups of 64 rows of the vector block held at once
+constexpr int TS_BBOX = 256;             // rows of a B copy (groups x columns of a group)
 
 enum { TS_FWD = 0, TS_BWD = 1 };
 enum { IT_CONV = 0, IT_DIAG = 1, IT_LINK = 2, IT_END = 3 };
@@ -72,13 +91,14 @@ struct TsParams {
     int64_t rs, cs;           // vector element (row, column q0 + q) at row * rs + (q0 + q) * cs
     float *rhs;               // FWD: y, BWD: z (updated in place)
     float *out;               // FWD: z, BWD: x
-    float *mx_in, *mx_out;    // per-slab column maxima of rhs / out blocks, [nt][S][TS_NPMAX]
-    float *bm_in, *bm_out;    // their block column maxima, [nt][TS_NPMAX]
-    __half *vin, *vout;       // FP16 pairs of rhs / out blocks: [2 np][n_pad] (hi rows, then lo rows)
-    float *sin, *sout;        // their scales, [nt][np]
+    float *bm_in, *bm_out;    // column maxima of rhs / out blocks (zero at the start), [nt][TS_NPMAX]
+    __half *vin, *vout;       // FP16 pairs of rhs / out blocks: [n_pad / 64][2 np][64] (hi, then lo columns)
+    float *sin, *sout;        // exact scales of blocks converted as a whole, [nt][np]
     const TileDesc *ltab;
-    int *flags;               // [0] items, [1] abort, cin[nt], cout[nt], done[nt], ready[nt], seq[nt * S]
-    int stages, stage_bytes;
+    unsigned long long *st_in, *st_out;  // state of the rhs / out blocks, [nt]
+    int *flags;               // [0] items, [1] abort, xin[nt], xout[nt], seq[nt * S]
+    int stages;
+    int lkc, bseg;            // log2 KC; groups of B held at once (KC, or TS_BSEG)
     uint32_t idesc;
     uint64_t wait_ns;
     DevErrors *err;
@@ -95,11 +115,22 @@ struct ItemHdr {
     float inv_tscale;        // 1 / tile scale
 };
 
-__device__ __forceinline__ int *cin_ctr(const TsParams &p) { return p.flags + 2; }
-__device__ __forceinline__ int *cout_ctr(const TsParams &p) { return p.flags + 2 + p.nt; }
-__device__ __forceinline__ int *done_ctr(const TsParams &p) { return p.flags + 2 + 2 * p.nt; }
-__device__ __forceinline__ int *ready_ctr(const TsParams &p) { return p.flags + 2 + 3 * p.nt; }
-__device__ __forceinline__ int *seq_ctr(const TsParams &p) { return p.flags + 2 + 4 * p.nt; }
+// Whether a block of the right-hand side / of the solution was converted as a
+// whole with its exact scale, and the updates applied to each slab.
+__device__ __forceinline__ int *xin_ctr(const TsParams &p) { return p.flags + 2; }
+__device__ __forceinline__ int *xout_ctr(const TsParams &p) { return p.flags + 2 + p.nt; }
+__device__ __forceinline__ int *seq_ctr(const TsParams &p) { return p.flags + 2 + 2 * p.nt; }
+
+// State of a block, one 64-bit word: finished slabs (bits 0-15), columns found
+// too large for the predicted scale by some warp (a count, bits 16-31), and the
+// columns that some warp found large enough for it (bits 32-63).  A reader
+// learns with one load that the block is there and whether its predicted
+// scales hold: for every column the maximum lies in [PRED_LO, PRED_HI).
+__device__ __forceinline__ int state_slabs(unsigned long long v) { return (int)(v & 0xffff); }
+__device__ __forceinline__ bool state_holds(unsigned long long v, int pc) {
+    const uint32_t all = pc == 32 ? 0xffffffffu : (1u << pc) - 1u;
+    return ((v >> 16) & 0xffff) == 0 && ((uint32_t)(v >> 32) & all) == all;
+}
 
 __device__ __forceinline__ uint32_t smem_u32(const void *ptr) {
     return (uint32_t)__cvta_generic_to_shared(ptr);
@@ -139,6 +170,12 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
 __device__ __forceinline__ int ld_acquire(const int *ptr) {
     int v;
     asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(ptr) : "memory");
+    return v;
+}
+
+__device__ __forceinline__ unsigned long long ld_acquire64(const unsigned long long *ptr) {
+    unsigned long long v;
+    asm volatile("ld.acquire.gpu.global.b64 %0, [%1];" : "=l"(v) : "l"(ptr) : "memory");
     return v;
 }
 
@@ -196,6 +233,26 @@ __device__ __forceinline__ bool wait_count(const int *ctr, int target, const TsP
     }
 }
 
+// Bounded wait until all slabs of a block are finished; its state then.
+__device__ __forceinline__ bool wait_state(const unsigned long long *ptr, int slabs, unsigned long long *v,
+                                           const TsParams &p) {
+    if (state_slabs(*v = ld_acquire64(ptr)) >= slabs) return true;
+    const uint64_t t0 = globaltimer();
+    uint32_t nap = 32;
+    for (uint32_t it = 1;; ++it) {
+        __nanosleep(nap);
+        if (nap < 128) nap <<= 1;
+        if (state_slabs(*v = ld_acquire64(ptr)) >= slabs) return true;
+        if ((it & 15) == 0) {
+            if (aborted(p)) return false;
+            if (globaltimer() - t0 > p.wait_ns) {
+                record_timeout(p);
+                return false;
+            }
+        }
+    }
+}
+
 __device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, int x, int y, uint64_t *bar) {
     asm volatile(
         "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
@@ -237,6 +294,13 @@ __device__ __forceinline__ void mma_f16(uint32_t tmem_d, uint64_t adesc, uint64_
         "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc));
 }
 
+// One lane of the (converged) warp, the same each time.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t r;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r));
+    return r != 0;
+}
+
 __device__ __forceinline__ void mma_commit(uint64_t *bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
                  : "memory");
@@ -245,18 +309,38 @@ __device__ __forceinline__ void mma_commit(uint64_t *bar) {
 __device__ __forceinline__ void tmem_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tmem_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float *v) {
-    uint32_t r[16];
+// Sum of the eight groups of eight TMEM columns at t + g * step: every load is
+// in flight before the one wait.
+__device__ __forceinline__ void tmem_sum8x8(uint32_t t, uint32_t step, float *v) {
+    uint32_t r[64];
     asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,"
-        "%15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-          "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
-          "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%64];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%8,%9,%10,%11,%12,%13,%14,%15}, [%65];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%16,%17,%18,%19,%20,%21,%22,%23}, [%66];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%24,%25,%26,%27,%28,%29,%30,%31}, [%67];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%32,%33,%34,%35,%36,%37,%38,%39}, [%68];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%40,%41,%42,%43,%44,%45,%46,%47}, [%69];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%48,%49,%50,%51,%52,%53,%54,%55}, [%70];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%56,%57,%58,%59,%60,%61,%62,%63}, [%71];\n\t"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=&r"(r[0]), "=&r"(r[1]), "=&r"(r[2]), "=&r"(r[3]), "=&r"(r[4]), "=&r"(r[5]), "=&r"(r[6]), "=&r"(r[7]),
+          "=&r"(r[8]), "=&r"(r[9]), "=&r"(r[10]), "=&r"(r[11]), "=&r"(r[12]), "=&r"(r[13]), "=&r"(r[14]), "=&r"(r[15]),
+          "=&r"(r[16]), "=&r"(r[17]), "=&r"(r[18]), "=&r"(r[19]), "=&r"(r[20]), "=&r"(r[21]), "=&r"(r[22]), "=&r"(r[23]),
+          "=&r"(r[24]), "=&r"(r[25]), "=&r"(r[26]), "=&r"(r[27]), "=&r"(r[28]), "=&r"(r[29]), "=&r"(r[30]), "=&r"(r[31]),
+          "=&r"(r[32]), "=&r"(r[33]), "=&r"(r[34]), "=&r"(r[35]), "=&r"(r[36]), "=&r"(r[37]), "=&r"(r[38]), "=&r"(r[39]),
+          "=&r"(r[40]), "=&r"(r[41]), "=&r"(r[42]), "=&r"(r[43]), "=&r"(r[44]), "=&r"(r[45]), "=&r"(r[46]), "=&r"(r[47]),
+          "=&r"(r[48]), "=&r"(r[49]), "=&r"(r[50]), "=&r"(r[51]), "=&r"(r[52]), "=&r"(r[53]), "=&r"(r[54]), "=&r"(r[55]),
+          "=&r"(r[56]), "=&r"(r[57]), "=&r"(r[58]), "=&r"(r[59]), "=&r"(r[60]), "=&r"(r[61]), "=&r"(r[62]), "=&r"(r[63])
+        : "r"(t), "r"(t + step), "r"(t + 2 * step), "r"(t + 3 * step), "r"(t + 4 * step), "r"(t + 5 * step),
+          "r"(t + 6 * step), "r"(t + 7 * step)
+        : "memory");
 #pragma unroll
-    for (int e = 0; e < 16; ++e) v[e] = __uint_as_float(r[e]);
+    for (int e = 0; e < 8; ++e) {
+        float x[8];
+#pragma unroll
+        for (int g = 0; g < 8; ++g) x[g] = __uint_as_float(r[8 * g + e]);
+        v[e] = ((x[0] + x[2]) + (x[4] + x[6])) + ((x[1] + x[3]) + (x[5] + x[7]));
+    }
 }
 
 __device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
@@ -366,56 +450,34 @@ __device__ void decode_item(const TsParams &p, int64_t t, ItemHdr &h) {
 // [q0, q0 + pc) -> FP16 terms with the power-of-two scale s_q putting the
 // column maximum in [4096, 8192) (8x headroom below the FP16 maximum):
 // two terms hi = fp16(s v), lo = fp16(s v - hi) (about 22 significant bits).
-// Planes of np rows each; padding columns [pc, np) are zero.
+// Padding columns [pc, np) are zero.  The column maxima are those in bmax, or found here and written there (find).
 // ---------------------------------------------------------------------------
-__device__ void convert_block(const TsParams &p, const float *v, int64_t blk, __half *vb, float *sv,
-                              float *smax, float *sscale, int tid, const float *slabmax, float *bmax) {
-    const int64_t b = p.b, n_pad = p.n_pad, rs = p.rs, cs = p.cs;
+__device__ __noinline__ void convert_block(const TsParams &p, const float *v, int64_t blk, __half *vb, float *sv,
+                                           float *smax, float *sscale, int tid, bool find, float *bmax) {
+    const int64_t b = p.b, rs = p.rs, cs = p.cs;
     const int pc = p.pc, np = p.np;
-    if (slabmax) {
-        // column maxima published by the slabs of the block
-        if (tid < pc) {
+    const int wq = tid >> 5, lane = tid & 31;
+    for (int q = 0; q < np; ++q) {
+        if (find && q < pc) {
             float m = 0.f;
-            for (int64_t sl = 0; sl < p.S; ++sl) m = fmaxf(m, __ldcg(slabmax + (blk * p.S + sl) * TS_NPMAX + tid));
-            smax[tid] = m;
-            smax[TS_NPMAX + tid] = smax[2 * TS_NPMAX + tid] = smax[3 * TS_NPMAX + tid] = 0.f;
-        }
-    } else {
-        float mx[TS_NPMAX];
-#pragma unroll
-        for (int q = 0; q < TS_NPMAX; ++q) mx[q] = 0.f;
-        for (int64_t r = tid; r < b; r += TS_EPI) {
-            const float *row = v + (blk * b + r) * rs + p.q0 * cs;
-#pragma unroll
-            for (int q = 0; q < TS_NPMAX; ++q) {
-                if (q < pc) {
-                    mx[q] = fmaxf(mx[q], fabsf(__ldcg(row)));
-                    row += cs;
-                }
-            }
-        }
-        const int wq = tid >> 5, lane = tid & 31;
-#pragma unroll
-        for (int q = 0; q < TS_NPMAX; ++q) {
-            if (q < pc) {
-                float m = mx[q];
-                for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-                if (lane == 0) smax[wq * TS_NPMAX + q] = m;
-            }
+            for (int64_t r = tid; r < b; r += TS_EPI) m = fmaxf(m, fabsf(__ldcg(v + (blk * b + r) * rs + (p.q0 + q) * cs)));
+            for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+            if (lane == 0) smax[wq * TS_NPMAX + q] = m;
         }
     }
     epi_sync();
     if (tid < np) {
         float s = 1.f;
         if (tid < pc) {
-            const float m = fmaxf(fmaxf(smax[tid], smax[TS_NPMAX + tid]),
-                                  fmaxf(smax[2 * TS_NPMAX + tid], smax[3 * TS_NPMAX + tid]));
+            const float m = find ? fmaxf(fmaxf(smax[tid], smax[TS_NPMAX + tid]),
+                                         fmaxf(smax[2 * TS_NPMAX + tid], smax[3 * TS_NPMAX + tid]))
+                                 : __ldcg(bmax + blk * TS_NPMAX + tid);
             if (m > 0.f && m < 3.0e38f) {
                 int e;
                 frexpf(m, &e);  // m = f 2^e, f in [0.5, 1)
                 s = ldexpf(1.f, max(-126, min(126, 13 - e)));
             }
-            bmax[blk * TS_NPMAX + tid] = m;
+            if (find) bmax[blk * TS_NPMAX + tid] = m;
         }
         sscale[tid] = s;
         sv[blk * np + tid] = s;
@@ -423,24 +485,13 @@ __device__ void convert_block(const TsParams &p, const float *v, int64_t blk, __
     epi_sync();
     for (int64_t r = tid; r < b; r += TS_EPI) {
         const int64_t grow = blk * b + r;
-        const float *row = v + grow * rs + p.q0 * cs;
-        // the row's loads first (the FP16 stores below may alias them)
-        float xv[TS_NPMAX];
-#pragma unroll
-        for (int q = 0; q < TS_NPMAX; ++q) {
-            if (q < pc) {
-                xv[q] = __ldcg(row);
-                row += cs;
-            }
-        }
-#pragma unroll
-        for (int q = 0; q < TS_NPMAX; ++q) {
-            if (q < np) {
-                const float x = (q < pc) ? xv[q] * sscale[q] : 0.f;
-                const __half hh = __float2half_rn(x);
-                vb[(int64_t)q * n_pad + grow] = hh;
-                vb[(int64_t)(np + q) * n_pad + grow] = __float2half_rn(x - __half2float(hh));
-            }
+#pragma unroll 4
+        for (int q = 0; q < np; ++q) {
+            const float x = (q < pc) ? __ldcg(v + grow * rs + (p.q0 + q) * cs) * sscale[q] : 0.f;
+            const __half hh = __float2half_rn(x);
+            __half *dst = vb + (grow >> 6) * 2 * np * 64 + (grow & 63);
+            dst[q * 64] = hh;
+            dst[(np + q) * 64] = __float2half_rn(x - __half2float(hh));
         }
     }
     // publish: the block is read next by TMA (async proxy) on other SMs; the
@@ -452,30 +503,14 @@ __device__ void convert_block(const TsParams &p, const float *v, int64_t blk, __
     }
 }
 
-// Column maxima of |x| over the 128 rows of a slab (x one row per thread) into
-// dst[TS_NPMAX] (one block of the per-slab array).
-__device__ __forceinline__ void slab_max(const float (&x)[TS_NPMAX], int pc, float *smax, int tid, float *dst) {
-    const int wq = tid >> 5, lane = tid & 31;
-#pragma unroll
-    for (int q = 0; q < TS_NPMAX; ++q) {
-        if (q < pc) {
-            float m = fabsf(x[q]);
-            for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-            if (lane == 0) smax[wq * TS_NPMAX + q] = m;
-        }
-    }
-    epi_sync();
-    if (tid < pc)
-        dst[tid] = fmaxf(fmaxf(smax[tid], smax[TS_NPMAX + tid]), fmaxf(smax[2 * TS_NPMAX + tid], smax[3 * TS_NPMAX + tid]));
-}
-
 // Predicted scale of a block from the column maximum m of the block before
 // it in the sweep: puts m in [256, 512).  Blocks of one vector have similar
 // magnitudes, so each slab converts its own rows with this scale as soon as
 // they are final; the block keeps it if its own maximum lands in
 // [PRED_LO, PRED_HI) (about 22 significant bits relative to the maximum, as
-// with the exact scale, and 2x headroom below the FP16 maximum), else the last
+// with the exact scale, and 2x headroom below the FP16 maximum), else its last
 // slab converts the whole block again with the exact scale.
+// (A column of zeros has no maximum to place and takes the exact path too.)
 constexpr float PRED_LO = 8.f, PRED_HI = 32768.f;
 
 __device__ __forceinline__ float pred_scale(float m) {
@@ -485,44 +520,16 @@ __device__ __forceinline__ float pred_scale(float m) {
     return ldexpf(1.f, max(-126, min(126, 9 - e)));
 }
 
-// One row (one element per column, already final) as an FP16 pair with the
-// per-column scales sscale: planes q (hi) and np + q (lo); padding columns zero.
-__device__ __forceinline__ void store_pair_row(const TsParams &p, __half *vb, int64_t grow, const float (&x)[TS_NPMAX],
-                                               const float *sscale) {
-    const int pc = p.pc, np = p.np;
-    const int64_t n_pad = p.n_pad;
-#pragma unroll
-    for (int q = 0; q < TS_NPMAX; ++q) {
-        if (q < np) {
-            const float xs = (q < pc) ? x[q] * sscale[q] : 0.f;
-            const __half hh = __float2half_rn(xs);
-            vb[(int64_t)q * n_pad + grow] = hh;
-            vb[(int64_t)(np + q) * n_pad + grow] = __float2half_rn(xs - __half2float(hh));
-        }
-    }
+// Maxima that predict the scales of a block: the block before it in the sweep
+// (the right-hand side's own block for the first solution block).
+__device__ __forceinline__ const float *pred_from(const TsParams &p, bool out, int64_t blk) {
+    const bool fwd = (p.job == TS_FWD);
+    const int64_t prev = fwd ? blk - 1 : blk + 1;
+    const bool first = fwd ? (blk == 0) : (blk == p.nt - 1);
+    return !out ? p.bm_in + prev * TS_NPMAX : first ? p.bm_in + blk * TS_NPMAX : p.bm_out + prev * TS_NPMAX;
 }
 
-// Last slab of a block (128 epilogue threads): block column maxima from the
-// slab maxima into bmax; true (for every thread) if the predicted scales in
-// sscale hold for every column, and then they become the block's scales sv.
-__device__ bool accept_block(const TsParams &p, const float *slabmax, int64_t blk, const float *sscale, float *sv,
-                             float *bmax, int *sflag, int tid) {
-    if (tid == 0) sflag[3] = 1;
-    epi_sync();
-    if (tid < p.pc) {
-        float m = 0.f;
-        for (int64_t sl = 0; sl < p.S; ++sl) m = fmaxf(m, __ldcg(slabmax + (blk * p.S + sl) * TS_NPMAX + tid));
-        bmax[blk * TS_NPMAX + tid] = m;
-        const float ms = m * sscale[tid];
-        if (!(m == 0.f || (ms >= PRED_LO && ms < PRED_HI))) sflag[3] = 0;
-    }
-    epi_sync();
-    const bool ok = sflag[3] != 0;
-    if (ok && tid < p.np) sv[blk * p.np + tid] = sscale[tid];
-    epi_sync();
-    return ok;
-}
-
+template <int NP>
 __global__ void __launch_bounds__(TS_THREADS, 1)
     tcsweep_kernel(const __grid_constant__ CUtensorMap mPool, const __grid_constant__ CUtensorMap mWsh,
                    const __grid_constant__ CUtensorMap mLhi, const __grid_constant__ CUtensorMap mLlo,
@@ -530,23 +537,28 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
                    const TsParams p) {
     extern __shared__ __align__(1024) uint8_t ts_smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(ts_smem_raw) + 1023) & ~uintptr_t(1023));
-    const int NS = p.stages, SB = p.stage_bytes;
-    ItemHdr *hdrs = reinterpret_cast<ItemHdr *>(smem + NS * SB);
+    const int NS = p.stages;
+    uint8_t *bbuf = smem + NS * TS_ABYTES;
+    ItemHdr *hdrs = reinterpret_cast<ItemHdr *>(bbuf + p.bseg * 2 * NP * 128);
     float *smax = reinterpret_cast<float *>(hdrs + TS_IRING);    // [4][TS_NPMAX]
     float *sscale = smax + 4 * TS_NPMAX;                          // [TS_NPMAX]
     float *smul = sscale + TS_NPMAX;                              // [TS_NPMAX]
-    int *sflag = reinterpret_cast<int *>(smul + TS_NPMAX);        // [4]
+    int *sexact = reinterpret_cast<int *>(smul + TS_NPMAX);       // [TS_IRING] the block read has exact scales
+    int *sflag = sexact + TS_IRING;                               // [4]
     uint64_t *bars = reinterpret_cast<uint64_t *>(sflag + 4);
     uint64_t *full = bars, *empty = bars + NS, *tfull = bars + 2 * NS, *tempty = bars + 2 * NS + 2,
              *ifull = bars + 2 * NS + 4, *iempty = bars + 2 * NS + 4 + TS_IRING,
-             *drain = bars + 2 * NS + 4 + 2 * TS_IRING;
+             *sfull = bars + 2 * NS + 4 + 2 * TS_IRING, *bfull = bars + 2 * NS + 4 + 3 * TS_IRING, *bempty = bfull + 1,
+             *drain = bfull + 2;
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(drain + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int np = p.np;
-    // two accumulators of 2 np columns: products with the hi half of B, then
-    // with the lo half (one MMA of N = 2 np per K step reads A once)
-    const uint32_t tcols = (np * 4 <= 32) ? 32u : (np * 4 <= 64 ? 64u : (np * 4 <= 128 ? 128u : 256u));
+    // two accumulators of four partial sums of 2 np columns: products with the
+    // hi half of B, then with the lo half (one MMA of N = 2 np per K step reads
+    // A once).  The four K steps of a chunk go to different partial sums: FP32
+    // sums a quarter as long (the substitution's error at b = 2048: 2.5e-6
+    // against 8.6e-6 with one) at no cost.
+    constexpr uint32_t ACC = 2 * NP, TCOLS = 8 * ACC;
     if (threadIdx.x == 0) {
         for (int s = 0; s < NS; ++s) {
             mbar_init(&full[s], 1);
@@ -559,14 +571,17 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
         for (int q = 0; q < TS_IRING; ++q) {
             mbar_init(&ifull[q], 1);
             mbar_init(&iempty[q], TS_EPI / 32 + 1);  // epilogue warps and the MMA thread
+            mbar_init(&sfull[q], 1);
         }
+        mbar_init(bfull, 1);
+        mbar_init(bempty, 1);
         mbar_init(drain, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
-                     "r"(tcols)
+                     "r"(TCOLS)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
@@ -583,137 +598,187 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
     tmem_fence_after();
     const uint32_t tmem_base = *tmem_slot;
     const bool fwd = (p.job == TS_FWD);
-    const uint32_t bbytes = (uint32_t)(2 * np * 128);
     const int KC = (int)p.KC;
+    // an item's chunks, and after how many of them the next part of B is due:
+    // a block of up to TS_BSEG groups is loaded once for all phases
+    auto b_period = [&](int nch) { return p.bseg == KC ? nch : p.bseg; };
 
     if (warp == 0) {
-        if (lane == 0) {
-            // ------------------------------ producer ------------------------------
-            const CUtensorMap *amaps[4] = {&mPool, &mWsh, &mLhi, &mLlo};
-            int s = 0;
-            uint32_t ph = 0;
-            int slot = 0;
-            uint32_t sph = 0;
-            int issued = 0;
-            bool ok = true;
-            // A chunk c of the item (phase c / KC, K chunk c % KC) into stage st
-            auto load_a = [&](const ItemHdr &h, int c, uint8_t *st, uint64_t *bar) {
-                const int q = c / KC, kc = c % KC;
-                const CUtensorMap *m = amaps[h.amap[q]];
-                if (fwd) {
-                    tma_load_2d(st, m, kc * TS_KC, h.arow[q] + h.slab * TS_SLAB, bar);
-                } else {
-                    const int y = h.arow[q] + kc * TS_KC;
-                    tma_load_2d(st, m, h.slab * TS_SLAB, y, bar);
-                    tma_load_2d(st + TS_ABYTES / 2, m, h.slab * TS_SLAB + 64, y, bar);
+        // ------------------------------ producer ------------------------------
+        const CUtensorMap *amaps[4] = {&mPool, &mWsh, &mLhi, &mLlo};
+        int s = 0;
+        uint32_t ph = 0;
+        int slot = 0;
+        uint32_t sph = 0;
+        int issued = 0;
+        bool ok = true;
+        // A chunk c of the item (phase c / KC, K chunk c % KC) into the next stage
+        auto load_a = [&](const ItemHdr &h, int c) -> bool {
+            if (!wait_bar(&empty[s], ph ^ 1, p)) return false;
+            uint8_t *st = smem + s * TS_ABYTES;
+            const int q = c >> p.lkc, kc = c & (KC - 1);
+            const CUtensorMap *m = amaps[q ? h.amap[1] : h.amap[0]];
+            const int row = q ? h.arow[1] : h.arow[0];
+            mbar_arrive_expect_tx(&full[s], (uint32_t)TS_ABYTES);
+            if (fwd) {
+                tma_load_2d(st, m, kc * TS_KC, row + h.slab * TS_SLAB, &full[s]);
+            } else {
+                const int y = row + kc * TS_KC;
+                tma_load_2d(st, m, h.slab * TS_SLAB, y, &full[s]);
+                tma_load_2d(st + TS_ABYTES / 2, m, h.slab * TS_SLAB + 64, y, &full[s]);
+            }
+            ++issued;
+            if (++s == NS) { s = 0; ph ^= 1; }
+            return true;
+        };
+        // groups [g0, g0 + bseg) of the vector block that the item reads
+        auto load_b = [&](const ItemHdr &h, int g0, uint64_t *bar) {
+            const CUtensorMap *m = (h.type == IT_DIAG) ? &mVin : &mVout;
+            const int rows = p.bseg * 2 * NP, y = (h.src * KC + g0) * 2 * NP;
+            mbar_arrive_expect_tx(bar, (uint32_t)rows * 128);
+            for (int r = 0; r < rows; r += TS_BBOX) tma_load_2d(bbuf + r * 128, m, 0, y + r, bar);
+        };
+        uint32_t bph = 0;  // phase of the B buffer
+        int nb = 0;        // loads of B issued
+        int t = (lane == 0) ? atomicAdd(&p.flags[0], 1) : 0;
+        while (ok) {
+            t = __shfl_sync(0xffffffffu, t, 0);
+            ItemHdr h;
+            if (t >= p.items) {
+                memset(&h, 0, sizeof(h));
+                h.type = IT_END;
+            } else {
+                decode_item(p, t, h);
+            }
+            if (lane == 0) {
+                ok = wait_bar(&iempty[slot], sph ^ 1, p);
+                if (ok) {
+                    hdrs[slot] = h;
+                    mbar_arrive(&ifull[slot]);
                 }
-            };
-            auto load_b = [&](const ItemHdr &h, int c, uint8_t *st, uint64_t *bar) {
-                const int kc = c % KC;
-                const CUtensorMap *m = (h.type == IT_DIAG) ? &mVin : &mVout;
-                tma_load_2d(st + TS_ABYTES, m, (int)(h.src * p.b) + kc * TS_KC, 0, bar);
-            };
-            while (ok) {
-                int64_t t = atomicAdd(&p.flags[0], 1);
-                ItemHdr h;
-                if (t >= p.items) {
-                    memset(&h, 0, sizeof(h));
-                    h.type = IT_END;
-                } else {
-                    decode_item(p, t, h);
-                }
-                if (!wait_bar(&iempty[slot], sph ^ 1, p)) { ok = false; break; }
-                hdrs[slot] = h;
-                mbar_arrive(&ifull[slot]);
-                if (++slot == TS_IRING) { slot = 0; sph ^= 1; }
-                if (h.type == IT_END) break;
-                if (h.type == IT_CONV) continue;
-                const int nch = h.nph * KC;
-                // the first stages' A loads go out before the dependency wait
+            }
+            ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
+            if (!ok || h.type == IT_END) break;
+            if (lane == 0) t = atomicAdd(&p.flags[0], 1);  // the next item, while this one is loaded
+            if (h.type != IT_CONV) {
+                const int nch = h.nph * KC, bper = b_period(nch);
                 const int npre = min(NS, nch);
-                int pst[8];
-                for (int c = 0; c < npre && ok; ++c) {
-                    if (!wait_bar(&empty[s], ph ^ 1, p)) { ok = false; break; }
-                    uint8_t *st = smem + s * SB;
-                    mbar_arrive_expect_tx(&full[s], (uint32_t)TS_ABYTES + bbytes);
-                    load_a(h, c, st, &full[s]);
-                    pst[c] = s;
-                    ++issued;
-                    if (++s == NS) { s = 0; ph ^= 1; }
+                const bool diag = (h.type == IT_DIAG);
+                if (lane == 0) {
+                    // the first stages' A loads go out before the dependency wait
+                    for (int c = 0; c < npre && ok; ++c) ok = load_a(h, c);
+                    unsigned long long st = 0;
+                    ok = ok && wait_state((diag ? p.st_in : p.st_out) + h.src, (int)p.S, &st, p) &&
+                         wait_bar(bempty, bph ^ 1, p);
+                    // the first right-hand side block has exact scales
+                    bool exact = diag && h.src == (fwd ? 0 : (int)p.nt - 1);
+                    if (ok && !exact && !state_holds(st, p.pc)) {
+                        // the predicted scales do not hold: the block is being converted as a whole
+                        exact = true;
+                        ok = wait_count((diag ? xin_ctr(p) : xout_ctr(p)) + h.src, 1, p);
+                    }
+                    if (ok) {
+                        fence_proxy_async_global();
+                        load_b(h, 0, bfull);
+                        ++nb;
+                        bph ^= 1;
+                        sexact[slot] = exact ? 1 : 0;
+                        mbar_arrive(&sfull[slot]);
+                    }
+                    for (int c = npre; c < nch && ok; ++c) {
+                        if ((c & (bper - 1)) == 0) {  // the next part of B (bper is a power of two)
+                            ok = wait_bar(bempty, bph ^ 1, p);
+                            if (!ok) break;
+                            load_b(h, c & (KC - 1), bfull);
+                            ++nb;
+                            bph ^= 1;
+                        }
+                        ok = load_a(h, c);
+                    }
                 }
-                if (!ok) break;
-                const int *dep = (h.type == IT_DIAG) ? done_ctr(p) + h.blk : ready_ctr(p) + h.src;
-                ok = wait_count(dep, 1, p);
-                fence_proxy_async_global();
-                // (after an abort too, so every issued stage completes and can be drained)
-                for (int c = 0; c < npre; ++c) load_b(h, c, smem + pst[c] * SB, &full[pst[c]]);
-                for (int c = npre; c < nch && ok; ++c) {
-                    if (!wait_bar(&empty[s], ph ^ 1, p)) { ok = false; break; }
-                    uint8_t *st = smem + s * SB;
-                    mbar_arrive_expect_tx(&full[s], (uint32_t)TS_ABYTES + bbytes);
-                    load_a(h, c, st, &full[s]);
-                    load_b(h, c, st, &full[s]);
-                    ++issued;
-                    if (++s == NS) { s = 0; ph ^= 1; }
-                }
+                ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
             }
-            if (!ok) {
-                // drain: wait (bounded) for the loads of the last stages to land
-                const int n = issued < NS ? issued : NS;
-                int ss = s;
-                uint32_t pp = ph;
-                for (int e = 0; e < n; ++e) {
-                    if (--ss < 0) { ss = NS - 1; pp ^= 1; }
-                    const uint64_t t0 = globaltimer();
-                    while (!mbar_try_wait(&full[ss], pp) && globaltimer() - t0 < drain_limit(p.wait_ns)) {}
-                }
+            if (++slot == TS_IRING) { slot = 0; sph ^= 1; }
+        }
+        if (!ok && lane == 0) {
+            // drain: wait (bounded) for the loads of the last stages to land
+            const int n = issued < NS ? issued : NS;
+            int ss = s;
+            uint32_t pp = ph;
+            for (int e = 0; e < n; ++e) {
+                if (--ss < 0) { ss = NS - 1; pp ^= 1; }
+                const uint64_t t0 = globaltimer();
+                while (!mbar_try_wait(&full[ss], pp) && globaltimer() - t0 < drain_limit(p.wait_ns)) {}
             }
+            const uint64_t t0 = globaltimer();
+            while (nb > 0 && !mbar_try_wait(bfull, (uint32_t)(nb - 1) & 1) && globaltimer() - t0 < drain_limit(p.wait_ns)) {}
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            // ------------------------------ MMA issuer ------------------------------
-            int s = 0;
-            uint32_t ph = 0;
-            int slot = 0;
-            uint32_t sph = 0;
-            int acc = 0;
-            uint32_t aph = 0;
-            bool ok = true, any = false;
-            while (ok) {
-                if (!wait_bar(&ifull[slot], sph, p)) { ok = false; break; }
-                const ItemHdr h = hdrs[slot];
-                mbar_arrive(&iempty[slot]);
-                if (++slot == TS_IRING) { slot = 0; sph ^= 1; }
-                if (h.type == IT_END) break;
-                if (h.type == IT_CONV) continue;
-                if (!wait_bar(&tempty[acc], aph ^ 1, p)) { ok = false; break; }
-                tmem_fence_after();
-                const uint32_t tacc = tmem_base + (uint32_t)(acc * 2 * np);
-                const int nch = h.nph * KC;
-                for (int c = 0; c < nch; ++c) {
-                    if (!wait_bar(&full[s], ph, p)) { ok = false; break; }
+        // ------------------------------ MMA issuer ------------------------------
+        // The whole warp runs the loop and one lane issues: the descriptors are
+        // then computed in uniform registers, where the instruction reads them.
+        int s = 0;
+        uint32_t ph = 0, bph = 0;
+        int slot = 0;
+        uint32_t sph = 0;
+        int acc = 0;
+        uint32_t aph = 0;
+        bool ok = true, any = false;
+        const bool issuer = elect_one();
+        auto wwait = [&](uint64_t *bar, uint32_t parity) { return __all_sync(0xffffffffu, wait_bar(bar, parity, p)) != 0; };
+        // K steps of 16: 32 bytes of a K-major row, 16 rows of an MN-major one
+        const uint64_t ad0 = fwd ? desc_kmajor(smem_u32(smem)) : desc_mnmajor(smem_u32(smem));
+        const uint64_t bd0 = desc_kmajor(smem_u32(bbuf));
+        const uint32_t astep = fwd ? 32 >> 4 : 2048 >> 4;
+        while (ok) {
+            if (!wwait(&ifull[slot], sph)) { ok = false; break; }
+            const int type = __shfl_sync(0xffffffffu, hdrs[slot].type, 0);
+            const int nch = __shfl_sync(0xffffffffu, hdrs[slot].nph, 0) * KC;
+            if (issuer) mbar_arrive(&iempty[slot]);
+            if (++slot == TS_IRING) { slot = 0; sph ^= 1; }
+            if (type == IT_END) break;
+            if (type == IT_CONV) continue;
+            if (!wwait(&tempty[acc], aph ^ 1)) { ok = false; break; }
+            tmem_fence_after();
+            const uint32_t tacc = tmem_base + (uint32_t)acc * 4 * ACC;
+            const int bper = b_period(nch);
+            for (int c0 = 0; c0 < nch && ok; c0 += bper) {
+                if (!wwait(bfull, bph)) { ok = false; break; }
+                bph ^= 1;
+                // a stage's barrier is tested while the MMAs of the stage before
+                // it are issued: a wait in series costs as much as the four MMAs
+                bool landed = mbar_try_wait(&full[s], ph);
+                for (int c = c0; c < c0 + bper; ++c) {
+                    if (!__all_sync(0xffffffffu, landed) && !wwait(&full[s], ph)) { ok = false; break; }
                     tmem_fence_after();
-                    const uint32_t sa = smem_u32(smem + s * SB), sb = sa + TS_ABYTES;
+                    const int sn = (s + 1 == NS) ? 0 : s + 1;
+                    const uint32_t pn = (sn == 0) ? ph ^ 1 : ph;
+                    landed = c + 1 < c0 + bper && mbar_try_wait(&full[sn], pn);
+                    const uint64_t ad = ad0 + (uint32_t)(s * (TS_ABYTES >> 4));
+                    const uint64_t bd = bd0 + (uint32_t)((c & (p.bseg - 1)) * (2 * NP * 128 >> 4));
+                    if (issuer) {
 #pragma unroll
-                    for (int kk = 0; kk < 4; ++kk) {
-                        const uint64_t ad = fwd ? desc_kmajor(sa + kk * 32) : desc_mnmajor(sa + kk * 2048);
-                        // B rows [0, np) = hi half, [np, 2 np) = lo half
-                        mma_f16(tacc, ad, desc_kmajor(sb + kk * 32), p.idesc, (c > 0 || kk > 0) ? 1u : 0u);
+                        for (int kk = 0; kk < 4; ++kk)
+                            // B rows [0, np) = hi half, [np, 2 np) = lo half
+                            mma_f16(tacc + kk * ACC, ad + kk * astep, bd + kk * 2, p.idesc, c > 0 ? 1u : 0u);
+                        mma_commit(&empty[s]);
+                        if (c + 1 == c0 + bper) mma_commit(bempty);  // this part of B is read
+                        if (c + 1 == nch) mma_commit(&tfull[acc]);
                     }
                     any = true;
-                    mma_commit(&empty[s]);
-                    if (++s == NS) { s = 0; ph ^= 1; }
+                    s = sn;
+                    ph = pn;
                 }
-                if (!ok) break;
-                mma_commit(&tfull[acc]);
-                if (++acc == 2) { acc = 0; aph ^= 1; }
             }
-            if (!ok && any) {
-                mma_commit(drain);
-                const uint64_t t0 = globaltimer();
-                while (!mbar_try_wait(drain, 0) && globaltimer() - t0 < drain_limit(p.wait_ns)) {}
-            }
+            if (!ok) break;
+            if (++acc == 2) { acc = 0; aph ^= 1; }
         }
+        if (!ok && any && issuer) {
+            mma_commit(drain);
+            const uint64_t t0 = globaltimer();
+            while (!mbar_try_wait(drain, 0) && globaltimer() - t0 < drain_limit(p.wait_ns)) {}
+        }
+        __syncwarp();
     } else {
         // ------------------------------ epilogue ------------------------------
         const int tid = threadIdx.x - 64;
@@ -723,7 +788,7 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
         int acc = 0;
         uint32_t aph = 0;
         const int pc = p.pc;
-        const int64_t b = p.b, S = p.S;
+        const int64_t b = p.b, S = p.S, cs = p.cs;
         // one thread waits, the group follows its decision
         auto group_wait_bar = [&](uint64_t *bar, uint32_t parity) -> bool {
             if (tid == 0) sflag[0] = wait_bar(bar, parity, p) ? 1 : 0;
@@ -732,138 +797,124 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
             epi_sync();
             return r;
         };
+        uint32_t sfph = 0;  // bit i: phase of sfull[i]
         while (true) {
             if (!group_wait_bar(&ifull[slot], sph)) break;
             const ItemHdr h = hdrs[slot];
+            const int hslot = slot;
             epi_sync();
-            if (lane == 0) mbar_arrive(&iempty[slot]);
             if (++slot == TS_IRING) { slot = 0; sph ^= 1; }
             if (h.type == IT_END) break;
             if (h.type == IT_CONV) {
-                convert_block(p, p.rhs, h.blk, p.vin, p.sin, smax, sscale, tid, nullptr, p.bm_in);
-                if (tid == 0) st_release(done_ctr(p) + h.blk, 1);
+                if (lane == 0) mbar_arrive(&iempty[hslot]);
+                convert_block(p, p.rhs, h.blk, p.vin, p.sin, smax, sscale, tid, true, p.bm_in);
+                if (tid == 0) {
+                    __threadfence();
+                    atomicAdd(p.st_in + h.blk, (unsigned long long)S);
+                }
                 continue;
             }
+            const bool link = (h.type == IT_LINK), fin = !link || h.last_link;
             const int64_t grow = (int64_t)h.blk * b + (int64_t)h.slab * TS_SLAB + row;
-            // LINK: once the earlier updates of this slab are in, load the rows
-            // to update before waiting for the accumulator (the L2 round trip
-            // overlaps the MMAs)
-            float yv[TS_NPMAX];
-            float *y = p.rhs + grow * p.rs + p.q0 * p.cs;
+            // before waiting for the accumulator: the rows to update, once the
+            // earlier updates of this slab are in, and the scales
+            float yv[NP];
+            float *y = (link ? p.rhs : p.out) + grow * p.rs + p.q0 * cs;
             int *sq = seq_ctr(p) + (int64_t)h.blk * S + h.slab;
-            if (h.type == IT_LINK) {
-                if (tid == 0) sflag[2] = wait_count(sq, h.seqv, p) ? 1 : 0;
-                epi_sync();
-                if (!sflag[2]) break;
-                const float *yp = y;
+            if (tid == 0)
+                sflag[2] = ((!link || wait_count(sq, h.seqv, p)) && wait_bar(&sfull[hslot], (sfph >> hslot) & 1, p)) ? 1 : 0;
+            sfph ^= 1u << hslot;
+            epi_sync();
+            if (!sflag[2]) break;
 #pragma unroll
-                for (int q = 0; q < TS_NPMAX; ++q) {
-                    if (q < pc) {
-                        yv[q] = __ldcg(yp);
-                        yp += p.cs;
-                    }
-                }
+            for (int q = 0; q < NP; ++q) yv[q] = (link && q < pc) ? __ldcg(y + q * cs) : 0.f;
+            if (tid < NP) {
+                // column multipliers: 1 / (tile scale * vector block scale)
+                float sc = 1.f;
+                if (sexact[hslot]) sc = __ldcg((link ? p.sout : p.sin) + (int64_t)h.src * NP + tid);
+                else if (tid < pc) sc = pred_scale(__ldcg(pred_from(p, link, h.src) + tid));
+                smul[tid] = h.inv_tscale / sc;
+                if (fin) sscale[tid] = (tid < pc) ? pred_scale(__ldcg(pred_from(p, !link, h.blk) + tid)) : 1.f;
             }
             if (!group_wait_bar(&tfull[acc], aph)) break;
+            if (lane == 0) mbar_arrive(&iempty[hslot]);  // the header and the scales are read
             tmem_fence_after();
-            float v[TS_NPMAX];
-            const uint32_t tacc = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(acc * 2 * np);
+            float v[NP];
+            const uint32_t tacc = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)acc * 4 * ACC;
 #pragma unroll
-            for (int c16 = 0; c16 < TS_NPMAX / 16; ++c16) {
-                if (c16 * 16 < np) {
-                    float hv[16], lv[16];
-                    tmem_ld16(tacc + c16 * 16, hv);
-                    tmem_ld16(tacc + np + c16 * 16, lv);
-#pragma unroll
-                    for (int e = 0; e < 16; ++e) v[c16 * 16 + e] = hv[e] + lv[e];
-                }
-            }
+            for (int c8 = 0; c8 < NP; c8 += 8) tmem_sum8x8(tacc + c8, NP, v + c8);
             tmem_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&tempty[acc]);
             if (++acc == 2) { acc = 0; aph ^= 1; }
-            // column multipliers: 1 / (tile scale * vector block scale)
-            const float *sv = (h.type == IT_DIAG) ? p.sin + (int64_t)h.blk * np : p.sout + (int64_t)h.src * np;
-            if (tid < pc) smul[tid] = h.inv_tscale / __ldcg(sv + tid);
-            // predicted scale of the block this item finishes: from the block
-            // before it in the sweep (the right-hand side's own block for the
-            // first solution block)
-            const int64_t prev = fwd ? (int64_t)h.blk - 1 : (int64_t)h.blk + 1;
-            const bool first = fwd ? (h.blk == 0) : (h.blk == p.nt - 1);
-            if ((h.type == IT_DIAG || h.last_link) && tid < np) {
-                const float *bm = (h.type == IT_LINK) ? p.bm_in + prev * TS_NPMAX
-                                  : first            ? p.bm_in + (int64_t)h.blk * TS_NPMAX
-                                                     : p.bm_out + prev * TS_NPMAX;
-                sscale[tid] = (tid < pc) ? pred_scale(__ldcg(bm + tid)) : 1.f;
+#pragma unroll
+            for (int q = 0; q < NP; q += 4) {
+                const float4 m4 = *reinterpret_cast<const float4 *>(smul + q);
+                v[q] *= m4.x;
+                v[q + 1] *= m4.y;
+                v[q + 2] *= m4.z;
+                v[q + 3] *= m4.w;
             }
-            if (h.type == IT_DIAG) {
-                epi_sync();
-                float *o = p.out + grow * p.rs + p.q0 * p.cs;
-                {
-                    float *op = o;
 #pragma unroll
-                    for (int q = 0; q < TS_NPMAX; ++q) {
-                        if (q < pc) {
-                            v[q] *= smul[q];
-                            __stcg(op, v[q]);
-                            op += p.cs;
-                        }
+            for (int q = 0; q < NP; ++q) {
+                if (link) v[q] = yv[q] - v[q];
+                if (q < pc) __stcg(y + q * cs, v[q]);
+            }
+            if (fin) {
+                // the rows are final: FP16 pair with the predicted scales, and
+                // the column maxima of the slab
+                __half *vb = (link ? p.vin : p.vout) + (grow >> 6) * (2 * NP * 64) + (grow & 63);
+#pragma unroll
+                for (int q = 0; q < NP; q += 4) {
+                    const float4 s4 = *reinterpret_cast<const float4 *>(sscale + q);
+                    const float sq4[4] = {s4.x, s4.y, s4.z, s4.w};
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const float xs = (q + e < pc) ? v[q + e] * sq4[e] : 0.f;
+                        const __half hh = __float2half_rn(xs);
+                        vb[(q + e) * 64] = hh;
+                        vb[(NP + q + e) * 64] = __float2half_rn(xs - __half2float(hh));
                     }
                 }
-                store_pair_row(p, p.vout, grow, v, sscale);
-                slab_max(v, pc, smax, tid, p.mx_out + ((int64_t)h.blk * S + h.slab) * TS_NPMAX);
-                epi_sync();
-                if (tid == 0) {
-                    __threadfence();
-                    fence_proxy_async_global();  // the FP16 rows are read by TMA on other SMs
-                    const bool last = atomicAdd(cout_ctr(p) + h.blk, 1) == (int)S - 1;
-                    if (last) __threadfence();  // the other slabs' rows and maxima are read next
-                    sflag[1] = last ? 1 : 0;
+                uint32_t mine = 0;  // lane q: maximum of column q over the warp's rows
+#pragma unroll
+                for (int q = 0; q < NP; ++q) {
+                    const uint32_t m = __reduce_max_sync(0xffffffffu, __float_as_uint(fabsf(v[q])));
+                    if (lane == q) mine = m;
                 }
+                // the warp's part of the block's maxima and of the test of the scales
+                const float ms = __uint_as_float(mine) * (lane < NP ? sscale[lane] : 0.f);
+                const bool col = lane < pc;
+                const uint32_t ge = __ballot_sync(0xffffffffu, col && ms >= PRED_LO);
+                const uint32_t over = __ballot_sync(0xffffffffu, col && !(ms < PRED_HI));
+                unsigned long long *st = (link ? p.st_in : p.st_out) + h.blk;
+                if (col)
+                    atomicMax(reinterpret_cast<unsigned int *>((link ? p.bm_in : p.bm_out) + (int64_t)h.blk * TS_NPMAX) + lane,
+                              mine);
+                if (lane == 0) {
+                    atomicOr(st, (unsigned long long)ge << 32);
+                    if (over) atomicAdd(st, 1ull << 16);
+                }
+            }
+            epi_sync();
+            if (tid == 0) {
+                __threadfence();
+                if (fin) fence_proxy_async_global();  // the FP16 rows are read by TMA on other SMs
+                if (link) atomicAdd(sq, 1);
+                if (fin) {
+                    // the last slab of the block: if the prediction failed for any
+                    // column, the block is converted again (readers wait for that)
+                    const unsigned long long v = atomicAdd((link ? p.st_in : p.st_out) + h.blk, 1ull);
+                    sflag[1] = (state_slabs(v) == (int)S - 1 && !state_holds(v, pc)) ? 1 : 0;
+                    if (sflag[1]) __threadfence();  // the other slabs' rows and maxima are read next
+                }
+            }
+            if (fin) {
                 epi_sync();
                 if (sflag[1]) {
-                    if (!accept_block(p, p.mx_out, h.blk, sscale, p.sout, p.bm_out, sflag, tid))
-                        convert_block(p, p.out, h.blk, p.vout, p.sout, smax, sscale, tid, p.mx_out, p.bm_out);
-                    if (tid == 0) {
-                        __threadfence();
-                        st_release(ready_ctr(p) + h.blk, 1);
-                    }
-                }
-            } else {
-                // LINK: the rows were loaded before the accumulator wait
-                epi_sync();  // smul
-                {
-                    float *ys = y;
-#pragma unroll
-                    for (int q = 0; q < TS_NPMAX; ++q) {
-                        if (q < pc) {
-                            yv[q] -= v[q] * smul[q];
-                            __stcg(ys, yv[q]);
-                            ys += p.cs;
-                        }
-                    }
-                }
-                if (h.last_link) {
-                    store_pair_row(p, p.vin, grow, yv, sscale);
-                    slab_max(yv, pc, smax, tid, p.mx_in + ((int64_t)h.blk * S + h.slab) * TS_NPMAX);
-                }
-                epi_sync();
-                if (tid == 0) {
-                    __threadfence();
-                    if (h.last_link) fence_proxy_async_global();
-                    atomicAdd(sq, 1);
-                    const bool last = h.last_link && atomicAdd(cin_ctr(p) + h.blk, 1) == (int)S - 1;
-                    if (last) __threadfence();  // the other slabs' rows are read next
-                    sflag[1] = last ? 1 : 0;
-                }
-                epi_sync();
-                if (sflag[1]) {
-                    if (!accept_block(p, p.mx_in, h.blk, sscale, p.sin, p.bm_in, sflag, tid))
-                        convert_block(p, p.rhs, h.blk, p.vin, p.sin, smax, sscale, tid, p.mx_in, p.bm_in);
-                    if (tid == 0) {
-                        __threadfence();
-                        st_release(done_ctr(p) + h.blk, 1);
-                    }
+                    convert_block(p, link ? p.rhs : p.out, h.blk, link ? p.vin : p.vout, link ? p.sin : p.sout, smax,
+                                  sscale, tid, false, link ? p.bm_in : p.bm_out);
+                    if (tid == 0) st_release((link ? xin_ctr(p) : xout_ctr(p)) + h.blk, 1);
                 }
             }
         }
@@ -872,7 +923,7 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
     __syncthreads();
     if (warp == 1) {
         tmem_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(tcols) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TCOLS) : "memory");
     }
 }
 
@@ -1498,16 +1549,17 @@ krr_status map_f16(Ctx *c, CUtensorMap *m, const void *base, int64_t rows, int64
 
 constexpr size_t ts_smem_limit() { return 227 * 1024; }
 
-size_t ts_smem_bytes(int stages, int stage_bytes) {
-    return (size_t)stages * stage_bytes + TS_IRING * sizeof(ItemHdr) + (6 * TS_NPMAX + 4) * 4 +
-           (size_t)(2 * stages + 5 + 2 * TS_IRING) * 8 + 16 + 1024;
+size_t ts_smem_bytes(int stages, int b_bytes) {
+    return (size_t)stages * TS_ABYTES + b_bytes + TS_IRING * sizeof(ItemHdr) + (6 * TS_NPMAX + TS_IRING + 4) * 4 +
+           (size_t)(2 * stages + 7 + 3 * TS_IRING) * 8 + 16 + 1024;
 }
 
-int64_t ts_flag_count(const Ctx *c) { return 2 + 4 * c->nt + c->nt * (c->b / TS_SLAB); }
+int64_t ts_flag_count(const Ctx *c) { return 2 + 2 * c->nt + c->nt * (c->b / TS_SLAB); }
 
 // Auxiliary buffer: block scales of the two FP16 vector buffers ([nt][TS_NPMAX]
 // each), per-slab column maxima of the two ([nt][S][TS_NPMAX] each), their
-// block column maxima ([nt][TS_NPMAX] each), then the progress counters.
+// block column maxima ([nt][TS_NPMAX] each), the states of their blocks ([nt]
+// 64-bit words each), then the progress counters.
 int64_t ts_scale_count(const Ctx *c) { return c->nt * TS_NPMAX; }
 int64_t ts_max_count(const Ctx *c) { return c->nt * (c->b / TS_SLAB) * TS_NPMAX; }
 
@@ -1527,7 +1579,7 @@ krr_status ensure_ts_buffers(Ctx *c, int64_t p) {
         c->ts_vcap = vbytes;
     }
     const size_t abytes = (size_t)(4 * ts_scale_count(c) + 2 * ts_max_count(c)) * sizeof(float) +
-                          (size_t)ts_flag_count(c) * sizeof(int);
+                          (size_t)2 * c->nt * sizeof(unsigned long long) + (size_t)ts_flag_count(c) * sizeof(int);
     if (c->ts_aux_cap < abytes) {
         if (c->ts_aux) cudaFree(c->ts_aux);
         c->ts_aux = nullptr;
@@ -1557,7 +1609,8 @@ krr_status ensure_ts_buffers(Ctx *c, int64_t p) {
 float *ts_scales(Ctx *c) { return (float *)c->ts_aux; }
 float *ts_maxima(Ctx *c) { return ts_scales(c) + 2 * ts_scale_count(c); }
 float *ts_block_maxima(Ctx *c) { return ts_maxima(c) + 2 * ts_max_count(c); }
-int *ts_flags(Ctx *c) { return (int *)(ts_block_maxima(c) + 2 * ts_scale_count(c)); }
+unsigned long long *ts_states(Ctx *c) { return (unsigned long long *)(ts_block_maxima(c) + 2 * ts_scale_count(c)); }
+int *ts_flags(Ctx *c) { return (int *)(ts_states(c) + 2 * c->nt); }
 
 // dst (cols x rows, row-major) = src^T, src rows x cols row-major; with sum,
 // also sum += src^T.
@@ -1604,12 +1657,10 @@ krr_status run_ts(Ctx *c, int job, float *rhs, float *out, int64_t p) {
     int *flags = ts_flags(c);
     static PerDevice attr;
     if (!attr.has(c->device)) {
-        const cudaError_t e =
-            cudaFuncSetAttribute(tcsweep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ts_smem_limit());
-        if (e != cudaSuccess) {
-            c->last_error = std::string("cudaFuncSetAttribute (tensor-core sweep): ") + cudaGetErrorString(e);
-            return KRR_ECUDA;
-        }
+        KRR_CUDA_TRY(c, cudaFuncSetAttribute(tcsweep_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)ts_smem_limit()));
+        KRR_CUDA_TRY(c, cudaFuncSetAttribute(tcsweep_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)ts_smem_limit()));
         attr.put(c->device);
     }
     for (int64_t q0 = 0; q0 < p; q0 += TS_NPMAX) {
@@ -1631,8 +1682,6 @@ krr_status run_ts(Ctx *c, int job, float *rhs, float *out, int64_t p) {
         sp.cs = c->n_pad;
         sp.rhs = rhs;
         sp.out = out;
-        sp.mx_in = ts_maxima(c);
-        sp.mx_out = ts_maxima(c) + ts_max_count(c);
         sp.bm_in = ts_block_maxima(c);
         sp.bm_out = ts_block_maxima(c) + ts_scale_count(c);
         sp.vin = c->ts_v0;
@@ -1640,10 +1689,17 @@ krr_status run_ts(Ctx *c, int job, float *rhs, float *out, int64_t p) {
         sp.sin = sbase;
         sp.sout = sbase + ts_scale_count(c);
         sp.ltab = c->ltab;
+        sp.st_in = ts_states(c);
+        sp.st_out = ts_states(c) + nt;
         sp.flags = flags;
-        sp.stage_bytes = TS_ABYTES + 2 * sp.np * 128;
-        int stages = 8;
-        while (stages > 2 && ts_smem_bytes(stages, sp.stage_bytes) > ts_smem_limit()) --stages;
+        // B takes up to 64 KB (128 KB above 16 columns), A stages the rest: 9
+        // (5) of them; more would cross a part of B
+        sp.lkc = 0;
+        while ((1 << sp.lkc) < sp.KC) ++sp.lkc;
+        sp.bseg = (int)std::min<int64_t>(sp.KC, TS_BSEG);
+        const int b_bytes = sp.bseg * 2 * sp.np * 128;
+        int stages = 12;
+        while (stages > 2 && ts_smem_bytes(stages, b_bytes) > ts_smem_limit()) --stages;
         sp.stages = stages;
         // kind::f16, D = F32, A = B = F16, A K-major (forward) or MN-major
         // (backward), B K-major, N = 2 np (hi and lo halves), M = 128
@@ -1651,12 +1707,20 @@ krr_status run_ts(Ctx *c, int job, float *rhs, float *out, int64_t p) {
                    ((uint32_t)(TS_SLAB >> 4) << 24);
         sp.wait_ns = (uint64_t)c->opt.wait_budget_ns;
         sp.err = c->derr;
-        KRR_TRY(map_f16(c, &mvi, c->ts_v0, 2 * sp.np, c->n_pad, 2 * sp.np));
-        KRR_TRY(map_f16(c, &mvo, c->ts_v1, 2 * sp.np, c->n_pad, 2 * sp.np));
-        KRR_CUDA_TRY(c, cudaMemsetAsync(flags, 0, (size_t)ts_flag_count(c) * sizeof(int), c->stream));
-        const size_t smem = ts_smem_bytes(stages, sp.stage_bytes);
+        const int64_t vrows = c->n_pad / 64 * 2 * sp.np;
+        const int vbox = std::min(TS_BBOX, sp.bseg * 2 * sp.np);
+        KRR_TRY(map_f16(c, &mvi, c->ts_v0, vrows, 64, vbox));
+        KRR_TRY(map_f16(c, &mvo, c->ts_v1, vrows, 64, vbox));
+        // the block maxima and the states and counters behind them
+        KRR_CUDA_TRY(c, cudaMemsetAsync(ts_block_maxima(c), 0,
+                                        (size_t)2 * ts_scale_count(c) * sizeof(float) +
+                                            (size_t)2 * nt * sizeof(unsigned long long) +
+                                            (size_t)ts_flag_count(c) * sizeof(int),
+                                        c->stream));
+        const size_t smem = ts_smem_bytes(stages, b_bytes);
         const int64_t grid = std::min<int64_t>(sp.items, grid_limit(c, GL_SWEEP));
-        count_launch(), tcsweep_kernel<<<(unsigned)grid, TS_THREADS, smem, c->stream>>>(mp, mw, mlh, mll, mvi, mvo, sp);
+        const auto kernel = (sp.np == 16) ? tcsweep_kernel<16> : tcsweep_kernel<32>;
+        count_launch(), kernel<<<(unsigned)grid, TS_THREADS, smem, c->stream>>>(mp, mw, mlh, mll, mvi, mvo, sp);
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) {
             c->last_error = std::string("tensor-core sweep launch: ") + cudaGetErrorString(e);

@@ -945,11 +945,12 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
 // slabs than SMs.  With
 // one item per slab over all tiles, one epilogue group and the tiles read
 // twice from HBM a residual took 1.27 ms at N = 32768 and 10 columns, 11.3 ms
-// at N = 98304 and 20, 0.16 ms at N = 5000 and 2; now 0.88, 8.5 and 0.06 ms.
+// at N = 98304 and 20, 0.16 ms at N = 5000 and 2; now 0.80, 7.8 and 0.056 ms
+// (0.88 and 8.5 with one group of converter warps).
 //   warp 0       producer: TMA of the FP32 K chunk (128 x 64 rows x columns, or
 //                64 x 128 for a column slab) and of the FP16 terms of a_j (B);
-//   warps 6..9   converters: (K - c) 2^12 -> FP16 pair (hi, lo), written in
-//                place over the staged FP32 chunk (each thread overwrites only
+//   warps 6..9 and 14..17  converters, each group every other chunk: (K - c)
+//                2^12 -> FP16 pair (hi, lo), written in place over the staged FP32 chunk (each thread overwrites only
 //                the bytes its own warp read) in the MMA's K-major or MN-major
 //                128-byte-swizzled layout, so the staging ring is also the
 //                operand ring;
@@ -966,7 +967,7 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
 // FP32 accumulation: the residual keeps FP32 accuracy.
 // Every wait is bounded and ends the kernel with KRR_ETIMEOUT.
 // ---------------------------------------------------------------------------
-constexpr int RS_THREADS = 448;
+constexpr int RS_THREADS = 576;
 constexpr int RS_STG = 32768;      // FP32 chunk: 128 x 64 or 64 x 128
 constexpr int RS_NSTG = 5;         // stages (FP32 K chunk by TMA, converted in place, and the terms of a)
 constexpr int RS_NACC = 4;         // TMEM accumulators of 3 np columns
@@ -1092,7 +1093,7 @@ __global__ void __launch_bounds__(RS_THREADS, 1)
         }
         for (int q = 0; q < TS_IRING; ++q) {
             mbar_init(&ifull[q], 1);
-            mbar_init(&iempty[q], 8 + 4 + 1);  // epilogue, converter warps, MMA thread
+            mbar_init(&iempty[q], 8 + 8 + 1);  // epilogue, converter warps, MMA warp
         }
         mbar_init(drain, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -1170,57 +1171,70 @@ __global__ void __launch_bounds__(RS_THREADS, 1)
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            // ------------------------------ MMA issuer ------------------------------
-            int ss = 0, slot = 0, acc = 0;
-            uint32_t sph = 0, iph = 0, aph = 0;
-            bool ok = true, any = false;
-            while (ok) {
-                if (!rs_wait(&ifull[slot], iph, p)) { ok = false; break; }
-                const int t = items[slot];
-                mbar_arrive(&iempty[slot]);
-                if (++slot == TS_IRING) { slot = 0; iph ^= 1; }
-                if (t < 0) break;
-                RsItem it;
-                rs_decode(p, t, it);
-                for (int j = it.j0; j < it.j1 && ok; ++j) {
-                    const bool kmaj = (j <= it.i);
-                    for (int kc = it.kc0; kc < it.kc1; ++kc) {
-                        // one accumulation per 64-wide chunk: the FP32 sums in TMEM stay short
-                        if (!rs_wait(&tempty[acc], aph ^ 1, p)) { ok = false; break; }
-                        const uint32_t tacc = tmem_base + (uint32_t)(acc * 3 * NP);
-                        if (!rs_wait(&sfull[ss], sph, p)) { ok = false; break; }
-                        if (!rs_wait(&cfull[ss], sph, p)) { ok = false; break; }
-                        tmem_fence_after();
-                        const uint32_t sa = smem_u32(smem + ss * SB), sb = sa + RS_STG;
+        // ------------------------------ MMA issuer ------------------------------
+        // (the warp runs the loop, one lane issues, as in the sweeps)
+        int ss = 0, slot = 0, acc = 0;
+        uint32_t sph = 0, iph = 0, aph = 0;
+        bool ok = true, any = false;
+        const bool issuer = elect_one();
+        auto wwait = [&](uint64_t *bar, uint32_t parity) { return __all_sync(0xffffffffu, rs_wait(bar, parity, p)) != 0; };
+        const uint64_t kd0 = desc_kmajor(smem_u32(smem)), md0 = desc_mnmajor(smem_u32(smem)),
+                       bd0 = desc_kmajor(smem_u32(smem + RS_STG));
+        while (ok) {
+            if (!wwait(&ifull[slot], iph)) { ok = false; break; }
+            const int t = __shfl_sync(0xffffffffu, items[slot], 0);
+            if (issuer) mbar_arrive(&iempty[slot]);
+            if (++slot == TS_IRING) { slot = 0; iph ^= 1; }
+            if (t < 0) break;
+            RsItem it;
+            rs_decode(p, t, it);
+            bool ready = false;  // the chunk's barriers, tested while the MMAs before it are issued
+            for (int j = it.j0; j < it.j1 && ok; ++j) {
+                const bool kmaj = (j <= it.i);
+                const uint64_t ad0 = kmaj ? kd0 : md0;
+                const uint32_t astep = kmaj ? 32 >> 4 : 2048 >> 4;
+                const uint32_t id3 = kmaj ? p.idesc_k : p.idesc_mn, id2 = kmaj ? p.idesc_k2 : p.idesc_mn2;
+                for (int kc = it.kc0; kc < it.kc1; ++kc) {
+                    // one accumulation per 64-wide chunk: the FP32 sums in TMEM stay short
+                    if (!__all_sync(0xffffffffu, ready) &&
+                        !(wwait(&tempty[acc], aph ^ 1) && wwait(&sfull[ss], sph) && wwait(&cfull[ss], sph))) {
+                        ok = false;
+                        break;
+                    }
+                    tmem_fence_after();
+                    const int sn = (ss + 1 == RS_NSTG) ? 0 : ss + 1, an = (acc + 1 == RS_NACC) ? 0 : acc + 1;
+                    const uint32_t spn = (sn == 0) ? sph ^ 1 : sph, apn = (an == 0) ? aph ^ 1 : aph;
+                    ready = (j + 1 < it.j1 || kc + 1 < it.kc1) && mbar_try_wait(&cfull[sn], spn) &&
+                            mbar_try_wait(&sfull[sn], spn) && mbar_try_wait(&tempty[an], apn ^ 1);
+                    const uint32_t tacc = tmem_base + (uint32_t)(acc * 3 * NP);
+                    const uint32_t so = (uint32_t)(ss * (SB >> 4));
+                    if (issuer) {
 #pragma unroll
                         for (int kk = 0; kk < 4; ++kk) {
-                            const uint64_t bd = desc_kmajor(sb + kk * 32);
-                            if (kmaj) {
-                                mma_f16(tacc, desc_kmajor(sa + kk * 32), bd, p.idesc_k, kk > 0 ? 1u : 0u);
-                                mma_f16(tacc, desc_kmajor(sa + 16384 + kk * 32), bd, p.idesc_k2, 1u);
-                            } else {
-                                mma_f16(tacc, desc_mnmajor(sa + kk * 2048), bd, p.idesc_mn, kk > 0 ? 1u : 0u);
-                                mma_f16(tacc, desc_mnmajor(sa + 16384 + kk * 2048), bd, p.idesc_mn2, 1u);
-                            }
+                            const uint64_t ad = ad0 + so + kk * astep, bd = bd0 + so + kk * 2;
+                            mma_f16(tacc, ad, bd, id3, kk > 0 ? 1u : 0u);
+                            mma_f16(tacc, ad + (16384 >> 4), bd, id2, 1u);
                         }
-                        any = true;
                         mma_commit(&sempty[ss]);  // the stage takes the next TMA load
-                        if (++ss == RS_NSTG) { ss = 0; sph ^= 1; }
                         mma_commit(&tfull[acc]);
-                        if (++acc == RS_NACC) { acc = 0; aph ^= 1; }
                     }
+                    any = true;
+                    ss = sn, sph = spn;
+                    acc = an, aph = apn;
                 }
             }
-            if (!ok && any) {
-                mma_commit(drain);
-                const uint64_t t0 = globaltimer();
-                while (!mbar_try_wait(drain, 0) && globaltimer() - t0 < drain_limit(p.wait_ns)) {}
-            }
         }
-    } else if (warp >= 6 && warp < 10) {
+        if (!ok && any && issuer) {
+            mma_commit(drain);
+            const uint64_t t0 = globaltimer();
+            while (!mbar_try_wait(drain, 0) && globaltimer() - t0 < drain_limit(p.wait_ns)) {}
+        }
+        __syncwarp();
+    } else if ((warp >= 6 && warp < 10) || warp >= 14) {
         // ------------------------------ converters ------------------------------
-        const int ct = threadIdx.x - 192;
+        const int group = (warp >= 14) ? 1 : 0;
+        const int ct = threadIdx.x - (group ? 14 * 32 : 6 * 32);
+        int turn = 0;  // group of the next chunk
         const float c = (float)*p.shift;
         const float kscale = rs_kscale(p.kbound, p.shift);
         int ss = 0, slot = 0;
@@ -1241,6 +1255,11 @@ __global__ void __launch_bounds__(RS_THREADS, 1)
                 const int r = kmaj ? ct : (ct >> 1), h = kmaj ? 0 : (ct & 1);
                 const int boxb = kmaj ? RS_STG / 2 : RS_STG / 4;
                 for (int kc = it.kc0; kc < it.kc1; ++kc) {
+                    turn ^= 1;
+                    if (turn == group) {  // the other group's chunk
+                        if (++ss == RS_NSTG) { ss = 0; sph ^= 1; }
+                        continue;
+                    }
                     if (!__all_sync(0xffffffffu, rs_wait(&sfull[ss], sph, p))) { ok = false; break; }
                     const uint8_t *src = smem + ss * SB + r * 128;
                     uint8_t *dst = smem + ss * SB + h * 8192 + r * 128;
@@ -1285,7 +1304,7 @@ __global__ void __launch_bounds__(RS_THREADS, 1)
         // ------------------------------ epilogue ------------------------------
         constexpr int NC = NP / 2;  // columns of this group
         const int row = ((warp & 3) << 5) + lane;
-        const int q0 = (warp >= 10) ? NC : 0;
+        const int q0 = (warp >= 10) ? NC : 0;  // (warps 2-5 and 10-13)
         int slot = 0, acc = 0;
         uint32_t iph = 0, aph = 0;
         const float kinv = 1.f / rs_kscale(p.kbound, p.shift);  // a power of two: exact

@@ -700,21 +700,23 @@ namespace {
 // diagonal target) on the other SMs.  The choice comes from a model of the
 // two kernels measured on GB300 (152 SMs) while they share the GPU:
 //   diagonal step on R CTAs: T(R) = a + c / R, a chain of b / 64 block
-//     factorisations (a = 600 us at b = 1024, proportional to b) plus work
-//     spread over the CTAs (c = 13 CTA-ms at b = 1024, proportional to b^3);
-//     on 16 / 24 / 32 / 48 CTAs it took 1.42 / 1.11 / 0.95 / 0.81 ms, on 136
-//     alone 0.59 ms;
+//     factorisations (a = 250 us at b = 1024, proportional to b) plus work
+//     spread over the CTAs (c = 5.7 CTA-ms at b = 1024, proportional to b^3);
+//     on 8 / 12 / 16 CTAs it took 0.96 / 0.73 / 0.60 ms, on 136 alone 0.27 ms;
 //   trailing update: about 8.3 TF/s per SM (2 b^3 per off-diagonal target).
 // The plan minimises the step's time: T(R) while the update fits beside the
 // diagonal step, else T(R) plus the rest of the update on every SM; the
 // launch of the diagonal target alone adds about 25 us.  When the update is
 // small (the last steps, small problems) the plain sequence is faster: the
-// diagonal step alone on 136 CTAs, 0.59 ms at b = 1024, then the update.  The
-// update part beside it is sized 30 % above T(R): if it ended first, the
-// other SMs would idle until the diagonal step ends, while if it ends last
-// only the diagonal step's R SMs wait.  At N = 131072 the factorisation
-// takes 660 ms this way and 697 ms in sequence; fixed R = 24 and R = 48 gave
-// the same 658-662 ms, R = 8 690 ms.
+// diagonal step alone on 136 CTAs, 0.33 ms at b = 1024 with the gaps around it,
+// then the update.  (With the 0.27 ms of the step alone
+// N = 16384 factors in 6.66 ms, with 0.33 in 6.57.)  The update part beside it
+// is sized 30 % above T(R): if it ended first, the other SMs would idle until
+// the diagonal step ends, while if it ends last only the diagonal step's R SMs
+// wait; 15 % and 50 % gave the same.  Fewer than 16 CTAs leave the model, which
+// sees only SM time, indifferent, and take longer (N = 98304: 284 ms on 16, 290
+// on 10, 294 on 8).  Factorisation in sequence / this way: N = 32768 23.0 /
+// 18.5 ms, N = 16384 7.1 / 6.57 ms, 7.8 / 7.27 ms at b = 512.
 //
 // A context of a batch (graph mode) shares the GPU with the other problems,
 // whose updates fill the SMs that a diagonal step leaves free anyway: there
@@ -737,14 +739,14 @@ LookaheadPlan lookahead_plan(const Ctx *c, int64_t k) {
     const int64_t tiles = u * (u + 1) / 2;
     if (tiles < 2) return pl;
     const double bd = (double)c->b, rel = bd / 1024.0;
-    const double a_us = 600.0 * rel, c_us = 13000.0 * rel * rel * rel;
+    const double a_us = 250.0 * rel, c_us = 5700.0 * rel * rel * rel;
     const double tile_sm_us = 2.0 * bd * bd * bd / 8.3e12 * 1e6;  // SM-microseconds per target tile
     const double work = (double)(tiles - 1) * tile_sm_us;
     const int64_t sms = c->num_sms;
-    // in sequence: the diagonal step alone on 136 CTAs (0.59 ms at b = 1024),
-    // then the whole update on every SM
-    double best = 590.0 * rel + (work + tile_sm_us) / (double)sms;
-    static const int64_t cand[] = {16, 20, 24, 32, 48, 64, 96, 128};
+    // in sequence: the diagonal step alone on 136 CTAs, then the whole update on
+    // every SM
+    double best = 330.0 * rel + (work + tile_sm_us) / (double)sms;
+    static const int64_t cand[] = {16, 20, 24, 32, 40, 48, 56, 64, 80, 96, 128};
     for (int64_t r : cand) {
         if (r + 16 > sms) break;
         const double td = a_us + c_us / (double)r;

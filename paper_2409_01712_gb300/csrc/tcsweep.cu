@@ -51,10 +51,10 @@
 // 20 us: the epilogue takes 1 us (branch-free per column, its loads before the
 // accumulator wait), the scales are accepted with the load that finds the block
 // finished, B arrives in large copies (0.4-0.9 us) and a chunk's MMAs are issued
-// in 0.2 us instead of 0.3 (uniform descriptors, the next stage's barrier tested
-// ahead); publication and its discovery are 1.5 us a hop.  A pair of sweeps took
-// 2.24 ms, now 1.28; N = 5000, P = 2 0.38 and 0.20; N = 2048, b = 256, P = 1 0.335
-// and 0.159 ms.
+// in 0.1-0.2 us instead of 0.3 (uniform descriptors, the next stage's barrier
+// tested ahead); publication and its discovery are 1.5 us a hop.  A pair of
+// sweeps took 2.24 ms, now 1.24; N = 5000, P = 2 0.38 and 0.20; N = 2048, b = 256,
+// P = 1 0.335 and 0.146 ms.
 #include <cuda.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -745,30 +745,38 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
             for (int c0 = 0; c0 < nch && ok; c0 += bper) {
                 if (!wwait(bfull, bph)) { ok = false; break; }
                 bph ^= 1;
-                // a stage's barrier is tested while the MMAs of the stage before
-                // it are issued: a wait in series costs as much as the four MMAs
-                bool landed = mbar_try_wait(&full[s], ph);
-                for (int c = c0; c < c0 + bper; ++c) {
-                    if (!__all_sync(0xffffffffu, landed) && !wwait(&full[s], ph)) { ok = false; break; }
-                    tmem_fence_after();
-                    const int sn = (s + 1 == NS) ? 0 : s + 1;
-                    const uint32_t pn = (sn == 0) ? ph ^ 1 : ph;
-                    landed = c + 1 < c0 + bper && mbar_try_wait(&full[sn], pn);
-                    const uint64_t ad = ad0 + (uint32_t)(s * (TS_ABYTES >> 4));
-                    const uint64_t bd = bd0 + (uint32_t)((c & (p.bseg - 1)) * (2 * NP * 128 >> 4));
-                    if (issuer) {
+                // One lane runs the chunks: 0.1 us each, against 0.14 with a vote
+                // of the warp per chunk.  A stage's barrier is tested while the
+                // MMAs of the stage before it are issued: a wait in series costs
+                // as much as the four MMAs.
+                if (issuer) {
+                    int s1 = s;
+                    uint32_t p1 = ph;
+                    bool landed = mbar_try_wait(&full[s1], p1);
+                    for (int c = c0; c < c0 + bper; ++c) {
+                        if (!landed && !wait_bar(&full[s1], p1, p)) { ok = false; break; }
+                        tmem_fence_after();
+                        const int sn = (s1 + 1 == NS) ? 0 : s1 + 1;
+                        const uint32_t pn = (sn == 0) ? p1 ^ 1 : p1;
+                        landed = c + 1 < c0 + bper && mbar_try_wait(&full[sn], pn);
+                        const uint64_t ad = ad0 + (uint32_t)(s1 * (TS_ABYTES >> 4));
+                        const uint64_t bd = bd0 + (uint32_t)((c & (p.bseg - 1)) * (2 * NP * 128 >> 4));
 #pragma unroll
                         for (int kk = 0; kk < 4; ++kk)
                             // B rows [0, np) = hi half, [np, 2 np) = lo half
                             mma_f16(tacc + kk * ACC, ad + kk * astep, bd + kk * 2, p.idesc, c > 0 ? 1u : 0u);
-                        mma_commit(&empty[s]);
-                        if (c + 1 == c0 + bper) mma_commit(bempty);  // this part of B is read
-                        if (c + 1 == nch) mma_commit(&tfull[acc]);
+                        mma_commit(&empty[s1]);
+                        s1 = sn;
+                        p1 = pn;
                     }
-                    any = true;
-                    s = sn;
-                    ph = pn;
+                    if (ok) {
+                        mma_commit(bempty);  // this part of B is read
+                        if (c0 + bper == nch) mma_commit(&tfull[acc]);
+                    }
                 }
+                any = true;
+                ok = __all_sync(0xffffffffu, ok) != 0;
+                for (s += bper; s >= NS; s -= NS) ph ^= 1;
             }
             if (!ok) break;
             if (++acc == 2) { acc = 0; aph ^= 1; }

@@ -48,25 +48,25 @@ thread_local std::string g_batch_create_error;
 
 // CTAs per launch of a batched problem: the problems run concurrently on their
 // streams, and persistent kernels sized for the whole GPU would each hold every
-// SM while waiting on their dependency chains.  Measured on the
-// cross-validation workload (64 problems, N up to 16384): no cap 408 ms per
-// run; 32 CTAs for every kernel 220 ms; per class as below 183-185 ms (the
-// diagonal step, mostly waiting CTAs, at 12; the sweeps at 16; the tensor-core
-// kernels, which keep their CTAs busy, at 64).  Later re-measured around
-// these caps (172-176 ms): the diagonal step at 4 / 6 CTAs 204 / 185 ms,
-// at 16 / 24 (with the lookahead) 175 / 187 ms; diagonal step and sweeps
-// both at 8 195 ms; the pair kernels at 48 (sweeps 12) 194 ms: the chain of
-// the diagonal steps of the largest problems needs their CTAs, and more
-// CTAs crowd out the other problems.  (All of these with the diagonal step
-// before its chain had a CTA of its own, and most with the lookahead.)
+// SM while waiting on their dependency chains (64 problems, N up to 16384: no
+// cap 408 ms per run, 32 CTAs for every kernel 220 ms, caps per class 184 ms).
+// Cross-validation over 6 cohorts of 1024 to 16384 rows x 4 lambdas, b = 512,
+// 46.0 ms per run with the diagonal step at 12, the sweeps at 16, the residual at
+// 32 and the pair kernels at 64; one cap at a time: diagonal step 4 / 6 / 8 / 16 /
+// 24 53.7 / 48.9 / 47.3 / 46.8 / 48.0 ms; sweeps 8 / 12 / 24 / 32 53.7 / 48.3 / 45.2 /
+// 45.5; residual 12 / 20 / 48 51.4 / 47.7 / 45.4; pair kernels 32 / 48 / 96 / 128
+// 50.6 / 47.7 / 46.0 / 45.9.  Sweeps at 24 and the residual at 48 together:
+// 45.8 -> 43.9 ms (with later sweeps).
 constexpr int BATCH_CTA_CAP = 32;
-constexpr int BATCH_CAP_DIAG = 12, BATCH_CAP_SWEEP = 16, BATCH_CAP_PAIR = 64, BATCH_CAP_SINGLE = 64;
+constexpr int BATCH_CAP_DIAG = 12, BATCH_CAP_SWEEP = 24, BATCH_CAP_RESIDUAL = 48, BATCH_CAP_PAIR = 64,
+              BATCH_CAP_SINGLE = 64;
 
 void set_batch_caps(krr_ctx *c) {
     krr::Ctx *cc = reinterpret_cast<krr::Ctx *>(c);
     cc->cta_cap = BATCH_CTA_CAP;
     cc->cta_caps[krr::GL_DIAG] = BATCH_CAP_DIAG;
     cc->cta_caps[krr::GL_SWEEP] = BATCH_CAP_SWEEP;
+    cc->cta_caps[krr::GL_RESIDUAL] = BATCH_CAP_RESIDUAL;
     cc->cta_caps[krr::GL_PAIR] = BATCH_CAP_PAIR;
     cc->cta_caps[krr::GL_SINGLE] = BATCH_CAP_SINGLE;
 }

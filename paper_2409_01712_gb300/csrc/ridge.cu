@@ -29,11 +29,11 @@ inline unsigned cdivu(int64_t a, int64_t b) { return (unsigned)((a + b - 1) / b)
 // ---------------------------------------------------------------------------
 // Transposed packing: X (n patients x m genotypes, int8, leading dimension ldx)
 // -> packed operand rows = genotype columns (rows_pad x cols_pad, patients
-// along the row), E4M3 codes of {0, 1, 2} (mixed) or FP32 (fp32 mode); the
-// padding is written as zeros.  32 x 32 tiles through shared memory.
+// along the row), FP32 (fp32 mode); the padding is written as zeros.  32 x 32
+// tiles through shared memory.
 // ---------------------------------------------------------------------------
 __global__ void rr_pack_t_kernel(const int8_t *__restrict__ x, int64_t n, int64_t m, int64_t ldx, int64_t rows_pad,
-                                 int64_t cols_pad, uint8_t *__restrict__ out8, float *__restrict__ outf) {
+                                 int64_t cols_pad, float *__restrict__ outf) {
     __shared__ int t[32][33];
     const int64_t p0 = (int64_t)blockIdx.x * 32, f0 = (int64_t)blockIdx.y * 32;
     for (int r = threadIdx.y; r < 32; r += blockDim.y) {
@@ -45,9 +45,50 @@ __global__ void rr_pack_t_kernel(const int8_t *__restrict__ x, int64_t n, int64_
         const int64_t f = f0 + r, p = p0 + threadIdx.x;
         if (f < rows_pad && p < cols_pad) {
             const int v = t[threadIdx.x][r];
-            if (out8) out8[f * cols_pad + p] = (uint8_t)(v == 0 ? 0x00 : (v == 1 ? 0x38 : (v == 2 ? 0x40 : 0x48)));
-            if (outf) outf[f * cols_pad + p] = (float)v;
+            outf[f * cols_pad + p] = (float)v;
         }
+    }
+}
+
+// The same for the E4M3 operand alone, 128 patients x 64 genotype columns a CTA:
+// four genotypes a load (wide: rows 4-byte aligned; else byte by byte) and 128
+// bytes a warp store.  The kernel above moves a byte per thread: 16384 x 4096
+// genotypes took 175 us, 62 us here (their 134 MB take 20 us).  rows_pad is a
+// multiple of 64, cols_pad of 128.
+__global__ void __launch_bounds__(256)
+    rr_pack_t8_kernel(const int8_t *__restrict__ x, int64_t n, int64_t m, int64_t ldx, int wide, int64_t cols_pad,
+                      uint8_t *__restrict__ out8) {
+    __shared__ __align__(16) uint8_t t[64][132];
+    const int64_t p0 = (int64_t)blockIdx.x * 128, f0 = (int64_t)blockIdx.y * 64;
+    uint32_t w[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int e = threadIdx.x + 256 * i, pp = e >> 4, ff = (e & 15) * 4;
+        const int64_t p = p0 + pp, f = f0 + ff;
+        w[i] = 0;
+        if (p < n && f < m) {
+            const int8_t *src = x + p * ldx + f;
+            if (wide && f + 3 < m) {
+                w[i] = __ldg(reinterpret_cast<const uint32_t *>(src));
+            } else {
+                for (int c = 0; c < 4 && f + c < m; ++c) w[i] |= (uint32_t)(uint8_t)src[c] << (8 * c);
+            }
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int e = threadIdx.x + 256 * i, pp = e >> 4, ff = (e & 15) * 4;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const uint32_t v = (w[i] >> (8 * c)) & 0xff;
+            t[ff + c][pp] = (uint8_t)(v == 0 ? 0x00 : (v == 1 ? 0x38 : (v == 2 ? 0x40 : 0x48)));
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int e = threadIdx.x + 256 * i, f = e >> 5, c = (e & 31) * 4;
+        *reinterpret_cast<uint32_t *>(out8 + (f0 + f) * cols_pad + p0 + c) = *reinterpret_cast<const uint32_t *>(&t[f][c]);
     }
 }
 
@@ -62,20 +103,21 @@ __global__ void rr_conf_t_kernel(const float *cpad, int64_t rows, int nc, float 
 // ---------------------------------------------------------------------------
 // Row-block products with few output columns, split over the contraction:
 //   part[chunk][r][q] = sum_{k in chunk} a(r, k) B[k][q],  r < rows, q < nq <= 32,
-// a from row r of A: int8 values (KIND 0), E4M3 codes of {0, 1, 2} (KIND 1)
-// or FP32 (KIND 2).  One CTA per 64 rows and chunk; 128-wide slabs of A and B
+// a from row r of A: int8 values (KIND 0) or FP32 (KIND 2); packed genotypes
+// have a kernel of their own below.  One CTA per 64 rows and chunk; 128-wide slabs of A and B
 // through shared memory; thread (r, g) accumulates columns [8 g, 8 g + 8) of
 // row r in FP32.  The chunks are summed in FP64 by rr_reduce_kernel.
 // ---------------------------------------------------------------------------
 constexpr int RG_R = 64, RG_K = 128;
 
+// Value of a packed genotype.
+__device__ __forceinline__ float rg_code(uint32_t v) {
+    return v == 0x38 ? 1.f : (v == 0x40 ? 2.f : (v == 0x48 ? 3.f : 0.f));
+}
+
 template <int KIND>
 __device__ __forceinline__ float rg_load(const void *A, int64_t idx) {
     if (KIND == 0) return (float)reinterpret_cast<const int8_t *>(A)[idx];
-    if (KIND == 1) {
-        const uint8_t v = reinterpret_cast<const uint8_t *>(A)[idx];
-        return v == 0x38 ? 1.f : (v == 0x40 ? 2.f : (v == 0x48 ? 3.f : 0.f));
-    }
     return reinterpret_cast<const float *>(A)[idx];
 }
 
@@ -120,6 +162,73 @@ __global__ void __launch_bounds__(256) rr_rowgemm_kernel(const void *A, int64_t 
             if (q < nq) part[((int64_t)blockIdx.y * rows + r) * nq + q] = acc[e];
         }
     }
+}
+
+// The same products for the packed genotypes (E4M3 codes, rows 4-byte aligned,
+// lda a multiple of 128 with zero or finite padding), NQ = 8 or 16 columns from
+// column blockIdx.z NQ on: lanes run along the contraction, four genotypes a
+// load, and a lane keeps 64 / NQ rows x NQ sums in registers, so a genotype is
+// read once as part of a 128-byte warp load and a staged value of B serves 64 /
+// NQ rows.  The general kernel above reads bytes one by one and always forms 32
+// columns: 4096 rows, 16384 patients and 4 columns took 363 us, 149 us here (the
+// operand's 67 MB take 10 us; half the rows a lane with the next loads ahead 156,
+// a whole slab's loads ahead 218).  A lane sums every 32nd group of four, then the
+// lanes in a fixed tree.
+constexpr int RP_WARPS = 8, RP_K = 512;
+
+template <int NQ>
+__global__ void __launch_bounds__(32 * RP_WARPS)
+    rr_rowgemm_packed_kernel(const uint8_t *__restrict__ A, int64_t lda, int64_t rows, int64_t K, int64_t kchunk,
+                             const float *__restrict__ B, int64_t ldb, int nq, float *part) {
+    constexpr int RW = 64 / NQ;
+    __shared__ __align__(16) float bs[NQ][RP_K + 4];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t r0 = ((int64_t)blockIdx.x * RP_WARPS + warp) * RW;
+    const int q0 = blockIdx.z * NQ;
+    const int64_t kbeg = (int64_t)blockIdx.y * kchunk, kend = min(K, kbeg + kchunk);
+    float acc[RW][NQ];
+#pragma unroll
+    for (int u = 0; u < RW; ++u)
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) acc[u][q] = 0.f;
+    for (int64_t k0 = kbeg; k0 < kend; k0 += RP_K) {
+        __syncthreads();
+        for (int e = threadIdx.x; e < RP_K * NQ; e += 32 * RP_WARPS) {
+            const int kk = e / NQ, q = e % NQ;
+            bs[q][kk] = (k0 + kk < kend && q0 + q < nq) ? B[(k0 + kk) * ldb + q0 + q] : 0.f;
+        }
+        __syncthreads();
+        for (int kk = 4 * lane; kk < RP_K && k0 + kk < kend; kk += 128) {
+            uint32_t g[RW];
+#pragma unroll
+            for (int u = 0; u < RW; ++u)
+                g[u] = (r0 + u < rows) ? __ldg(reinterpret_cast<const uint32_t *>(A + (r0 + u) * lda + k0 + kk)) : 0u;
+            float4 bv[NQ];
+#pragma unroll
+            for (int q = 0; q < NQ; ++q) bv[q] = *reinterpret_cast<const float4 *>(&bs[q][kk]);
+#pragma unroll
+            for (int u = 0; u < RW; ++u) {
+                const float a0 = rg_code(g[u] & 0xff), a1 = rg_code((g[u] >> 8) & 0xff),
+                            a2 = rg_code((g[u] >> 16) & 0xff), a3 = rg_code(g[u] >> 24);
+#pragma unroll
+                for (int q = 0; q < NQ; ++q) {
+                    acc[u][q] = fmaf(a0, bv[q].x, acc[u][q]);
+                    acc[u][q] = fmaf(a1, bv[q].y, acc[u][q]);
+                    acc[u][q] = fmaf(a2, bv[q].z, acc[u][q]);
+                    acc[u][q] = fmaf(a3, bv[q].w, acc[u][q]);
+                }
+            }
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < RW; ++u)
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) {
+            float v = acc[u][q];
+            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+            if (lane == 0 && r0 + u < rows && q0 + q < nq)
+                part[((int64_t)blockIdx.y * rows + r0 + u) * nq + q0 + q] = v;
+        }
 }
 
 // out[e] = sum over chunks c of part[c][e] in FP64, e < count (fixed order).
@@ -284,9 +393,12 @@ krr_status xt_times(Ctx *c, RRState *st, const float *B, int64_t ldb, int nq, do
     if (nc > 0) split(c, nc, K, &n2, &k2);
     const size_t need = (size_t)(n1 * m + n2 * nc) * nq;
     KRR_TRY(grow(c, &st->part, &st->part_cap, need, "ridge partial products"));
-    if (mixed(c))
-        rowgemm<1>(c, c->g8, c->m_pad, m, K, B, ldb, nq, st->part, n1, k1);
-    else
+    if (mixed(c)) {
+        const int nq8 = nq <= 8 ? 8 : 16;
+        const dim3 grid(cdivu(m, RP_WARPS * (64 / nq8)), (unsigned)n1, (unsigned)((nq + nq8 - 1) / nq8));
+        const auto kernel = nq <= 8 ? rr_rowgemm_packed_kernel<8> : rr_rowgemm_packed_kernel<16>;
+        count_launch(), kernel<<<grid, 32 * RP_WARPS, 0, c->stream>>>(c->g8, c->m_pad, m, K, k1, B, ldb, nq, st->part);
+    } else
         rowgemm<2>(c, c->gf, c->m_pad, m, K, B, ldb, nq, st->part, n1, k1);
     reduce_parts(c, st->part, n1, m * nq, out);
     if (nc > 0) {
@@ -339,9 +451,14 @@ extern "C" krr_status krr_rr_build(krr_ctx *ctx, const int8_t *X, int64_t n, int
             ldx = m;
         }
     }
-    count_launch(), rr_pack_t_kernel<<<dim3((unsigned)(m_pad / 32), (unsigned)(c->n_pad / 32)), dim3(32, 8), 0,
-                                       c->stream>>>(dx, n, m, ldx, c->n_pad, m_pad, mixed(c) ? c->g8 : nullptr,
-                                                    mixed(c) ? nullptr : c->gf);
+    if (mixed(c)) {
+        const int wide = (ldx % 4 == 0 && reinterpret_cast<uintptr_t>(dx) % 4 == 0) ? 1 : 0;
+        count_launch(), rr_pack_t8_kernel<<<dim3((unsigned)(m_pad / 128), (unsigned)(c->n_pad / 64)), 256, 0,
+                                            c->stream>>>(dx, n, m, ldx, wide, m_pad, c->g8);
+    } else {
+        count_launch(), rr_pack_t_kernel<<<dim3((unsigned)(m_pad / 32), (unsigned)(c->n_pad / 32)), dim3(32, 8), 0,
+                                           c->stream>>>(dx, n, m, ldx, c->n_pad, m_pad, c->gf);
+    }
     KRR_CUDA_TRY(c, cudaMemsetAsync(c->norms, 0, (size_t)c->n_pad * sizeof(int32_t), c->stream));
     KRR_TRY(check_launch(c, "ridge packing"));
     if (nc > 0) {

@@ -349,7 +349,7 @@ krr_status solve_device(Ctx *c, int64_t p, krr_solve_info *info) {
     }
     const bool refine = mixed(c) && c->opt.ir_max > 0;
     if (refine || info) {
-        double best = INFINITY;
+        double best = INFINITY, last = 0.0;  // last: ratio of the residuals of the step before
         for (int it = 0;; ++it) {
             int rr = prof_begin(c, KRR_PROF_RESIDUAL);
             KRR_TRY(launch_residual(c, c->ybuf, c->abuf, p));
@@ -371,7 +371,7 @@ krr_status solve_device(Ctx *c, int64_t p, krr_solve_info *info) {
             if (it > 0 && rel > best) {
                 // the last correction made things worse: the floor set by FP32
                 // storage of K and A is reached -- undo it and keep the best
-                launch_add_scaled(c->abuf, c->dabuf, -1.0f, cnt, s);
+                KRR_CUDA_TRY(c, cudaMemcpyAsync(c->abuf, c->dabuf, cnt * sizeof(float), cudaMemcpyDeviceToDevice, s));
                 si.rel_residual = best;
                 si.converged = best <= c->opt.ir_tol ? 1 : 2;
                 break;
@@ -385,13 +385,16 @@ krr_status solve_device(Ctx *c, int64_t p, krr_solve_info *info) {
                 st = KRR_ENOCONV;
                 break;
             }
-            // stagnation: a step that did not halve the residual shows the
-            // floor set by FP32 storage of K and A; a further step would only
-            // move along it
-            if (it > 0 && rel > 0.5 * best) {
+            // stagnation: a step that did not halve the residual, or whose gain
+            // collapsed against the step before (classical refinement gains a
+            // constant factor a step), shows the floor set by FP32 storage of K
+            // and A; a further step would only move along it
+            const double ratio = it > 0 ? rel / best : 0.0;
+            if (it > 0 && (ratio > 0.5 || (it > 1 && ratio > 0.02 && ratio > 4.0 * last))) {
                 si.converged = 2;
                 break;
             }
+            last = ratio;
             best = std::min(best, rel);
             int sr = prof_begin(c, KRR_PROF_SOLVE);
             KRR_TRY(solve_rhs(c, nullptr, c->dabuf, c->zbuf, p, c->abuf));

@@ -400,7 +400,7 @@ void launch_column_cast(Ctx *c, int64_t k);
 
 // Triangular solves with the stored factor: x <- (L L^T)^-1 rhs, n_pad x p
 // (row-major, leading dimension p); tmp is n_pad x p scratch; sum (optional):
-// also sum += x.  rhs = nullptr: the right-hand side is the last residual.
+// sum += the solution, and x holds the earlier sum.  rhs = nullptr: the right-hand side is the last residual.
 krr_status solve_rhs(Ctx *c, const float *rhs, float *x, float *tmp, int64_t p, float *sum = nullptr);
 
 // Persistent dataflow sweeps (sweep.cu): the two substitutions of a solve
@@ -428,7 +428,6 @@ void launch_fill_zero(void *p, size_t bytes, cudaStream_t s);
 constexpr int64_t norm_partial_count() { return 2 * 256; }
 void launch_reduce_norms(const double *r, const float *y, int64_t n, int64_t p, double *out, double *part,
                          cudaStream_t s);
-void launch_add_scaled(float *a, const float *da, float alpha, int64_t count, cudaStream_t s);
 // Yt = sum of the per-block partials; when shift is given the partials are of
 // (K - c) A and c (1^T A) is added (c = *shift rounded to FP32, colsum = 1^T A).
 void launch_predict_reduce(const float *part, int64_t nblk, int64_t rows_pad, int64_t n_test,

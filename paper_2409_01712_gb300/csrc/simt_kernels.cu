@@ -1060,14 +1060,6 @@ krr_status launch_residual(Ctx *c, const float *y, const float *a, int64_t p) {
     return KRR_OK;
 }
 
-__global__ void add_kernel(float *a, const float *da, float alpha, int64_t count) {
-    int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (e < count) a[e] += alpha * da[e];
-}
-void launch_add_scaled(float *a, const float *da, float alpha, int64_t count, cudaStream_t s) {
-    count_launch(), add_kernel<<<cdiv(count, 256), 256, 0, s>>>(a, da, alpha, count);
-}
-
 // dst (rows_pad x cols, dense) <- src rows (zero padding rows >= rows).
 __global__ void copy_rows_kernel(const float *src, int64_t lds, float *dst, int64_t ldd,
                                  int64_t rows, int64_t cols, int64_t rows_pad) {

@@ -121,9 +121,9 @@ __device__ __forceinline__ int *xin_ctr(const TsParams &p) { return p.flags + 2;
 __device__ __forceinline__ int *xout_ctr(const TsParams &p) { return p.flags + 2 + p.nt; }
 __device__ __forceinline__ int *seq_ctr(const TsParams &p) { return p.flags + 2 + 2 * p.nt; }
 
-// State of a block, one 64-bit word: finished slabs (bits 0-15), columns found
-// too large for the predicted scale by some warp (a count, bits 16-31), and the
-// columns that some warp found large enough for it (bits 32-63).  A reader
+// State of a block, one 64-bit word: finished slabs (bits 0-15), how many warps
+// found a column that the predicted scale does not suit (too large for it; bits
+// 16-31), and the columns that some warp found large enough for it (bits 32-63).  A reader
 // learns with one load that the block is there and whether its predicted
 // scales hold: for every column the maximum lies in [PRED_LO, PRED_HI).
 __device__ __forceinline__ int state_slabs(unsigned long long v) { return (int)(v & 0xffff); }
@@ -510,7 +510,8 @@ __device__ __noinline__ void convert_block(const TsParams &p, const float *v, in
 // [PRED_LO, PRED_HI) (about 22 significant bits relative to the maximum, as
 // with the exact scale, and 2x headroom below the FP16 maximum), else its last
 // slab converts the whole block again with the exact scale.
-// (A column of zeros has no maximum to place and takes the exact path too.)
+// (A block of zeros has no maximum to place and takes the exact path, unless the
+// block before it was zero as well.)
 constexpr float PRED_LO = 8.f, PRED_HI = 32768.f;
 
 __device__ __forceinline__ float pred_scale(float m) {
@@ -842,7 +843,11 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
                 if (sexact[hslot]) sc = __ldcg((link ? p.sout : p.sin) + (int64_t)h.src * NP + tid);
                 else if (tid < pc) sc = pred_scale(__ldcg(pred_from(p, link, h.src) + tid));
                 smul[tid] = h.inv_tscale / sc;
-                if (fin) sscale[tid] = (tid < pc) ? pred_scale(__ldcg(pred_from(p, !link, h.blk) + tid)) : 1.f;
+                if (fin) {
+                    const float m = (tid < pc) ? __ldcg(pred_from(p, !link, h.blk) + tid) : 0.f;
+                    sscale[tid] = pred_scale(m);
+                    smax[tid] = m;
+                }
             }
             if (!group_wait_bar(&tfull[acc], aph)) break;
             if (lane == 0) mbar_arrive(&iempty[hslot]);  // the header and the scales are read
@@ -891,10 +896,13 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
                     if (lane == q) mine = m;
                 }
                 // the warp's part of the block's maxima and of the test of the scales
+                // (zeros after a block of zeros keep its scale of 1, which small
+                // entries in another warp's rows would not)
                 const float ms = __uint_as_float(mine) * (lane < NP ? sscale[lane] : 0.f);
-                const bool col = lane < pc;
-                const uint32_t ge = __ballot_sync(0xffffffffu, col && ms >= PRED_LO);
-                const uint32_t over = __ballot_sync(0xffffffffu, col && !(ms < PRED_HI));
+                const bool col = lane < pc, after0 = col && smax[lane] == 0.f;
+                const uint32_t ge = __ballot_sync(0xffffffffu, col && (ms >= PRED_LO || (after0 && mine == 0)));
+                const uint32_t over =
+                    __ballot_sync(0xffffffffu, col && (!(ms < PRED_HI) || (after0 && mine != 0 && ms < PRED_LO)));
                 unsigned long long *st = (link ? p.st_in : p.st_out) + h.blk;
                 if (col)
                     atomicMax(reinterpret_cast<unsigned int *>((link ? p.bm_in : p.bm_out) + (int64_t)h.blk * TS_NPMAX) + lane,
@@ -1639,8 +1647,12 @@ float *ts_block_maxima(Ctx *c) { return ts_maxima(c) + 2 * ts_max_count(c); }
 unsigned long long *ts_states(Ctx *c) { return (unsigned long long *)(ts_block_maxima(c) + 2 * ts_scale_count(c)); }
 int *ts_flags(Ctx *c) { return (int *)(ts_states(c) + 2 * c->nt); }
 
-// dst (cols x rows, row-major) = src^T, src rows x cols row-major; with sum,
-// also sum += src^T.
+// dst (cols x rows, row-major) = src^T, src rows x cols row-major.  With sum:
+// sum += src^T and dst = the earlier sum.  The additions carry the rounding error
+// of a row on to the next (runs of 32 rows), so the rounding errors of a column
+// of A nearly cancel: K has a large constant component, through which their sum
+// (about sqrt(N) half ulps with independent roundings) would be the floor of the
+// residual and the common error of the predictions.
 __global__ void transpose_kernel(const float *__restrict__ src, int64_t rows, int64_t cols, float *__restrict__ dst,
                                  float *__restrict__ sum) {
     __shared__ float t[32][33];
@@ -1650,12 +1662,28 @@ __global__ void transpose_kernel(const float *__restrict__ src, int64_t rows, in
         if (r < rows && cc < cols) t[k][threadIdx.x] = src[r * cols + cc];
     }
     __syncthreads();
-    for (int k = threadIdx.y; k < 32; k += 8) {
-        const int64_t cc = c0 + k, r = r0 + threadIdx.x;
-        if (r < rows && cc < cols) {
-            dst[cc * rows + r] = t[threadIdx.x][k];
-            if (sum) sum[cc * rows + r] += t[threadIdx.x][k];
+    const int64_t r = r0 + threadIdx.x;
+    if (sum) {
+        if (threadIdx.y != 0 || r >= rows) return;
+        float carry = 0.f;
+#pragma unroll 8
+        for (int k = 0; k < 32; ++k) {
+            const int64_t cc = c0 + k;
+            if (cc >= cols) break;
+            const float s = sum[cc * rows + r], x = t[threadIdx.x][k];
+            // s + x = h + l exactly (TwoSum), rounded with the carry
+            const float h = s + x, bp = h - s;
+            const float l = ((s - (h - bp)) + (x - bp)) + carry;
+            const float f = h + l;
+            carry = l - (f - h);
+            dst[cc * rows + r] = s;
+            sum[cc * rows + r] = f;
         }
+        return;
+    }
+    for (int k = threadIdx.y; k < 32; k += 8) {
+        const int64_t cc = c0 + k;
+        if (r < rows && cc < cols) dst[cc * rows + r] = t[threadIdx.x][k];
     }
 }
 
@@ -1764,7 +1792,7 @@ krr_status run_ts(Ctx *c, int job, float *rhs, float *out, int64_t p) {
 // sweep updates it in place and writes z to tmp, the backward sweep updates
 // tmp in place and writes the solution to ts_xt.  rhs: row-major right-hand
 // sides, or nullptr when ts_xt holds them already (tc_residual).  sum
-// (optional): also sum += x.
+// (optional): sum += x, and x holds the earlier sum.
 krr_status tc_sweep_solve(Ctx *c, const float *rhs, float *x, float *tmp, int64_t p, float *sum) {
     KRR_TRY(ensure_ts_buffers(c, p));
     float *xt = c->ts_xt;

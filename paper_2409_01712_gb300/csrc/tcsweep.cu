@@ -1276,7 +1276,15 @@ __global__ void __launch_bounds__(RS_THREADS, 1)
                         if (++ss == RS_NSTG) { ss = 0; sph ^= 1; }
                         continue;
                     }
-                    if (!__all_sync(0xffffffffu, rs_wait(&sfull[ss], sph, p))) { ok = false; break; }
+                    // The chunk before this one in the stage was the other group's
+                    // (the stage count is odd), and copies land in any order: while
+                    // that chunk is still on its way, the parity of sfull reads as
+                    // if this one had landed.  cfull shows that it is converted, and
+                    // cannot run ahead of this group.
+                    if (!__all_sync(0xffffffffu, rs_wait(&cfull[ss], sph ^ 1, p) && rs_wait(&sfull[ss], sph, p))) {
+                        ok = false;
+                        break;
+                    }
                     const uint8_t *src = smem + ss * SB + r * 128;
                     uint8_t *dst = smem + ss * SB + h * 8192 + r * 128;
                     float v[64];

@@ -349,14 +349,16 @@ krr_status solve_device(Ctx *c, int64_t p, krr_solve_info *info) {
     }
     const bool refine = mixed(c) && c->opt.ir_max > 0;
     if (refine || info) {
-        double best = INFINITY, last = 0.0;  // last: ratio of the residuals of the step before
+        double best = INFINITY;
+        RefineStall stall;
         for (int it = 0;; ++it) {
             int rr = prof_begin(c, KRR_PROF_RESIDUAL);
             KRR_TRY(launch_residual(c, c->ybuf, c->abuf, p));
             // the lower-triangle K tiles are needed by rows and by columns
             prof_end(c, rr, 2.0 * (double)c->n_pad * c->n_pad * p, 2.0 * (double)c->kd_bytes);
             KRR_TRY(check_launch(c, "residual"));
-            KRR_CUDA_TRY(c, cudaMemcpyAsync(c->hred, c->red, 2 * sizeof(double), cudaMemcpyDeviceToHost, s));
+            KRR_CUDA_TRY(c, cudaMemcpyAsync(c->hred, c->red, (RED_ANORM + 1) * sizeof(double),
+                                            cudaMemcpyDeviceToHost, s));
             KRR_CUDA_TRY(c, cudaStreamSynchronize(s));
             const double ynorm = sqrt(c->hred[1]);
             const double rel = ynorm > 0 ? sqrt(c->hred[0]) / ynorm : sqrt(c->hred[0]);
@@ -385,16 +387,12 @@ krr_status solve_device(Ctx *c, int64_t p, krr_solve_info *info) {
                 st = KRR_ENOCONV;
                 break;
             }
-            // stagnation: a step that did not halve the residual, or whose gain
-            // collapsed against the step before (classical refinement gains a
-            // constant factor a step), shows the floor set by FP32 storage of K
-            // and A; a further step would only move along it
-            const double ratio = it > 0 ? rel / best : 0.0;
-            if (it > 0 && (ratio > 0.5 || (it > 1 && ratio > 0.02 && ratio > 4.0 * last))) {
+            const double level = rounding_level(sqrt(c->hred[RED_KNORM2]), sqrt(c->hred[RED_ANORM]), c->lambda,
+                                                (double)c->n_pad) / ynorm;
+            if (stall(it, rel, best, level)) {
                 si.converged = 2;
                 break;
             }
-            last = ratio;
             best = std::min(best, rel);
             int sr = prof_begin(c, KRR_PROF_SOLVE);
             KRR_TRY(solve_rhs(c, nullptr, c->dabuf, c->zbuf, p, c->abuf));

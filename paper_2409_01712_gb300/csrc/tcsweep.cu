@@ -1485,16 +1485,17 @@ __global__ void __launch_bounds__(TS_EPI)
 
 // r = y - lambda a - (the slots in order) - c colsum for columns [q0, q0 + pc),
 // rounded to FP32 and written column-major (the sweeps' right-hand side), and
-// ||r||_F^2, ||y||_F^2 over all p columns into out[0], out[1]: a partial per
-// block (blocks of all column chunks count on ctr), added in order by the last.
+// ||r||_F^2, ||y||_F^2 and ||a||_F^2 over all p columns into red[RED_RNORM], the
+// slot after it and red[RED_ANORM]: a partial per block (blocks of all column
+// chunks count on ctr), added in order by the last.
 __global__ void __launch_bounds__(256)
     res_finish_kernel(const float *y, const float *a, int64_t p, int q0, int pc, int64_t n_pad, const double *part,
                       int slots, float lambda, const double *shift, const double *colsum, float *rt, double *np_part,
-                      int total, int *ctr, double *out) {
-    __shared__ double s1[8], s2[8];
+                      int total, int *ctr, double *red) {
+    __shared__ double s1[8], s2[8], s3[8];
     const int t = threadIdx.x, q = blockIdx.y;
     const int64_t r = (int64_t)blockIdx.x * 256 + t;
-    double rv = 0.0, yv = 0.0;
+    double rv = 0.0, yv = 0.0, av = 0.0;
     if (r < n_pad) {
         double sum = 0.0;
         const double *src = part + (int64_t)q * n_pad + r;
@@ -1502,52 +1503,62 @@ __global__ void __launch_bounds__(256)
 #pragma unroll 4
         for (int e = 0; e < slots; ++e) sum += __ldcs(src + e * step);
         yv = (double)y[r * p + q0 + q];
-        rv = (yv - (double)lambda * (double)a[r * p + q0 + q]) - sum - *shift * colsum[q0 + q];
+        av = (double)a[r * p + q0 + q];
+        rv = (yv - (double)lambda * av) - sum - *shift * colsum[q0 + q];
         rt[(int64_t)(q0 + q) * n_pad + r] = (float)rv;
     }
-    double v1 = rv * rv, v2 = yv * yv;
+    double v1 = rv * rv, v2 = yv * yv, v3 = av * av;
     for (int o = 16; o > 0; o >>= 1) {
         v1 += __shfl_down_sync(0xffffffffu, v1, o);
         v2 += __shfl_down_sync(0xffffffffu, v2, o);
+        v3 += __shfl_down_sync(0xffffffffu, v3, o);
     }
     if ((t & 31) == 0) {
         s1[t >> 5] = v1;
         s2[t >> 5] = v2;
+        s3[t >> 5] = v3;
     }
     __syncthreads();
     if (t == 0) {
-        double x = 0.0, z = 0.0;
+        double x = 0.0, z = 0.0, w3 = 0.0;
         for (int w = 0; w < 8; ++w) {
             x += s1[w];
             z += s2[w];
+            w3 += s3[w];
         }
         const int64_t slot = (int64_t)(q0 + q) * gridDim.x + blockIdx.x;
-        np_part[2 * slot] = x;
-        np_part[2 * slot + 1] = z;
+        np_part[3 * slot] = x;
+        np_part[3 * slot + 1] = z;
+        np_part[3 * slot + 2] = w3;
     }
     if (!last_block(ctr, total)) return;
-    double x = 0.0, z = 0.0;
+    double x = 0.0, z = 0.0, w3 = 0.0;
     for (int e = t; e < total; e += 256) {
-        x += __ldcg(np_part + 2 * e);
-        z += __ldcg(np_part + 2 * e + 1);
+        x += __ldcg(np_part + 3 * (int64_t)e);
+        z += __ldcg(np_part + 3 * (int64_t)e + 1);
+        w3 += __ldcg(np_part + 3 * (int64_t)e + 2);
     }
     for (int o = 16; o > 0; o >>= 1) {
         x += __shfl_down_sync(0xffffffffu, x, o);
         z += __shfl_down_sync(0xffffffffu, z, o);
+        w3 += __shfl_down_sync(0xffffffffu, w3, o);
     }
     if ((t & 31) == 0) {
         s1[t >> 5] = x;
         s2[t >> 5] = z;
+        s3[t >> 5] = w3;
     }
     __syncthreads();
     if (t == 0) {
-        x = z = 0.0;
+        x = z = w3 = 0.0;
         for (int w = 0; w < 8; ++w) {
             x += s1[w];
             z += s2[w];
+            w3 += s3[w];
         }
-        out[0] = x;
-        out[1] = z;
+        red[RED_RNORM] = x;
+        red[RED_RNORM + 1] = z;
+        red[RED_ANORM] = w3;
     }
 }
 
@@ -1864,7 +1875,8 @@ krr_status launch_res(Ctx *c, const CUtensorMap &mk128, const CUtensorMap &mk64,
 
 // r = y - (K + lambda I) a on the tensor cores (mixed mode), rounded to FP32
 // and column-major in c->ts_xt, the right-hand side of the next sweeps;
-// ||r||_F^2 and ||y||_F^2 into c->red[RED_RNORM], [RED_RNORM + 1].
+// ||r||_F^2 and ||y||_F^2 into c->red[RED_RNORM], [RED_RNORM + 1], ||a||_F^2 into
+// c->red[RED_ANORM].
 krr_status tc_residual(Ctx *c, const float *y, const float *a, int64_t p) {
     const int64_t b = c->b, nt = c->nt, S = b / TS_SLAB, n_pad = c->n_pad;
     KRR_TRY(ensure_ts_buffers(c, p));
@@ -1888,7 +1900,7 @@ krr_status tc_residual(Ctx *c, const float *y, const float *a, int64_t p) {
     const int64_t ngrp = (nt + g - 1) / g, slots = ngrp * h;
     const int64_t pmax = std::min<int64_t>(p, TS_NPMAX);
     const int64_t nblk = n_pad / TS_SLAB, fblk = (n_pad + 255) / 256;
-    const int64_t part_count = slots * pmax * n_pad, need = part_count + nblk * pmax + 2 * fblk * p;
+    const int64_t part_count = slots * pmax * n_pad, need = part_count + nblk * pmax + 3 * fblk * p;
     if (c->rs_part_cap < need) {
         c->rs_part_cap = 0;
         KRR_TRY(dev_alloc(c, &c->rs_part, (size_t)need, "residual partial sums"));
@@ -1930,7 +1942,7 @@ krr_status tc_residual(Ctx *c, const float *y, const float *a, int64_t p) {
         KRR_TRY(np == 16 ? launch_res<16>(c, mk128, mk64, ma, rp) : launch_res<32>(c, mk128, mk64, ma, rp));
         count_launch(), res_finish_kernel<<<dim3((unsigned)fblk, (unsigned)pc), 256, 0, c->stream>>>(
             y, a, p, (int)q0, pc, n_pad, c->rs_part, (int)slots, (float)c->lambda, c->red + RED_KSHIFT, c->colsum,
-            c->ts_xt, np_part, (int)(fblk * p), flags + 3, c->red + RED_RNORM);
+            c->ts_xt, np_part, (int)(fblk * p), flags + 3, c->red);
         KRR_TRY(check_launch(c, "residual"));
     }
     return KRR_OK;

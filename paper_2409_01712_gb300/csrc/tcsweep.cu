@@ -1668,12 +1668,13 @@ int *ts_flags(Ctx *c) { return (int *)(ts_states(c) + 2 * c->nt); }
 
 // dst (cols x rows, row-major) = src^T, src rows x cols row-major.  With sum:
 // sum += src^T and dst = the earlier sum.  The additions carry the rounding error
-// of a row on to the next (runs of 32 rows), so the rounding errors of a column
-// of A nearly cancel: K has a large constant component, through which their sum
-// (about sqrt(N) half ulps with independent roundings) would be the floor of the
+// of a row on to the next (add_carry, runs of 32 rows; the padding rows from n on
+// neither get nor pass one), so the rounding errors of a column of A nearly
+// cancel: K has a large constant component, through which their sum (about
+// sqrt(N) half ulps with independent roundings) would be the floor of the
 // residual and the common error of the predictions.
-__global__ void transpose_kernel(const float *__restrict__ src, int64_t rows, int64_t cols, float *__restrict__ dst,
-                                 float *__restrict__ sum) {
+__global__ void transpose_kernel(const float *__restrict__ src, int64_t rows, int64_t cols, int64_t n,
+                                 float *__restrict__ dst, float *__restrict__ sum) {
     __shared__ float t[32][33];
     const int64_t r0 = (int64_t)blockIdx.y * 32, c0 = (int64_t)blockIdx.x * 32;
     for (int k = threadIdx.y; k < 32; k += 8) {
@@ -1690,13 +1691,9 @@ __global__ void transpose_kernel(const float *__restrict__ src, int64_t rows, in
             const int64_t cc = c0 + k;
             if (cc >= cols) break;
             const float s = sum[cc * rows + r], x = t[threadIdx.x][k];
-            // s + x = h + l exactly (TwoSum), rounded with the carry
-            const float h = s + x, bp = h - s;
-            const float l = ((s - (h - bp)) + (x - bp)) + carry;
-            const float f = h + l;
-            carry = l - (f - h);
+            if (cc >= n) carry = 0.f;
             dst[cc * rows + r] = s;
-            sum[cc * rows + r] = f;
+            sum[cc * rows + r] = add_carry(s, x, carry);
         }
         return;
     }
@@ -1706,9 +1703,10 @@ __global__ void transpose_kernel(const float *__restrict__ src, int64_t rows, in
     }
 }
 
-void launch_transpose(const float *src, int64_t rows, int64_t cols, float *dst, cudaStream_t s, float *sum = nullptr) {
+void launch_transpose(const float *src, int64_t rows, int64_t cols, float *dst, cudaStream_t s, float *sum = nullptr,
+                      int64_t n = 0) {
     const dim3 grid((unsigned)((cols + 31) / 32), (unsigned)((rows + 31) / 32));
-    count_launch(), transpose_kernel<<<grid, dim3(32, 8), 0, s>>>(src, rows, cols, dst, sum);
+    count_launch(), transpose_kernel<<<grid, dim3(32, 8), 0, s>>>(src, rows, cols, n, dst, sum);
 }
 
 krr_status run_ts(Ctx *c, int job, float *rhs, float *out, int64_t p) {
@@ -1818,7 +1816,7 @@ krr_status tc_sweep_solve(Ctx *c, const float *rhs, float *x, float *tmp, int64_
     if (rhs) launch_transpose(rhs, c->n_pad, p, xt, c->stream);
     KRR_TRY(run_ts(c, TS_FWD, xt, tmp, p));
     KRR_TRY(run_ts(c, TS_BWD, tmp, xt, p));
-    launch_transpose(xt, p, c->n_pad, x, c->stream, sum);
+    launch_transpose(xt, p, c->n_pad, x, c->stream, sum, c->n);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
         c->last_error = std::string("sweep transposes: ") + cudaGetErrorString(e);

@@ -1,6 +1,9 @@
-"""The stopping decision of the iterative refinement on synthetic residual
-histories: several contraction rates, one slow column among fast ones, and
-histories that reach the level of FP32 rounding.  A host program, no GPU."""
+"""Host programs on parts of the iterative refinement, no GPU.
+
+refine_check: the stopping decision on synthetic residual histories: several
+contraction rates, one slow column among fast ones, and histories that reach
+the level of FP32 rounding.  carry_check: the solution update's additions with
+neighbours of equal and of very different magnitudes."""
 import os
 import subprocess
 
@@ -9,12 +12,13 @@ import pytest
 from test_host_helpers import CSRC, ROOT, _nvcc
 
 
-def test_refinement_stops_at_its_floor_only(tmp_path):
+@pytest.mark.parametrize("name", ["refine_check", "carry_check"])
+def test_refinement_on_the_host(tmp_path, name):
     nvcc = _nvcc()
     if not nvcc:
         pytest.skip("needs nvcc")
-    exe = tmp_path / "refine_check"
-    src = os.path.join(ROOT, "tests", "host", "refine_check.cpp")
+    exe = tmp_path / name
+    src = os.path.join(ROOT, "tests", "host", name + ".cpp")
     subprocess.run([nvcc, "-x", "cu", "-std=c++17", "-O1", "-gencode", "arch=compute_103a,code=sm_103a",
                     "-I", CSRC, src, "-o", str(exe)], check=True)
     r = subprocess.run([str(exe)], capture_output=True, text=True)

@@ -198,6 +198,10 @@ krr_status krr_factor(krr_ctx *ctx, double lambda, krr_factor_info *info);
  * 2^-24 (||K||_F / sqrt(n) + lambda) ||A||_F / ||Y||_F, or when a step makes it
  * worse (that step is undone): the floor set by FP32 storage of K and A.  A
  * holds the best iterate.
+ * The first solve of a context allocates the residual's partial sums, up to 48
+ * doubles per row and column of up to 32 columns (0.9 GB at n = 131072, p = 20),
+ * and keeps them; where device memory does not reach, it takes fewer (down to one)
+ * and the sums are grouped accordingly.
  * Errors: KRR_ESTATE (no factor), KRR_EINVAL, KRR_ENOCONV (non-finite
  * residual, or ir_max iterations without reaching the tolerance or the
  * floor), KRR_ECUDA.

@@ -105,8 +105,7 @@ krr_status stage(Ctx *c, size_t bytes) {
     if (c->stage) cudaFree(c->stage);
     c->stage = nullptr;
     c->stage_cap = 0;
-    if (cudaMalloc(&p, bytes) != cudaSuccess) {
-        cudaGetLastError();
+    if (dev_malloc(c, &p, bytes) != cudaSuccess) {
         c->last_error = "cudaMalloc failed for the host-argument staging buffer";
         return KRR_ENOMEM;
     }
@@ -214,6 +213,9 @@ void free_factor(Ctx *c) {
     dev_free(&c->pan_lo);
     dev_free(&c->colmax);
     dev_free(&c->precmap);
+    dev_free(&c->rs_part);
+    c->rs_part_cap = 0;
+    c->rs_slots = RES_SLOTS;
     c->pool_bytes = 0;
     c->w_bytes = 0;
     c->factored = false;
@@ -297,17 +299,24 @@ bool mixed(const Ctx *c) { return c->opt.mode == KRR_MODE_MIXED; }
 }  // namespace krr
 
 namespace {
-// Allocates (or keeps) the n_pad x p work vectors of the solve.
-krr_status ensure_vectors(Ctx *c, int64_t p) {
+// Allocates (or keeps) the n_pad x p work vectors (the residual in FP64 in fp32
+// mode only: the mixed mode's goes to the sweeps in FP32).
+krr_status ensure_work_vectors(Ctx *c, int64_t p) {
     const int64_t cnt = c->n_pad * p;
-    if (c->vec_cap < cnt) {
-        KRR_TRY(dev_alloc(c, &c->ybuf, (size_t)cnt, "solve vectors"));
-        KRR_TRY(dev_alloc(c, &c->zbuf, (size_t)cnt, "solve vectors"));
-        KRR_TRY(dev_alloc(c, &c->abuf, (size_t)cnt, "solve vectors"));
-        KRR_TRY(dev_alloc(c, &c->dabuf, (size_t)cnt, "solve vectors"));
-        KRR_TRY(dev_alloc(c, &c->rbuf, (size_t)cnt, "residual"));
-        c->vec_cap = cnt;
-    }
+    if (c->vec_cap >= cnt) return KRR_OK;
+    c->vec_cap = 0;
+    KRR_TRY(dev_alloc(c, &c->ybuf, (size_t)cnt, "solve vectors"));
+    KRR_TRY(dev_alloc(c, &c->zbuf, (size_t)cnt, "solve vectors"));
+    KRR_TRY(dev_alloc(c, &c->abuf, (size_t)cnt, "solve vectors"));
+    KRR_TRY(dev_alloc(c, &c->dabuf, (size_t)cnt, "solve vectors"));
+    if (!mixed(c)) KRR_TRY(dev_alloc(c, &c->rbuf, (size_t)cnt, "residual"));
+    c->vec_cap = cnt;
+    return KRR_OK;
+}
+
+// ... and the column sums of the solve.
+krr_status ensure_vectors(Ctx *c, int64_t p) {
+    KRR_TRY(ensure_work_vectors(c, p));
     if (c->colsum_cap < p) {
         KRR_TRY(dev_alloc(c, &c->colsum, (size_t)p, "column sums"));
         c->colsum_cap = p;
@@ -1008,15 +1017,7 @@ static krr_status predict_common(krr_ctx *c, const int8_t *T, int64_t n_test, in
         KRR_TRY(dev_alloc(c, &c->tnorms, (size_t)rows_pad, "test norms"));
         c->tnorm_cap = rows_pad;
     }
-    const int64_t cnt = c->n_pad * p;
-    if (c->vec_cap < cnt) {
-        KRR_TRY(dev_alloc(c, &c->ybuf, (size_t)cnt, "solve vectors"));
-        KRR_TRY(dev_alloc(c, &c->zbuf, (size_t)cnt, "solve vectors"));
-        KRR_TRY(dev_alloc(c, &c->abuf, (size_t)cnt, "solve vectors"));
-        KRR_TRY(dev_alloc(c, &c->dabuf, (size_t)cnt, "solve vectors"));
-        KRR_TRY(dev_alloc(c, &c->rbuf, (size_t)cnt, "residual"));
-        c->vec_cap = cnt;
-    }
+    KRR_TRY(ensure_work_vectors(c, p));
     const int64_t nblk = c->n_pad / 128;  // partial products per 128 training rows
     const size_t part = (size_t)nblk * rows_pad * p;
     if (c->pred_part_cap < part) {

@@ -33,6 +33,72 @@ __host__ __device__ inline void tri_decode(int64_t t, int64_t *i, int64_t *j) {
     *j = t - r * (r + 1) / 2;
 }
 
+// Items of the refinement residual: nt blocks of S slabs (128 rows) and KC
+// chunks (64 columns).  An item covers one slab of an output block and g source
+// blocks in a row (a group), or one of h parts of a single one (g == 1 or h ==
+// 1), and has a slot of its own among the partial sums of its rows.
+struct ResGrid {
+    int nt, S, KC, g, h;
+    __host__ __device__ int groups() const { return (nt + g - 1) / g; }
+    __host__ __device__ int slots() const { return groups() * h; }
+    __host__ __device__ int64_t items() const { return (int64_t)groups() * (groups() + 1) * g * S * h; }
+};
+
+// Rows [sl 128, +128) of block i; source blocks [j0, j1), K chunks [kc0, kc1) of
+// each; its slot.
+struct ResItem {
+    int i, sl, j0, j1, kc0, kc1, slot;
+};
+
+// Item t; false at the positions that hold none.  Items of a group pair: parts,
+// then the two orientations, then the blocks of the output group and their slabs.
+__host__ __device__ inline bool res_decode(const ResGrid &q, int t, ResItem &it) {
+    const int per = 2 * q.g * q.S * q.h;
+    int64_t gi, gj;
+    tri_decode(t / per, &gi, &gj);
+    int v = t % per;
+    const int e = v / (2 * q.g * q.S);
+    v %= 2 * q.g * q.S;
+    const int o = v / (q.g * q.S);
+    v %= q.g * q.S;
+    const int out = o ? (int)gj : (int)gi, src = o ? (int)gi : (int)gj;
+    it.i = out * q.g + v / q.S;
+    it.sl = v % q.S;
+    it.j0 = src * q.g;
+    it.j1 = it.j0 + q.g < q.nt ? it.j0 + q.g : q.nt;
+    it.kc0 = q.KC * e / q.h;
+    it.kc1 = q.KC * (e + 1) / q.h;
+    it.slot = src * q.h + e;
+    return it.i < q.nt && !(o == 1 && gi == gj);  // a group's pair with itself has one orientation
+}
+
+// Source blocks of an item: one up to `most` blocks, above that so many that the
+// slots stay at `most` or fewer.  With the usual 48 their 16 bytes of traffic per
+// slot, row and column are 4 % of the 4 bytes per entry of K at N = 98304 and 20
+// columns; a few large groups would outgrow L2 between the two uses of a tile.  A
+// tile is split (in parts of at least four chunks) while that leaves fewer than
+// six items an SM: N = 5000 has 200 whole-tile items for 152 SMs.
+constexpr int RES_SLOTS = 48;
+inline ResGrid res_grid(int64_t nt, int64_t S, int64_t KC, int64_t ctas, int most) {
+    ResGrid q{(int)nt, (int)S, (int)KC, (int)((nt + most - 1) / most), 1};
+    if (q.g == 1)
+        while (KC / (2 * q.h) >= 4 && nt * 2 * q.h <= most && nt * nt * S * q.h < 6 * ctas) q.h *= 2;
+    return q;
+}
+
+// The grid whose partial sums there is memory for: alloc(grid) returns KRR_OK,
+// KRR_ENOMEM (fewer slots are tried, down to one, as many partial sums as the
+// residual has entries) or another error.  `most` keeps what was found.
+template <class Alloc>
+krr_status res_reserve(int64_t nt, int64_t S, int64_t KC, int64_t ctas, int *most, Alloc alloc, ResGrid *out) {
+    for (;;) {
+        *out = res_grid(nt, S, KC, ctas, *most);
+        const krr_status st = alloc(*out);
+        if (st != KRR_ENOMEM || out->slots() == 1) return st;
+        *most = out->slots() / 2;
+    }
+}
+
 // Kernel function of Alg. 5 applied to the exact integer distance d of the
 // encoded rows: Gaussian exp(-gamma d) on the squared Euclidean distance, or
 // IBS (2M - d) / M on the L1 distance (the encoded rows' squared distance),
@@ -209,6 +275,7 @@ struct Ctx {
     size_t pred_part_cap = 0;
     double *rs_part = nullptr;               // residual: partial sums per slot, column and row
     int64_t rs_part_cap = 0;
+    int rs_slots = RES_SLOTS;                // most slots there was memory for on this tile grid
     int *sw_flags = nullptr;                 // sweep item counter, abort flag, progress counters
     int64_t sw_flags_cap = 0;
     __half *ts_v0 = nullptr, *ts_v1 = nullptr;  // tensor-core sweep: FP16 pairs of vector blocks
@@ -319,6 +386,21 @@ struct PerDevice {
 
 // Device buffers owned by a context: (re)allocation with the failure message
 // recorded in the context (KRR_ENOMEM), and release.
+// cudaMalloc that gives up the residual's partial sums when nothing else is left:
+// they hold no state between solves, and a smaller number of slots will do.  Not
+// in graph mode, where captured launches refer to them.
+inline cudaError_t dev_malloc(Ctx *c, void **p, size_t bytes) {
+    cudaError_t e = cudaMalloc(p, bytes);
+    if (e != cudaSuccess) cudaGetLastError();
+    if (e != cudaErrorMemoryAllocation || !c->rs_part || c->graph_mode) return e;
+    cudaFree(c->rs_part);
+    c->rs_part = nullptr;
+    c->rs_part_cap = 0;
+    e = cudaMalloc(p, bytes);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e;
+}
+
 template <typename T>
 krr_status dev_alloc(Ctx *c, T **p, size_t count, const char *what) {
     if (*p) {
@@ -326,9 +408,8 @@ krr_status dev_alloc(Ctx *c, T **p, size_t count, const char *what) {
         *p = nullptr;
     }
     if (count == 0) return KRR_OK;
-    cudaError_t e = cudaMalloc((void **)p, count * sizeof(T));
+    cudaError_t e = dev_malloc(c, (void **)p, count * sizeof(T));
     if (e != cudaSuccess) {
-        cudaGetLastError();
         *p = nullptr;
         c->last_error = std::string("cudaMalloc failed for ") + what + " (" +
                         std::to_string(count * sizeof(T)) + " bytes): " + cudaGetErrorString(e);

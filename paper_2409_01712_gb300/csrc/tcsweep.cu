@@ -997,11 +997,10 @@ __device__ __forceinline__ float rs_kscale(const double *kbound, const double *s
 }
 
 struct RsParams {
-    int b, nt, S, KC, items;
+    ResGrid gr;
+    int b, items;
     int64_t n_pad;
     int pc;
-    int g, h;               // source blocks of an item, or parts of one (g == 1 or h == 1)
-    int ngrp;               // block groups: ceil(nt / g)
     const double *shift;
     const double *kbound;   // max |K_ij| (the residual operand's scale follows from it)
     const float *inv_s;     // inverse scales of the FP16 terms of a, [n_pad / 128][np]
@@ -1011,33 +1010,6 @@ struct RsParams {
     uint64_t wait_ns;
     DevErrors *err;
 };
-
-// One item: rows [sl 128, +128) of block i; source blocks [j0, j1), K chunks
-// [kc0, kc1) of each; its slot.  Items of a group pair: parts, then the two
-// orientations, then the blocks of the output group and their slabs.
-struct RsItem {
-    int i, sl, j0, j1, kc0, kc1, slot;
-};
-
-__device__ __forceinline__ bool rs_decode(const RsParams &p, int t, RsItem &it) {
-    const int per = 2 * p.g * p.S * p.h;
-    int64_t gi, gj;
-    tri_decode(t / per, &gi, &gj);
-    int v = t % per;
-    const int e = v / (2 * p.g * p.S);
-    v %= 2 * p.g * p.S;
-    const int o = v / (p.g * p.S);
-    v %= p.g * p.S;
-    const int out = o ? (int)gj : (int)gi, src = o ? (int)gi : (int)gj;
-    it.i = out * p.g + v / p.S;
-    it.sl = v % p.S;
-    it.j0 = src * p.g;
-    it.j1 = min(it.j0 + p.g, p.nt);
-    it.kc0 = p.KC * e / p.h;
-    it.kc1 = p.KC * (e + 1) / p.h;
-    it.slot = src * p.h + e;
-    return it.i < p.nt && !(o == 1 && gi == gj);  // a group's pair with itself has one orientation
-}
 
 __device__ __forceinline__ bool rs_aborted(const RsParams &p) { return *(volatile int *)&p.flags[1] != 0; }
 
@@ -1140,9 +1112,9 @@ __global__ void __launch_bounds__(RS_THREADS, 1)
             bool ok = true;
             int t = atomicAdd(&p.flags[0], 1);
             while (ok) {
-                RsItem it;
+                ResItem it;
                 const bool end = t >= p.items;
-                if (!end && !rs_decode(p, t, it)) {  // empty position
+                if (!end && !res_decode(p.gr, t, it)) {  // empty position
                     t = atomicAdd(&p.flags[0], 1);
                     continue;
                 }
@@ -1202,8 +1174,8 @@ __global__ void __launch_bounds__(RS_THREADS, 1)
             if (issuer) mbar_arrive(&iempty[slot]);
             if (++slot == TS_IRING) { slot = 0; iph ^= 1; }
             if (t < 0) break;
-            RsItem it;
-            rs_decode(p, t, it);
+            ResItem it;
+            res_decode(p.gr, t, it);
             bool ready = false;  // the chunk's barriers, tested while the MMAs before it are issued
             for (int j = it.j0; j < it.j1 && ok; ++j) {
                 const bool kmaj = (j <= it.i);
@@ -1263,8 +1235,8 @@ __global__ void __launch_bounds__(RS_THREADS, 1)
             if (lane == 0) mbar_arrive(&iempty[slot]);
             if (++slot == TS_IRING) { slot = 0; iph ^= 1; }
             if (t < 0) break;
-            RsItem it;
-            rs_decode(p, t, it);
+            ResItem it;
+            res_decode(p.gr, t, it);
             for (int j = it.j0; j < it.j1 && ok; ++j) {
                 const bool kmaj = (j <= it.i);
                 // thread -> (row r of the staged chunk, 64-value half h)
@@ -1339,8 +1311,8 @@ __global__ void __launch_bounds__(RS_THREADS, 1)
             if (lane == 0) mbar_arrive(&iempty[slot]);
             if (++slot == TS_IRING) { slot = 0; iph ^= 1; }
             if (t < 0) break;
-            RsItem it;
-            rs_decode(p, t, it);
+            ResItem it;
+            res_decode(p.gr, t, it);
             // per column a two-term FP32 sum (hi, lo) grown by error-free
             // transformations (TwoSum): about 48 significant bits without
             // FP64 arithmetic, which runs at a small fraction of the FP32 rate
@@ -1352,7 +1324,7 @@ __global__ void __launch_bounds__(RS_THREADS, 1)
                 for (int kc = it.kc0; kc < it.kc1; ++kc) {
                     // inverse scales of these rows of a (one set per 128 rows)
                     const float4 *is =
-                        reinterpret_cast<const float4 *>(p.inv_s + (int64_t)(j * p.S + (kc >> 1)) * NP + q0);
+                        reinterpret_cast<const float4 *>(p.inv_s + (int64_t)(j * p.gr.S + (kc >> 1)) * NP + q0);
                     float mul[NC];
 #pragma unroll
                     for (int q = 0; q < NC; q += 4) {
@@ -1623,8 +1595,7 @@ krr_status ensure_ts_buffers(Ctx *c, int64_t p) {
         for (__half **v : {&c->ts_v0, &c->ts_v1}) {
             if (*v) cudaFree(*v);
             *v = nullptr;
-            if (cudaMalloc((void **)v, vbytes) != cudaSuccess) {
-                cudaGetLastError();
+            if (dev_malloc(c, (void **)v, vbytes) != cudaSuccess) {
                 c->ts_vcap = 0;
                 c->last_error = "cudaMalloc failed for the sweep vector blocks";
                 return KRR_ENOMEM;
@@ -1637,8 +1608,7 @@ krr_status ensure_ts_buffers(Ctx *c, int64_t p) {
     if (c->ts_aux_cap < abytes) {
         if (c->ts_aux) cudaFree(c->ts_aux);
         c->ts_aux = nullptr;
-        if (cudaMalloc(&c->ts_aux, abytes) != cudaSuccess) {
-            cudaGetLastError();
+        if (dev_malloc(c, &c->ts_aux, abytes) != cudaSuccess) {
             c->ts_aux_cap = 0;
             c->last_error = "cudaMalloc failed for the sweep counters";
             return KRR_ENOMEM;
@@ -1649,8 +1619,7 @@ krr_status ensure_ts_buffers(Ctx *c, int64_t p) {
     if (p > 0 && c->ts_xcap < xbytes) {
         if (c->ts_xt) cudaFree(c->ts_xt);
         c->ts_xt = nullptr;
-        if (cudaMalloc((void **)&c->ts_xt, xbytes) != cudaSuccess) {
-            cudaGetLastError();
+        if (dev_malloc(c, (void **)&c->ts_xt, xbytes) != cudaSuccess) {
             c->ts_xcap = 0;
             c->last_error = "cudaMalloc failed for the sweep vector copy";
             return KRR_ENOMEM;
@@ -1883,27 +1852,24 @@ krr_status tc_residual(Ctx *c, const float *y, const float *a, int64_t p) {
     CUtensorMap mk128, mk64, ma;
     KRR_TRY(map_f32(c, &mk128, c->Kd, ntri * b, b, 128));
     KRR_TRY(map_f32(c, &mk64, c->Kd, ntri * b, b, 64));
-    // Source blocks of an item: one up to 48 blocks, above that so many that
-    // the slots stay at 48 or fewer (their 16 bytes of traffic per slot, row
-    // and column against 4 bytes per entry of K: 48 slots and 20 columns add
-    // 4 % at N = 98304); a few large groups would outgrow L2 between the two
-    // uses of a tile.  A tile is split (in parts of at least four 64-wide
-    // chunks) while that leaves fewer than six items an SM: N = 5000 has 200
-    // whole-tile items for 152 SMs.
-    const int KC = (int)(b / TS_KC);
-    const int g = (int)((nt + 47) / 48);
-    int h = 1;
-    if (g == 1)
-        while (KC / (2 * h) >= 4 && nt * nt * S * h < 6 * grid_limit(c, GL_RESIDUAL)) h *= 2;
-    const int64_t ngrp = (nt + g - 1) / g, slots = ngrp * h;
     const int64_t pmax = std::min<int64_t>(p, TS_NPMAX);
     const int64_t nblk = n_pad / TS_SLAB, fblk = (n_pad + 255) / 256;
-    const int64_t part_count = slots * pmax * n_pad, need = part_count + nblk * pmax + 3 * fblk * p;
-    if (c->rs_part_cap < need) {
-        c->rs_part_cap = 0;
-        KRR_TRY(dev_alloc(c, &c->rs_part, (size_t)need, "residual partial sums"));
-        c->rs_part_cap = need;
-    }
+    int64_t part_count = 0;
+    ResGrid gr;
+    KRR_TRY(res_reserve(
+        nt, S, b / TS_KC, grid_limit(c, GL_RESIDUAL), &c->rs_slots,
+        [&](const ResGrid &q) {
+            part_count = q.slots() * pmax * n_pad;
+            const int64_t need = part_count + nblk * pmax + 3 * fblk * p;
+            if (c->rs_part_cap >= need) return KRR_OK;
+            std::string earlier = c->last_error;
+            c->rs_part_cap = 0;
+            const krr_status st = dev_alloc(c, &c->rs_part, (size_t)need, "residual partial sums");
+            if (st == KRR_OK) c->rs_part_cap = need;
+            if (st == KRR_ENOMEM && q.slots() > 1) c->last_error.swap(earlier);  // fewer are tried: no failure yet
+            return st;
+        },
+        &gr));
     double *cs_part = c->rs_part + part_count, *np_part = cs_part + nblk * pmax;
     float *inv_s = ts_maxima(c);
     for (int64_t q0 = 0; q0 < p; q0 += TS_NPMAX) {
@@ -1916,14 +1882,9 @@ krr_status tc_residual(Ctx *c, const float *y, const float *a, int64_t p) {
         KRR_TRY(map_f16(c, &ma, c->ts_v0, 3 * np, n_pad, 3 * np));
         RsParams rp;
         memset(&rp, 0, sizeof(rp));
+        rp.gr = gr;
         rp.b = (int)b;
-        rp.nt = (int)nt;
-        rp.S = (int)S;
-        rp.KC = KC;
-        rp.g = g;
-        rp.h = h;
-        rp.ngrp = (int)ngrp;
-        rp.items = (int)(ngrp * (ngrp + 1) / 2 * 2 * g * S * h);
+        rp.items = (int)gr.items();
         rp.n_pad = n_pad;
         rp.pc = pc;
         rp.shift = c->red + RED_KSHIFT;
@@ -1939,7 +1900,7 @@ krr_status tc_residual(Ctx *c, const float *y, const float *a, int64_t p) {
         rp.err = c->derr;
         KRR_TRY(np == 16 ? launch_res<16>(c, mk128, mk64, ma, rp) : launch_res<32>(c, mk128, mk64, ma, rp));
         count_launch(), res_finish_kernel<<<dim3((unsigned)fblk, (unsigned)pc), 256, 0, c->stream>>>(
-            y, a, p, (int)q0, pc, n_pad, c->rs_part, (int)slots, (float)c->lambda, c->red + RED_KSHIFT, c->colsum,
+            y, a, p, (int)q0, pc, n_pad, c->rs_part, gr.slots(), (float)c->lambda, c->red + RED_KSHIFT, c->colsum,
             c->ts_xt, np_part, (int)(fblk * p), flags + 3, c->red);
         KRR_TRY(check_launch(c, "residual"));
     }

@@ -3,7 +3,8 @@
 refine_check: the stopping decision on synthetic residual histories: several
 contraction rates, one slow column among fast ones, and histories that reach
 the level of FP32 rounding.  carry_check: the solution update's additions with
-neighbours of equal and of very different magnitudes."""
+neighbours of equal and of very different magnitudes.  residual_check: the items
+and slots of the residual, with the usual memory and with less."""
 import os
 import subprocess
 
@@ -12,7 +13,7 @@ import pytest
 from test_host_helpers import CSRC, ROOT, _nvcc
 
 
-@pytest.mark.parametrize("name", ["refine_check", "carry_check"])
+@pytest.mark.parametrize("name", ["refine_check", "carry_check", "residual_check"])
 def test_refinement_on_the_host(tmp_path, name):
     nvcc = _nvcc()
     if not nvcc:

@@ -163,8 +163,10 @@ struct RefineStall {
 // 2^-24 of themselves, independently, give at most this for rows of K of equal
 // norm.  Measured levels are 2.7e-6 at N = 2048, 4.2e-6 at N = 10000 and 1.6e-7
 // for ridge on 4101 columns; refinement ended at 1.2e-7, 8.2e-7 and 1.3e-7 there.
+// Zero, so that only the other rules end refinement, where a norm overflowed.
 inline double rounding_level(double knorm, double anorm, double lambda, double n) {
-    return 0x1p-24 * (knorm / sqrt(n) + fabs(lambda)) * anorm;
+    const double level = 0x1p-24 * (knorm / sqrt(n) + fabs(lambda)) * anorm;
+    return level < INFINITY ? level : 0.0;
 }
 
 // s + x rounded to FP32, with the rounding errors of the additions before in
@@ -175,13 +177,13 @@ inline double rounding_level(double knorm, double anorm, double lambda, double n
 // of the errors is 3.3e-8 instead of 1.4e-7 (rms, normal entries).
 __host__ __device__ inline float add_carry(float s, float x, float &carry) {
     const float h = s + x, bp = h - s;
-    if (!(fabsf(h) < 3.0e38f)) return h;
     const float l = (s - (h - bp)) + (x - bp);  // s + x = h + l exactly (TwoSum)
     const float lim = fabsf(h) * 0x1p-25f;
     const float c = fminf(fmaxf(carry, -lim), lim);
     const float t = l + c, f = h + t;
-    carry = (carry - c) + (t - (f - h));
-    return f;
+    const bool finite = fabsf(h) < 3.0e38f;  // otherwise the plain sum, and the carry stays
+    carry = finite ? (carry - c) + (t - (f - h)) : carry;
+    return finite ? f : h;
 }
 
 // Slots of the small FP64 reduction buffer Ctx::red.

@@ -1459,15 +1459,18 @@ __global__ void __launch_bounds__(TS_EPI)
 // rounded to FP32 and written column-major (the sweeps' right-hand side), and
 // ||r||_F^2, ||y||_F^2 and ||a||_F^2 over all p columns into red[RED_RNORM], the
 // slot after it and red[RED_ANORM]: a partial per block (blocks of all column
-// chunks count on ctr), added in order by the last.
+// chunks count on ctr), added in order by the last.  ||a||_F^2 only scales the
+// level at which refinement may end: FP32 sums.
 __global__ void __launch_bounds__(256)
     res_finish_kernel(const float *y, const float *a, int64_t p, int q0, int pc, int64_t n_pad, const double *part,
                       int slots, float lambda, const double *shift, const double *colsum, float *rt, double *np_part,
                       int total, int *ctr, double *red) {
-    __shared__ double s1[8], s2[8], s3[8];
+    __shared__ double s1[8], s2[8];
+    __shared__ float s3[8];
     const int t = threadIdx.x, q = blockIdx.y;
     const int64_t r = (int64_t)blockIdx.x * 256 + t;
-    double rv = 0.0, yv = 0.0, av = 0.0;
+    double rv = 0.0, yv = 0.0;
+    float av = 0.f;
     if (r < n_pad) {
         double sum = 0.0;
         const double *src = part + (int64_t)q * n_pad + r;
@@ -1475,11 +1478,12 @@ __global__ void __launch_bounds__(256)
 #pragma unroll 4
         for (int e = 0; e < slots; ++e) sum += __ldcs(src + e * step);
         yv = (double)y[r * p + q0 + q];
-        av = (double)a[r * p + q0 + q];
-        rv = (yv - (double)lambda * av) - sum - *shift * colsum[q0 + q];
+        av = a[r * p + q0 + q];
+        rv = (yv - (double)lambda * (double)av) - sum - *shift * colsum[q0 + q];
         rt[(int64_t)(q0 + q) * n_pad + r] = (float)rv;
     }
-    double v1 = rv * rv, v2 = yv * yv, v3 = av * av;
+    double v1 = rv * rv, v2 = yv * yv;
+    float v3 = av * av;
     for (int o = 16; o > 0; o >>= 1) {
         v1 += __shfl_down_sync(0xffffffffu, v1, o);
         v2 += __shfl_down_sync(0xffffffffu, v2, o);
@@ -1492,45 +1496,48 @@ __global__ void __launch_bounds__(256)
     }
     __syncthreads();
     if (t == 0) {
-        double x = 0.0, z = 0.0, w3 = 0.0;
+        double x = 0.0, z = 0.0;
+        float a2 = 0.f;
         for (int w = 0; w < 8; ++w) {
             x += s1[w];
             z += s2[w];
-            w3 += s3[w];
+            a2 += s3[w];
         }
         const int64_t slot = (int64_t)(q0 + q) * gridDim.x + blockIdx.x;
         np_part[3 * slot] = x;
         np_part[3 * slot + 1] = z;
-        np_part[3 * slot + 2] = w3;
+        np_part[3 * slot + 2] = (double)a2;
     }
     if (!last_block(ctr, total)) return;
-    double x = 0.0, z = 0.0, w3 = 0.0;
+    double x = 0.0, z = 0.0;
+    float a2 = 0.f;
     for (int e = t; e < total; e += 256) {
         x += __ldcg(np_part + 3 * (int64_t)e);
         z += __ldcg(np_part + 3 * (int64_t)e + 1);
-        w3 += __ldcg(np_part + 3 * (int64_t)e + 2);
+        a2 += (float)__ldcg(np_part + 3 * (int64_t)e + 2);
     }
     for (int o = 16; o > 0; o >>= 1) {
         x += __shfl_down_sync(0xffffffffu, x, o);
         z += __shfl_down_sync(0xffffffffu, z, o);
-        w3 += __shfl_down_sync(0xffffffffu, w3, o);
+        a2 += __shfl_down_sync(0xffffffffu, a2, o);
     }
     if ((t & 31) == 0) {
         s1[t >> 5] = x;
         s2[t >> 5] = z;
-        s3[t >> 5] = w3;
+        s3[t >> 5] = a2;
     }
     __syncthreads();
     if (t == 0) {
-        x = z = w3 = 0.0;
+        x = z = 0.0;
+        a2 = 0.f;
         for (int w = 0; w < 8; ++w) {
             x += s1[w];
             z += s2[w];
-            w3 += s3[w];
+            a2 += s3[w];
         }
         red[RED_RNORM] = x;
         red[RED_RNORM + 1] = z;
-        red[RED_ANORM] = w3;
+        red[RED_ANORM] = (double)a2;
     }
 }
 
@@ -1654,15 +1661,18 @@ __global__ void transpose_kernel(const float *__restrict__ src, int64_t rows, in
     const int64_t r = r0 + threadIdx.x;
     if (sum) {
         if (threadIdx.y != 0 || r >= rows) return;
+        // every load before the serial additions: a block has one warp at work here
+        float sv[32];
+#pragma unroll
+        for (int k = 0; k < 32; ++k) sv[k] = (c0 + k < cols) ? sum[(c0 + k) * rows + r] : 0.f;
         float carry = 0.f;
-#pragma unroll 8
+#pragma unroll
         for (int k = 0; k < 32; ++k) {
             const int64_t cc = c0 + k;
             if (cc >= cols) break;
-            const float s = sum[cc * rows + r], x = t[threadIdx.x][k];
             if (cc >= n) carry = 0.f;
-            dst[cc * rows + r] = s;
-            sum[cc * rows + r] = add_carry(s, x, carry);
+            dst[cc * rows + r] = sv[k];
+            sum[cc * rows + r] = add_carry(sv[k], t[threadIdx.x][k], carry);
         }
         return;
     }

@@ -509,6 +509,7 @@ __device__ void chain(const DiagParams &p, Blk *s, ChainBars &cb) {
         for (int64_t r = lane; r < b; r += 32) mx = fmaxf(mx, __ldcg(p.W + r * b + r));
         for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
         if (lane == 0) *p.lkk = sqrt((double)mx);
+        __syncwarp();  // the arrival counts the warp as a whole
         asm volatile("bar.arrive 2, 288;" ::: "memory");
         if (lane != 0) return;
         for (int q = 0; q < NB; ++q) {

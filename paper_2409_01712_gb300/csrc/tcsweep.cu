@@ -78,6 +78,10 @@ constexpr int TS_NPMAX = 32;             // right-hand sides per launch
 constexpr int TS_IRING = 4;              // item header slots
 constexpr int TS_BSEG = 16;              // most groups of 64 rows of the vector block held at once
 constexpr int TS_BBOX = 256;             // rows of a B copy (groups x columns of a group)
+constexpr int TS_NSMAX = 12;             // most A stages
+// The producer loads A of an item's first stages before it looks for the next
+// part of B, so these chunks must not reach beyond the first part.
+static_assert(TS_NSMAX <= TS_BSEG, "the A chunks loaded ahead stay within the first part of B");
 
 enum { TS_FWD = 0, TS_BWD = 1 };
 enum { IT_CONV = 0, IT_DIAG = 1, IT_LINK = 2, IT_END = 3 };
@@ -986,6 +990,10 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
 constexpr int RS_THREADS = 576;
 constexpr int RS_STG = 32768;      // FP32 chunk: 128 x 64 or 64 x 128
 constexpr int RS_NSTG = 5;         // stages (FP32 K chunk by TMA, converted in place, and the terms of a)
+// The two converter groups take every other chunk.  With an odd number of stages a
+// stage holds their chunks in turn, which is what a group's wait for the chunk
+// before its own rests on (see the converters).
+static_assert(RS_NSTG % 2 == 1, "the converter groups alternate on every stage");
 constexpr int RS_NACC = 4;         // TMEM accumulators of 3 np columns
 // (K - c) s in FP16 with the power of two s = 2^(e - 1) <= 8192 / (max|K| + |c|):
 // |(K - c) s| <= 8192, far below the FP16 maximum (s = 2^12 for the Gaussian
@@ -1743,13 +1751,13 @@ krr_status run_ts(Ctx *c, int job, float *rhs, float *out, int64_t p) {
         sp.st_in = ts_states(c);
         sp.st_out = ts_states(c) + nt;
         sp.flags = flags;
-        // B takes up to 64 KB (128 KB above 16 columns), A stages the rest: 9
-        // (5) of them; more would cross a part of B
+        // B takes up to 64 KB (128 KB above 16 columns), A stages the rest, as many
+        // as TS_NSMAX: 10 (6) of them from b = 1024 on
         sp.lkc = 0;
         while ((1 << sp.lkc) < sp.KC) ++sp.lkc;
         sp.bseg = (int)std::min<int64_t>(sp.KC, TS_BSEG);
         const int b_bytes = sp.bseg * 2 * sp.np * 128;
-        int stages = 12;
+        int stages = TS_NSMAX;
         while (stages > 2 && ts_smem_bytes(stages, b_bytes) > ts_smem_limit()) --stages;
         sp.stages = stages;
         // kind::f16, D = F32, A = B = F16, A K-major (forward) or MN-major

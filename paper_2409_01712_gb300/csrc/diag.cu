@@ -593,10 +593,8 @@ __device__ void chain(const DiagParams &p, Blk *s, ChainBars &cb) {
         for (int u = 0; u < 4; ++u) {
             const int r = ty + 16 * u, c = 4 * tx;
             float4 w = *reinterpret_cast<const float4 *>(&s[0][r][c]);
-            if ((c >> 4) < (r >> 4)) {
-                // below the diagonal blocks E is zero; the next product reads it
-                w = make_float4(0.f, 0.f, 0.f, 0.f);
-            }
+            // E is not kept below its diagonal 16-blocks (no product reads it there)
+            if ((c >> 4) < (r >> 4)) w = make_float4(0.f, 0.f, 0.f, 0.f);
             __stcg(reinterpret_cast<float4 *>(gt + (int64_t)r * b + c), w);
             const float4 l = *reinterpret_cast<const float4 *>(&A[r][c]);
             __stcg(reinterpret_cast<float4 *>(gl + (int64_t)r * b + c),
@@ -605,11 +603,6 @@ __device__ void chain(const DiagParams &p, Blk *s, ChainBars &cb) {
         }
         csync();
         arrive_pub(&cb.pubp, 2 * q + 1);
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int r = ty + 16 * u, c = 4 * tx;
-            if ((c >> 4) < (r >> 4)) *reinterpret_cast<float4 *>(&s[0][r][c]) = make_float4(0.f, 0.f, 0.f, 0.f);
-        }
     }
     if (t == 0) {
         p.err->min_pivot = fmin(p.err->min_pivot, (double)mpiv);

@@ -502,8 +502,8 @@ krr_status krr_create(krr_ctx **out, const krr_options *opt, void *stream) {
     krr_options o;
     krr_default_options(&o);
     if (opt) o = *opt;
-    // a power of two: the diagonal step inverts the factor by recursive
-    // doubling over 64-wide blocks
+    // a power of two: the sweeps take a tile's chunks in such parts, and the FP64
+    // diagonal step inverts its factor by recursive doubling over 64-wide blocks
     if (o.tile < 256 || o.tile > 4096 || (o.tile & (o.tile - 1)) != 0) {
         g_create_error = "tile must be a power of two in [256, 4096]";
         return KRR_EINVAL;

@@ -249,7 +249,7 @@ struct Ctx {
     float *Linv = nullptr;     // inverse of every diagonal factor tile, FP32
     float *LinvT = nullptr;    // and its transpose (row-oriented backward sweep)
     __half *Linv_hi = nullptr, *Linv_lo = nullptr;  // FP16 split of Linv (mixed)
-    double *diag64 = nullptr;  // FP64 scratch diagonal tile (diag_fp64); FP32 scratch otherwise
+    double *diag64 = nullptr;  // FP64 scratch diagonal tile (diag_fp64 only)
     int *diag_ctr = nullptr;   // progress counters of the diagonal-step kernel
     double *diag64_inv = nullptr;
     uint8_t *pool = nullptr;   // off-diagonal factor tiles, each in its precision
@@ -282,7 +282,7 @@ struct Ctx {
     int64_t sw_flags_cap = 0;
     __half *ts_v0 = nullptr, *ts_v1 = nullptr;  // tensor-core sweep: FP16 pairs of vector blocks
     size_t ts_vcap = 0;
-    void *ts_aux = nullptr;                  // tensor-core sweep: block scales, slab maxima, counters
+    void *ts_aux = nullptr;                  // tensor-core sweep: scales, block maxima, states, counters
     size_t ts_aux_cap = 0;
     float *ts_xt = nullptr;                  // tensor-core sweep: column-major copy of the right-hand sides
     size_t ts_xcap = 0;

@@ -90,7 +90,7 @@ enum { AM_POOL = 0, AM_WSH = 1, AM_LHI = 2, AM_LLO = 3 };
 
 struct TsParams {
     int job;
-    int64_t b, nt, S, KC, items, n_pad;
+    int64_t b, nt, S, KC, items;
     int np, pc, q0;
     int64_t rs, cs;           // vector element (row, column q0 + q) at row * rs + (q0 + q) * cs
     float *rhs;               // FWD: y, BWD: z (updated in place)
@@ -1597,12 +1597,12 @@ size_t ts_smem_bytes(int stages, int b_bytes) {
 
 int64_t ts_flag_count(const Ctx *c) { return 2 + 2 * c->nt + c->nt * (c->b / TS_SLAB); }
 
-// Auxiliary buffer: block scales of the two FP16 vector buffers ([nt][TS_NPMAX]
-// each), per-slab column maxima of the two ([nt][S][TS_NPMAX] each), their
-// block column maxima ([nt][TS_NPMAX] each), the states of their blocks ([nt]
-// 64-bit words each), then the progress counters.
+// Auxiliary buffer: exact block scales of the two FP16 vector buffers ([nt][TS_NPMAX]
+// each), the inverse scales of the residual's operand ([n_pad / 128][TS_NPMAX]),
+// the block column maxima of the two buffers ([nt][TS_NPMAX] each), the states of
+// their blocks ([nt] 64-bit words each), then the progress counters.
 int64_t ts_scale_count(const Ctx *c) { return c->nt * TS_NPMAX; }
-int64_t ts_max_count(const Ctx *c) { return c->nt * (c->b / TS_SLAB) * TS_NPMAX; }
+int64_t res_scale_count(const Ctx *c) { return c->n_pad / TS_SLAB * TS_NPMAX; }
 
 krr_status ensure_ts_buffers(Ctx *c, int64_t p) {
     const size_t vbytes = (size_t)3 * TS_NPMAX * c->n_pad * sizeof(__half);
@@ -1618,7 +1618,7 @@ krr_status ensure_ts_buffers(Ctx *c, int64_t p) {
         }
         c->ts_vcap = vbytes;
     }
-    const size_t abytes = (size_t)(4 * ts_scale_count(c) + 2 * ts_max_count(c)) * sizeof(float) +
+    const size_t abytes = (size_t)(4 * ts_scale_count(c) + res_scale_count(c)) * sizeof(float) +
                           (size_t)2 * c->nt * sizeof(unsigned long long) + (size_t)ts_flag_count(c) * sizeof(int);
     if (c->ts_aux_cap < abytes) {
         if (c->ts_aux) cudaFree(c->ts_aux);
@@ -1645,8 +1645,8 @@ krr_status ensure_ts_buffers(Ctx *c, int64_t p) {
 }
 
 float *ts_scales(Ctx *c) { return (float *)c->ts_aux; }
-float *ts_maxima(Ctx *c) { return ts_scales(c) + 2 * ts_scale_count(c); }
-float *ts_block_maxima(Ctx *c) { return ts_maxima(c) + 2 * ts_max_count(c); }
+float *res_scales(Ctx *c) { return ts_scales(c) + 2 * ts_scale_count(c); }
+float *ts_block_maxima(Ctx *c) { return res_scales(c) + res_scale_count(c); }
 unsigned long long *ts_states(Ctx *c) { return (unsigned long long *)(ts_block_maxima(c) + 2 * ts_scale_count(c)); }
 int *ts_flags(Ctx *c) { return (int *)(ts_states(c) + 2 * c->nt); }
 
@@ -1730,7 +1730,6 @@ krr_status run_ts(Ctx *c, int job, float *rhs, float *out, int64_t p) {
         sp.nt = nt;
         sp.S = b / TS_SLAB;
         sp.KC = b / TS_KC;
-        sp.n_pad = c->n_pad;
         sp.items = 1 + sp.S * nt * (nt + 1) / 2;  // sum of the section sizes
         sp.pc = (int)std::min<int64_t>(TS_NPMAX, p - q0);
         sp.np = (sp.pc + 15) & ~15;
@@ -1889,7 +1888,7 @@ krr_status tc_residual(Ctx *c, const float *y, const float *a, int64_t p) {
         },
         &gr));
     double *cs_part = c->rs_part + part_count, *np_part = cs_part + nblk * pmax;
-    float *inv_s = ts_maxima(c);
+    float *inv_s = res_scales(c);
     for (int64_t q0 = 0; q0 < p; q0 += TS_NPMAX) {
         const int pc = (int)std::min<int64_t>(TS_NPMAX, p - q0), np = (pc + 15) & ~15;
         // item counter, abort flag, block counters of the two small kernels

@@ -523,8 +523,8 @@ __device__ __forceinline__ float dist_f32(float ni, float nj, float s) { return 
 // division of the IBS form and the confounder loop are branches), and with two
 // epilogue warps a scheduler each entry's chain of exact distance, exponential
 // and sums was paid in full: 62 instructions an entry at 6 cycles each.  As
-// straight code for 16 entries Build takes 0.048 ms instead of 0.100 at
-// N = 5000, M = 700, 2.82 instead of 3.38 at N = 32768, M = 8192, and with 10
+// straight code for 16 entries Build takes 0.050 ms instead of 0.100 at
+// N = 5000, M = 700, 2.85 instead of 3.38 at N = 32768, M = 8192, and with 10
 // confounders 0.31 instead of 0.49 at N = 10000, M = 4000.
 enum { KV_GAUSS = 0, KV_CONF = 1, KV_IBS = 2, KV_GRAM = 3 };
 
@@ -560,28 +560,6 @@ __device__ __forceinline__ void own_conf(const TcParams &p, int64_t gi, float (&
 #pragma unroll
     for (int q = 0; q < CONF_MAX; ++q) ci[q] = (KV == KV_CONF) ? p.conf_a[gi * CONF_MAX + q] : 0.f;
 }
-
-// Running sum in two FP32 terms grown by error-free transformations (Knuth's
-// TwoSum): about 48 significant bits.  FP64 additions run at 1/64 of the FP32
-// rate here, and the two sums of a Build block (its entries and their squares)
-// kept its epilogue longer than its tensor work.  Build at N = 32768,
-// M = 8192: 4.03 ms with the FP64 sums and integer distances, 3.39 ms with
-// this; N = 16384, M = 8192: 1.07 and 0.87 ms.
-struct Sum2 {
-    float hi = 0.f, lo = 0.f;
-    __device__ __forceinline__ void add(float x) {
-        const float s = hi + x, bp = s - hi;
-        lo += (hi - (s - bp)) + (x - bp);
-        hi = s;
-    }
-    // x * x as the exact pair product + remainder
-    __device__ __forceinline__ void add_square(float x) {
-        const float q = x * x;
-        lo += fmaf(x, x, -q);
-        add(q);
-    }
-    __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
-};
 
 // Issues L2 prefetches for the trailing-update input row segment of this
 // thread, before it waits for the accumulator.
@@ -727,10 +705,13 @@ __device__ __forceinline__ double grad_half(const TcParams &p, const Work &w, ui
 
 // Build: the thread's row of the block against 128 of its columns: K entries
 // (the identity in padding), their sum and sum of squares, and the exact
-// distances when they are kept.
+// distances when they are kept.  The sums are formed without FP64 additions
+// (WideSum), which kept the epilogue longer than its tensor work: N = 32768,
+// M = 8192 4.03 ms with FP64 sums and integer distances, 3.39 ms without them,
+// 2.85 ms with the kernel function chosen per block.
 template <int KV>
 __device__ __forceinline__ void dist_half(const TcParams &p, const Work &w, uint32_t tacc, int row, int ch0,
-                                          const float *nb_s, const float *aw_s, Sum2 &sum2, Sum2 &sum1) {
+                                          const float *nb_s, const float *aw_s, WideSum &sum2, WideSum &sum1) {
     const int64_t b = p.b;
     const int64_t gi = w.i * b + w.sm * BM + row, j0 = w.j * b + w.sn * BN;
     const float ni = (float)p.norms_a[gi];
@@ -751,11 +732,14 @@ __device__ __forceinline__ void dist_half(const TcParams &p, const Work &w, uint
             const float k = entry<KV>(p, ni, nb_s[c], v[e], ci, aw_s + c * PRED_MAX_P + 16);
             kv[e] = (c < nreal) ? k : (c == cdiag ? 1.f : 0.f);
         }
+        ChunkSum c2, c1;
 #pragma unroll
-        for (int e = 0; e < 16; ++e) {
-            sum2.add_square(kv[e]);
-            sum1.add(kv[e]);
+        for (int e = 0; e < 16; e += 4) {
+            c2.add_squares4(kv[e], kv[e + 1], kv[e + 2], kv[e + 3]);
+            c1.add4(kv[e], kv[e + 1], kv[e + 2], kv[e + 3]);
         }
+        sum2.add(c2);
+        sum1.add(c1);
         float4 *dst = reinterpret_cast<float4 *>(krow + ch * 16);
 #pragma unroll
         for (int e = 0; e < 4; ++e) dst[e] = make_float4(kv[4 * e], kv[4 * e + 1], kv[4 * e + 2], kv[4 * e + 3]);
@@ -780,7 +764,7 @@ __device__ __forceinline__ void epilogue(const TcParams &p, const Work &w, uint3
     const int ch0 = half * CH_PER_HALF;
     if (OP == OP_DIST) {
         const int64_t tidx = tri_index(w.i, w.j);
-        Sum2 sum2, sum1;
+        WideSum sum2, sum1;
         if (p.kf.gram)
             dist_half<KV_GRAM>(p, w, tacc, row, ch0, nb_s, aw_s, sum2, sum1);
         else if (p.kf.ibs)

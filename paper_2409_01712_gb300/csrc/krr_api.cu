@@ -274,10 +274,7 @@ krr_status adopt_build(Ctx *dst, const Ctx *src) {
     dst->nconf = 0;
     dst->rr = 0;
     const size_t red_count = src->red_cap;
-    if (dst->red_cap < red_count) {
-        KRR_TRY(dev_alloc(dst, &dst->red, red_count, "reduction buffer"));
-        dst->red_cap = red_count;
-    }
+    KRR_TRY(grow(dst, &dst->red, &dst->red_cap, red_count, "reduction buffer"));
     if (!dst->hred && cudaMallocHost((void **)&dst->hred, 64 * sizeof(double)) != cudaSuccess) {
         cudaGetLastError();
         dst->hred = nullptr;
@@ -317,10 +314,7 @@ krr_status ensure_work_vectors(Ctx *c, int64_t p) {
 // ... and the column sums of the solve.
 krr_status ensure_vectors(Ctx *c, int64_t p) {
     KRR_TRY(ensure_work_vectors(c, p));
-    if (c->colsum_cap < p) {
-        KRR_TRY(dev_alloc(c, &c->colsum, (size_t)p, "column sums"));
-        c->colsum_cap = p;
-    }
+    KRR_TRY(grow(c, &c->colsum, &c->colsum_cap, (size_t)p, "column sums"));
     return KRR_OK;
 }
 
@@ -452,10 +446,7 @@ krr_status prepare_build(Ctx *c, int64_t n, int64_t m_pad, int keep_d) {
     c->nt = nt;
     c->n_pad = n_pad;
     const size_t red_count = RED_MINPIV + (size_t)nt * (b / 64) + (size_t)nt + 16 + (size_t)norm_partial_count();
-    if (c->red_cap < red_count) {
-        KRR_TRY(dev_alloc(c, &c->red, red_count, "reduction buffer"));
-        c->red_cap = red_count;
-    }
+    KRR_TRY(grow(c, &c->red, &c->red_cap, red_count, "reduction buffer"));
     if (!c->hred && cudaMallocHost((void **)&c->hred, 64 * sizeof(double)) != cudaSuccess) {
         cudaGetLastError();
         c->hred = nullptr;
@@ -668,10 +659,7 @@ static krr_status build_common(krr_ctx *c, const int8_t *G, int64_t n, int64_t m
     c->nconf = 0;
     if (nc > 0) {
         const size_t cnt = (size_t)n_pad * CONF_MAX;
-        if (c->conf_cap < cnt) {
-            KRR_TRY(dev_alloc(c, &c->conf, cnt, "confounders"));
-            c->conf_cap = cnt;
-        }
+        KRR_TRY(grow(c, &c->conf, &c->conf_cap, cnt, "confounders"));
         KRR_TRY(load_conf(c, C, n, nc, ldc, n_pad, c->conf));
         c->nconf = nc;
     }
@@ -774,6 +762,49 @@ LookaheadPlan lookahead_plan(const Ctx *c, int64_t k) {
     return pl;
 }
 
+// Buffers of a factor on the context's tile grid.
+krr_status alloc_factor(Ctx *c) {
+    const int64_t b = c->b, nt = c->nt, bb = b * b;
+    const int64_t noff = nt * (nt - 1) / 2;
+    const bool mx = mixed(c);
+    cudaStream_t s = c->stream;
+    if (noff > 0) {
+        if (mx) {
+            KRR_TRY(dev_alloc(c, (__half **)&c->W, (size_t)noff * bb, "trailing tiles"));
+        } else {
+            KRR_TRY(dev_alloc(c, (float **)&c->W, (size_t)noff * bb, "trailing tiles"));
+        }
+    }
+    KRR_TRY(dev_alloc(c, &c->Wd, (size_t)nt * bb, "diagonal tiles"));
+    KRR_TRY(dev_alloc(c, &c->Linv, (size_t)nt * bb, "diagonal inverses"));
+    KRR_TRY(dev_alloc(c, &c->LinvT, (size_t)nt * bb, "transposed diagonal inverses"));
+    // the diagonal step writes the inverses on and below the diagonal only
+    KRR_CUDA_TRY(c, cudaMemsetAsync(c->Linv, 0, (size_t)nt * bb * sizeof(float), s));
+    KRR_CUDA_TRY(c, cudaMemsetAsync(c->LinvT, 0, (size_t)nt * bb * sizeof(float), s));
+    if (c->opt.diag_fp64) {
+        KRR_TRY(dev_alloc(c, &c->diag64, (size_t)bb, "FP64 diagonal scratch"));
+        KRR_TRY(dev_alloc(c, &c->diag64_inv, (size_t)2 * bb, "FP64 inverse scratch"));
+    }
+    KRR_TRY(dev_alloc(c, &c->diag_ctr, (size_t)diag_counter_count(b), "diagonal-step counters"));
+    const size_t pool_bytes = (size_t)std::max<int64_t>(noff, 1) * bb * 4;
+    KRR_TRY(dev_alloc(c, &c->pool, pool_bytes, "factor pool"));
+    c->pool_bytes = pool_bytes;
+    KRR_TRY(dev_alloc(c, &c->ltab, (size_t)std::max<int64_t>(noff, 1), "tile table"));
+    KRR_TRY(dev_alloc(c, &c->precmap, (size_t)nt * nt, "precision map"));
+    if (mx) {
+        KRR_TRY(dev_alloc(c, &c->Linv_hi, (size_t)nt * bb, "inverse split"));
+        KRR_TRY(dev_alloc(c, &c->Linv_lo, (size_t)nt * bb, "inverse split"));
+        KRR_CUDA_TRY(c, cudaMemsetAsync(c->Linv_hi, 0, (size_t)nt * bb * sizeof(__half), s));
+        KRR_CUDA_TRY(c, cudaMemsetAsync(c->Linv_lo, 0, (size_t)nt * bb * sizeof(__half), s));
+        const size_t colt = (size_t)std::max<int64_t>(nt - 1, 1);
+        KRR_TRY(dev_alloc(c, &c->colbuf, colt * bb, "column buffer"));
+        KRR_TRY(dev_alloc(c, &c->pan_hi, colt * bb, "operand panel"));
+        KRR_TRY(dev_alloc(c, &c->pan_lo, colt * bb, "operand panel"));
+        KRR_TRY(dev_alloc(c, &c->colmax, colt * (size_t)tile_max_partials(b), "column maxima"));
+    }
+    return KRR_OK;
+}
+
 }  // namespace
 
 krr_status krr_factor(krr_ctx *c, double lambda, krr_factor_info *info) {
@@ -796,41 +827,12 @@ krr_status krr_factor(krr_ctx *c, double lambda, krr_factor_info *info) {
     const size_t w_bytes = (size_t)noff * bb * (mx ? 2 : 4);
     if (!c->Wd || c->w_bytes != w_bytes) {
         free_factor(c);
-        if (noff > 0) {
-            if (mx) {
-                KRR_TRY(dev_alloc(c, (__half **)&c->W, (size_t)noff * bb, "trailing tiles"));
-            } else {
-                KRR_TRY(dev_alloc(c, (float **)&c->W, (size_t)noff * bb, "trailing tiles"));
-            }
+        const krr_status st = alloc_factor(c);
+        if (st != KRR_OK) {
+            free_factor(c);  // all of them or none
+            return st;
         }
         c->w_bytes = w_bytes;
-        KRR_TRY(dev_alloc(c, &c->Wd, (size_t)nt * bb, "diagonal tiles"));
-        KRR_TRY(dev_alloc(c, &c->Linv, (size_t)nt * bb, "diagonal inverses"));
-        KRR_TRY(dev_alloc(c, &c->LinvT, (size_t)nt * bb, "transposed diagonal inverses"));
-        // the diagonal step writes the inverses on and below the diagonal only
-        KRR_CUDA_TRY(c, cudaMemsetAsync(c->Linv, 0, (size_t)nt * bb * sizeof(float), s));
-        KRR_CUDA_TRY(c, cudaMemsetAsync(c->LinvT, 0, (size_t)nt * bb * sizeof(float), s));
-        if (c->opt.diag_fp64) {
-            KRR_TRY(dev_alloc(c, &c->diag64, (size_t)bb, "FP64 diagonal scratch"));
-            KRR_TRY(dev_alloc(c, &c->diag64_inv, (size_t)2 * bb, "FP64 inverse scratch"));
-        }
-        KRR_TRY(dev_alloc(c, &c->diag_ctr, (size_t)diag_counter_count(b), "diagonal-step counters"));
-        const size_t pool_bytes = (size_t)std::max<int64_t>(noff, 1) * bb * 4;
-        KRR_TRY(dev_alloc(c, &c->pool, pool_bytes, "factor pool"));
-        c->pool_bytes = pool_bytes;
-        KRR_TRY(dev_alloc(c, &c->ltab, (size_t)std::max<int64_t>(noff, 1), "tile table"));
-        KRR_TRY(dev_alloc(c, &c->precmap, (size_t)nt * nt, "precision map"));
-        if (mx) {
-            KRR_TRY(dev_alloc(c, &c->Linv_hi, (size_t)nt * bb, "inverse split"));
-            KRR_TRY(dev_alloc(c, &c->Linv_lo, (size_t)nt * bb, "inverse split"));
-            KRR_CUDA_TRY(c, cudaMemsetAsync(c->Linv_hi, 0, (size_t)nt * bb * sizeof(__half), s));
-            KRR_CUDA_TRY(c, cudaMemsetAsync(c->Linv_lo, 0, (size_t)nt * bb * sizeof(__half), s));
-            const size_t colt = (size_t)std::max<int64_t>(nt - 1, 1);
-            KRR_TRY(dev_alloc(c, &c->colbuf, colt * bb, "column buffer"));
-            KRR_TRY(dev_alloc(c, &c->pan_hi, colt * bb, "operand panel"));
-            KRR_TRY(dev_alloc(c, &c->pan_lo, colt * bb, "operand panel"));
-            KRR_TRY(dev_alloc(c, &c->colmax, colt * (size_t)tile_max_partials(b), "column maxima"));
-        }
     }
     // reset the error record, the precision map and (fp32 mode) the tile
     // table on the device: no host data, so the sequence can be captured
@@ -1009,25 +1011,13 @@ static krr_status predict_common(krr_ctx *c, const int8_t *T, int64_t n_test, in
     const bool mx = mixed(c);
     const int64_t rows_pad = (n_test + 127) / 128 * 128;
     const size_t tbytes = (size_t)rows_pad * c->m_pad * (mx ? 1 : 4);
-    if (c->t_cap < tbytes) {
-        KRR_TRY(dev_alloc(c, &c->t8, tbytes, "test genotypes"));
-        c->t_cap = tbytes;
-    }
-    if (c->tnorm_cap < (size_t)rows_pad) {
-        KRR_TRY(dev_alloc(c, &c->tnorms, (size_t)rows_pad, "test norms"));
-        c->tnorm_cap = rows_pad;
-    }
+    KRR_TRY(grow(c, &c->t8, &c->t_cap, tbytes, "test genotypes"));
+    KRR_TRY(grow(c, &c->tnorms, &c->tnorm_cap, (size_t)rows_pad, "test norms"));
     KRR_TRY(ensure_work_vectors(c, p));
     const int64_t nblk = c->n_pad / 128;  // partial products per 128 training rows
     const size_t part = (size_t)nblk * rows_pad * p;
-    if (c->pred_part_cap < part) {
-        KRR_TRY(dev_alloc(c, &c->pred_part, part, "predict partials"));
-        c->pred_part_cap = part;
-    }
-    if (c->pred_out_cap < (size_t)rows_pad * p) {
-        KRR_TRY(dev_alloc(c, &c->pred_out, (size_t)rows_pad * p, "predictions"));
-        c->pred_out_cap = (size_t)rows_pad * p;
-    }
+    KRR_TRY(grow(c, &c->pred_part, &c->pred_part_cap, part, "predict partials"));
+    KRR_TRY(grow(c, &c->pred_out, &c->pred_out_cap, (size_t)rows_pad * p, "predictions"));
     KRR_TRY(pack(c, T, n_test, c->m, ldt, rows_pad, mx ? c->t8 : nullptr,
                  mx ? nullptr : (float *)c->t8, c->tnorms));
     float *aw = c->dabuf;  // padded copy of the weights
@@ -1035,18 +1025,12 @@ static krr_status predict_common(krr_ctx *c, const int8_t *T, int64_t n_test, in
     const float *tconf = nullptr;
     if (c->nconf > 0) {
         const size_t cnt = (size_t)rows_pad * CONF_MAX;
-        if (c->tconf_cap < cnt) {
-            KRR_TRY(dev_alloc(c, &c->tconf, cnt, "held-out confounders"));
-            c->tconf_cap = cnt;
-        }
+        KRR_TRY(grow(c, &c->tconf, &c->tconf_cap, cnt, "held-out confounders"));
         KRR_TRY(load_conf(c, Ct, n_test, c->nconf, ldct, rows_pad, c->tconf));
         tconf = c->tconf;
     }
     float *out = c->pred_out;
-    if (mx && c->colsum_cap < p) {
-        KRR_TRY(dev_alloc(c, &c->colsum, (size_t)p, "column sums"));
-        c->colsum_cap = p;
-    }
+    if (mx) KRR_TRY(grow(c, &c->colsum, &c->colsum_cap, (size_t)p, "column sums"));
     int pr = prof_begin(c, KRR_PROF_PREDICT);
     if (mx) {
         // products of the shifted kernel K - c, then + c (1^T A) in FP64
@@ -1248,16 +1232,11 @@ extern "C" krr_status krr_grad_hyper(krr_ctx *c, const int8_t *T, int64_t n_test
     const int64_t npad = c->n_pad;
     // buffers
     const size_t tbytes = (size_t)rows * c->m_pad;
-    if (c->t_cap < tbytes) {
-        KRR_TRY(dev_alloc(c, &c->t8, tbytes, "test genotypes"));
-        c->t_cap = tbytes;
-    }
-    if (c->tnorm_cap < (size_t)rows) {
-        KRR_TRY(dev_alloc(c, &c->tnorms, (size_t)rows, "test norms"));
-        c->tnorm_cap = rows;
-    }
+    KRR_TRY(grow(c, &c->t8, &c->t_cap, tbytes, "test genotypes"));
+    KRR_TRY(grow(c, &c->tnorms, &c->tnorm_cap, (size_t)rows, "test norms"));
     KRR_TRY(ensure_vectors(c, p));
     if (c->g_rows_cap < (size_t)rows * p) {
+        c->pred_out_cap = c->g_rows_cap = 0;
         KRR_TRY(dev_alloc(c, &c->g_yt, (size_t)rows * p, "gradient buffers"));
         KRR_TRY(dev_alloc(c, &c->g_gp, (size_t)rows * p, "gradient buffers"));
         KRR_TRY(dev_alloc(c, &c->g_sq, (size_t)rows * p, "gradient buffers"));
@@ -1265,27 +1244,15 @@ extern "C" krr_status krr_grad_hyper(krr_ctx *c, const int8_t *T, int64_t n_test
         c->pred_out_cap = (size_t)rows * p;
         c->g_rows_cap = (size_t)rows * p;
     }
-    if (c->g_aw_cap < (size_t)npad * p) {
-        KRR_TRY(dev_alloc(c, &c->g_aw, (size_t)npad * p, "gradient buffers"));
-        c->g_aw_cap = (size_t)npad * p;
-    }
+    KRR_TRY(grow(c, &c->g_aw, &c->g_aw_cap, (size_t)npad * p, "gradient buffers"));
     const size_t part_pred = (size_t)(npad / 128) * rows * p;      // Yhat partials
     const size_t part_t = (size_t)(2 * rows / 256) * npad * p;     // K_t^T G_p partials
     const size_t part = std::max(part_pred, part_t);
-    if (c->g_part_cap < part) {
-        KRR_TRY(dev_alloc(c, &c->g_part, part, "gradient partials"));
-        c->g_part_cap = part;
-    }
+    KRR_TRY(grow(c, &c->g_part, &c->g_part_cap, part, "gradient partials"));
     const size_t it = (size_t)(rows / 128) * (npad / 256);
     const size_t ik = (size_t)c->nt * (c->nt + 1) / 2 * (c->b / 128) * (c->b / 256);
-    if (c->g_tpart_cap < it) {
-        KRR_TRY(dev_alloc(c, &c->g_tpart, it, "gradient partials"));
-        c->g_tpart_cap = it;
-    }
-    if (c->g_kpart_cap < ik) {
-        KRR_TRY(dev_alloc(c, &c->g_kpart, ik, "gradient partials"));
-        c->g_kpart_cap = ik;
-    }
+    KRR_TRY(grow(c, &c->g_tpart, &c->g_tpart_cap, it, "gradient partials"));
+    KRR_TRY(grow(c, &c->g_kpart, &c->g_kpart_cap, ik, "gradient partials"));
     if (!c->g_scal) KRR_TRY(dev_alloc(c, &c->g_scal, (size_t)8, "gradient scalars"));
 
     // 1. inputs: packed test genotypes, padded weights and held-out phenotypes
@@ -1293,10 +1260,7 @@ extern "C" krr_status krr_grad_hyper(krr_ctx *c, const int8_t *T, int64_t n_test
     KRR_TRY(load_rows_f32(c, A, c->n, p, lda, npad, c->g_aw));
     KRR_TRY(load_rows_f32(c, Yt, n_test, p, ldy, rows, c->g_yt));
     // 2. Yhat = K_t A (Alg. 4), as in krr_predict: (K - c) A + c (1^T A)
-    if (c->colsum_cap < p) {
-        KRR_TRY(dev_alloc(c, &c->colsum, (size_t)p, "column sums"));
-        c->colsum_cap = p;
-    }
+    KRR_TRY(grow(c, &c->colsum, &c->colsum_cap, (size_t)p, "column sums"));
     launch_colsum(c->g_aw, npad, p, c->colsum, s);
     KRR_TRY(tc_predict(c, c->t8, c->tnorms, n_test, rows, c->g_aw, p, p, c->g_part, c->red + RED_KSHIFT));
     launch_predict_reduce(c->g_part, npad / 128, rows, n_test, p, c->pred_out, p, s, c->red + RED_KSHIFT,

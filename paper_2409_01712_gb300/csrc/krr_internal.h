@@ -467,6 +467,17 @@ krr_status dev_alloc(Ctx *c, T **p, size_t count, const char *what) {
     return KRR_OK;
 }
 
+// At least `count` elements; the buffer is kept while it has them.  A buffer that
+// could not be had has none: its capacity must not outlive it.
+template <typename T, typename N>
+krr_status grow(Ctx *c, T **p, N *cap, size_t count, const char *what) {
+    if ((size_t)*cap >= count) return KRR_OK;
+    *cap = 0;
+    const krr_status st = dev_alloc(c, p, count, what);
+    if (st == KRR_OK) *cap = (N)count;
+    return st;
+}
+
 template <typename T>
 void dev_free(T **p) {
     if (*p) cudaFree(*p);

@@ -319,14 +319,6 @@ RRState *state(Ctx *c) {
     return (RRState *)c->rr_state;
 }
 
-template <typename T>
-krr_status grow(Ctx *c, T **p, size_t *cap, size_t count, const char *what) {
-    if (*cap >= count) return KRR_OK;
-    KRR_TRY(dev_alloc(c, p, count, what));
-    *cap = count;
-    return KRR_OK;
-}
-
 // rows x row_bytes of a caller matrix (host or device, ld_bytes apart) into a
 // dense device buffer.
 krr_status copy_in(Ctx *c, void *dst, const void *src, int64_t rows, size_t row_bytes, size_t ld_bytes) {

@@ -5,7 +5,8 @@ histories: several contraction rates, one slow column among fast ones, and
 histories that reach the level of FP32 rounding.  carry_check: the solution
 update's additions with neighbours of equal and of very different magnitudes.
 residual_check: the items and slots of the residual, with the usual memory and
-with less.  sum_check: the Build epilogue's sums against FP64 ones."""
+with less.  sum_check: the Build epilogue's sums against FP64 ones.  alloc_check:
+a buffer's capacity after a failed allocation."""
 import os
 import subprocess
 
@@ -14,7 +15,7 @@ import pytest
 from test_host_helpers import CSRC, ROOT, _nvcc
 
 
-@pytest.mark.parametrize("name", ["refine_check", "carry_check", "residual_check", "sum_check"])
+@pytest.mark.parametrize("name", ["refine_check", "carry_check", "residual_check", "sum_check", "alloc_check"])
 def test_on_the_host(tmp_path, name):
     nvcc = _nvcc()
     if not nvcc:

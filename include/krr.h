@@ -98,7 +98,9 @@ typedef struct krr_options {
     int32_t kernel;          /* KRR_KERNEL_GAUSSIAN (default) or KRR_KERNEL_IBS */
     int32_t lookahead;       /* 1: the diagonal step of column k + 1 overlaps the trailing
                                 update of step k on a second stream (mixed mode, FP32
-                                diagonal step; default 1), 0: strictly in sequence */
+                                diagonal step; default 1), 0: strictly in sequence.
+                                The problems of a batch run in sequence either way:
+                                their launches fill the GPU side by side */
     int32_t reserved;        /* must be 0 */
 } krr_options;
 

@@ -718,9 +718,11 @@ namespace {
 //
 // A context of a batch (graph mode) shares the GPU with the other problems,
 // whose updates fill the SMs that a diagonal step leaves free anyway: there
-// the plain sequence is faster (cross-validation over 6 cohorts of 1024 to
-// 16384 rows x 4 lambdas: 53.4 ms per run, 175 ms with the lookahead, whose
-// diagonal steps wait for SMs that their own problem's update holds).
+// the plain sequence is faster, whatever options.lookahead says (cross-validation
+// over 6 cohorts of 1024 to 16384 rows x 4 lambdas: 53.4 ms per run, 175 ms with the
+// lookahead, whose diagonal steps wait for SMs that their own problem's update
+// holds; 64 problems of 16 cohorts: 120 ms, 168 ms with the lookahead and the
+// kernels of that time).
 struct LookaheadPlan {
     bool on = false;
     int64_t ctas = 0, tiles = 0;  // 0 CTAs: the class limit

@@ -48,15 +48,15 @@ thread_local std::string g_batch_create_error;
 
 // CTAs per launch of a batched problem: the problems run concurrently on their
 // streams, and persistent kernels sized for the whole GPU would each hold every
-// SM while waiting on their dependency chains (64 problems, N up to 16384: no
-// cap 408 ms per run, 32 CTAs for every kernel 220 ms, caps per class 184 ms).
-// Cross-validation over 6 cohorts of 1024 to 16384 rows x 4 lambdas, b = 512,
-// 46.0 ms per run with the diagonal step at 12, the sweeps at 16, the residual at
-// 32 and the pair kernels at 64; one cap at a time: diagonal step 4 / 6 / 8 / 16 /
-// 24 53.7 / 48.9 / 47.3 / 46.8 / 48.0 ms; sweeps 8 / 12 / 24 / 32 53.7 / 48.3 / 45.2 /
+// SM while waiting on their dependency chains.  The caps were set on
+// cross-validation over 6 cohorts of 1024 to 16384 rows x 4 lambdas, b = 512: 46.0
+// ms per run with the diagonal step at 12, the sweeps at 16, the residual at 32 and
+// the pair kernels at 64; one cap at a time: diagonal step 4 / 6 / 8 / 16 / 24
+// 53.7 / 48.9 / 47.3 / 46.8 / 48.0 ms; sweeps 8 / 12 / 24 / 32 53.7 / 48.3 / 45.2 /
 // 45.5; residual 12 / 20 / 48 51.4 / 47.7 / 45.4; pair kernels 32 / 48 / 96 / 128
 // 50.6 / 47.7 / 46.0 / 45.9.  Sweeps at 24 and the residual at 48 together:
-// 45.8 -> 43.9 ms (with later sweeps).
+// 45.8 -> 43.9 ms (with later sweeps).  The 64 problems of 16 cohorts x 4 lambdas
+// (1024 to 16384 rows) take 120 ms with them.
 constexpr int BATCH_CTA_CAP = 32;
 constexpr int BATCH_CAP_DIAG = 12, BATCH_CAP_SWEEP = 24, BATCH_CAP_RESIDUAL = 48, BATCH_CAP_PAIR = 64,
               BATCH_CAP_SINGLE = 64;
@@ -123,8 +123,8 @@ krr_status instantiate(krr_batch *bt, std::string *msg) {
     const int64_t m = bt->m, p = bt->p;
     // problems are captured by decreasing N (stable: the first problem of a
     // shared Build stays ahead of the others), so the longest dependency
-    // chains start first: 168-169 ms per run on the cross-validation
-    // workload against 168-173 ms in problem order (stream priorities by
+    // chains start first: 168-169 ms per run of 64 problems against 168-173 ms
+    // in problem order, measured when a run took that long (stream priorities by
     // size on top of it changed nothing)
     std::vector<int32_t> order(count);
     for (int32_t i = 0; i < count; ++i) order[i] = i;

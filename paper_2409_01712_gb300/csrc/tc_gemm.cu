@@ -111,6 +111,7 @@ struct TcParams {
     const float *gp;   // OP_GRADT: G_p, padded test rows x ldaw
     double *gpart;     // OP_GRADT / OP_GRADK: one partial sum per block
     const double *kshift;  // OP_PREDICT: shift c subtracted from every K entry (nullptr: none)
+    int sum64;             // OP_DIST: FP64 additions in the sums of K and K^2
     KernelFn kf;           // OP_DIST / OP_PREDICT: kernel function of the distance
     // OP_DIST / OP_PREDICT: confounders of the A rows and the B rows
     // (rows x CONF_MAX), nconf of them (0: none)
@@ -703,15 +704,42 @@ __device__ __forceinline__ double grad_half(const TcParams &p, const Work &w, ui
     return val;
 }
 
+// The two sums of a thread's entries, sixteen at a time.
+struct SumsFP32 {  // FP32 additions, see WideSum
+    WideSum s1, s2;
+    __device__ __forceinline__ void add(const float (&kv)[16]) {
+        ChunkSum c2, c1;
+#pragma unroll
+        for (int e = 0; e < 16; e += 4) {
+            c2.add_squares4(kv[e], kv[e + 1], kv[e + 2], kv[e + 3]);
+            c1.add4(kv[e], kv[e + 1], kv[e + 2], kv[e + 3]);
+        }
+        s2.add(c2);
+        s1.add(c1);
+    }
+    __device__ __forceinline__ double entries() const { return s1.value(); }
+    __device__ __forceinline__ double squares() const { return s2.value(); }
+};
+struct SumsFP64 {
+    double s1 = 0.0, s2 = 0.0;
+    __device__ __forceinline__ void add(const float (&kv)[16]) {
+#pragma unroll
+        for (int e = 0; e < 16; ++e) {
+            const double x = (double)kv[e];
+            s2 = fma(x, x, s2);  // the square is exact
+            s1 += x;
+        }
+    }
+    __device__ __forceinline__ double entries() const { return s1; }
+    __device__ __forceinline__ double squares() const { return s2; }
+};
+
 // Build: the thread's row of the block against 128 of its columns: K entries
 // (the identity in padding), their sum and sum of squares, and the exact
-// distances when they are kept.  The sums are formed without FP64 additions
-// (WideSum), which kept the epilogue longer than its tensor work: N = 32768,
-// M = 8192 4.03 ms with FP64 sums and integer distances, 3.39 ms without them,
-// 2.85 ms with the kernel function chosen per block.
-template <int KV>
+// distances when they are kept.
+template <int KV, class Sums>
 __device__ __forceinline__ void dist_half(const TcParams &p, const Work &w, uint32_t tacc, int row, int ch0,
-                                          const float *nb_s, const float *aw_s, WideSum &sum2, WideSum &sum1) {
+                                          const float *nb_s, const float *aw_s, Sums &sums) {
     const int64_t b = p.b;
     const int64_t gi = w.i * b + w.sm * BM + row, j0 = w.j * b + w.sn * BN;
     const float ni = (float)p.norms_a[gi];
@@ -732,14 +760,7 @@ __device__ __forceinline__ void dist_half(const TcParams &p, const Work &w, uint
             const float k = entry<KV>(p, ni, nb_s[c], v[e], ci, aw_s + c * PRED_MAX_P + 16);
             kv[e] = (c < nreal) ? k : (c == cdiag ? 1.f : 0.f);
         }
-        ChunkSum c2, c1;
-#pragma unroll
-        for (int e = 0; e < 16; e += 4) {
-            c2.add_squares4(kv[e], kv[e + 1], kv[e + 2], kv[e + 3]);
-            c1.add4(kv[e], kv[e + 1], kv[e + 2], kv[e + 3]);
-        }
-        sum2.add(c2);
-        sum1.add(c1);
+        sums.add(kv);
         float4 *dst = reinterpret_cast<float4 *>(krow + ch * 16);
 #pragma unroll
         for (int e = 0; e < 4; ++e) dst[e] = make_float4(kv[4 * e], kv[4 * e + 1], kv[4 * e + 2], kv[4 * e + 3]);
@@ -757,6 +778,22 @@ __device__ __forceinline__ void dist_half(const TcParams &p, const Work &w, uint
     }
 }
 
+template <class Sums>
+__device__ __forceinline__ void dist_sums(const TcParams &p, const Work &w, uint32_t tacc, int row, int ch0,
+                                          const float *nb_s, const float *aw_s, double *squares, double *entries) {
+    Sums sums;
+    if (p.kf.gram)
+        dist_half<KV_GRAM>(p, w, tacc, row, ch0, nb_s, aw_s, sums);
+    else if (p.kf.ibs)
+        dist_half<KV_IBS>(p, w, tacc, row, ch0, nb_s, aw_s, sums);
+    else if (p.nconf)
+        dist_half<KV_CONF>(p, w, tacc, row, ch0, nb_s, aw_s, sums);
+    else
+        dist_half<KV_GAUSS>(p, w, tacc, row, ch0, nb_s, aw_s, sums);
+    *squares = sums.squares();
+    *entries = sums.entries();
+}
+
 template <int OP>
 __device__ __forceinline__ void epilogue(const TcParams &p, const Work &w, uint32_t tacc, int row, int half,
                                          float *nb_s, float *aw_s, double *red_s) {
@@ -764,16 +801,11 @@ __device__ __forceinline__ void epilogue(const TcParams &p, const Work &w, uint3
     const int ch0 = half * CH_PER_HALF;
     if (OP == OP_DIST) {
         const int64_t tidx = tri_index(w.i, w.j);
-        WideSum sum2, sum1;
-        if (p.kf.gram)
-            dist_half<KV_GRAM>(p, w, tacc, row, ch0, nb_s, aw_s, sum2, sum1);
-        else if (p.kf.ibs)
-            dist_half<KV_IBS>(p, w, tacc, row, ch0, nb_s, aw_s, sum2, sum1);
-        else if (p.nconf)
-            dist_half<KV_CONF>(p, w, tacc, row, ch0, nb_s, aw_s, sum2, sum1);
+        double ss, s1;
+        if (p.sum64)
+            dist_sums<SumsFP64>(p, w, tacc, row, ch0, nb_s, aw_s, &ss, &s1);
         else
-            dist_half<KV_GAUSS>(p, w, tacc, row, ch0, nb_s, aw_s, sum2, sum1);
-        double ss = sum2.value(), s1 = sum1.value();
+            dist_sums<SumsFP32>(p, w, tacc, row, ch0, nb_s, aw_s, &ss, &s1);
         // deterministic per-block sums of K^2 and K: warp sums, then the eight
         // warps in order.  Layout: all K^2 partials, then all K partials.
         for (int o = 16; o > 0; o >>= 1) {
@@ -1462,6 +1494,21 @@ krr_status tc_bind_genotypes(Ctx *c) {
     return make_map(c, &st->g_map, c->g8, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, c->n_pad, c->m_pad);
 }
 
+// Which additions the epilogue's sums use.  FP64 ones make the epilogue of a block
+// 36 us long; with FP32 ones (WideSum) it takes a few, which is 4.03 -> 2.85 ms at
+// N = 32768, M = 8192.  Where the tensor work of a block hides either, the short
+// epilogue's FP32 instructions cost tensor rate instead (the kernel without any sums
+// is as slow there), and the FP64 sums are the faster ones: N = 16384, M = 10240 /
+// 11264 / 12288 / 16384 FP32 0.917 / 1.006 / 1.089 / 1.448 ms, FP64 0.993 / 0.994 /
+// 1.053 / 1.390; N = 65536, M = 16384 21.8 and 20.7 ms; with 10 confounders M = 14336 /
+// 16384 1.314 / 1.488 and 1.337 / 1.435; IBS on 2 x 7168 / 2 x 8192 columns 1.242 /
+// 1.416 and 1.223 / 1.391.  The last blocks' epilogues are not hidden: with three
+// blocks per SM (N = 5000, M = 16384) 0.193 and 0.208 ms.
+bool build_sums_fp64(const Ctx *c, int64_t blocks) {
+    const int64_t cols = (c->nconf > 0 || is_ibs(c) || c->rr) ? 16384 : 12288;
+    return c->m_pad >= cols && blocks >= 16 * (int64_t)c->num_sms;
+}
+
 krr_status tc_build(Ctx *c) {
     TcState *st = (TcState *)c->tc;
     KRR_TRY(tc_bind_genotypes(c));
@@ -1476,6 +1523,7 @@ krr_status tc_build(Ctx *c) {
     p.n = real_rows(c);
     const int64_t ntri = c->nt * (c->nt + 1) / 2;
     p.items = ntri * (c->b / BM) * (c->b / BN);
+    p.sum64 = build_sums_fp64(c, p.items) ? 1 : 0;
     return launch<KIND_F8, OP_DIST>(c, st->g_map, st->g_map, st->g_map, st->g_map, p);
 }
 

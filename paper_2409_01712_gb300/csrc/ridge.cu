@@ -103,10 +103,11 @@ __global__ void rr_conf_t_kernel(const float *cpad, int64_t rows, int nc, float 
 // ---------------------------------------------------------------------------
 // Row-block products with few output columns, split over the contraction:
 //   part[chunk][r][q] = sum_{k in chunk} a(r, k) B[k][q],  r < rows, q < nq <= 32,
-// a from row r of A: int8 values (KIND 0) or FP32 (KIND 2); packed genotypes
-// have a kernel of their own below.  One CTA per 64 rows and chunk; 128-wide slabs of A and B
-// through shared memory; thread (r, g) accumulates columns [8 g, 8 g + 8) of
-// row r in FP32.  The chunks are summed in FP64 by rr_reduce_kernel.
+// a from row r of A: int8 values (KIND 0), packed genotypes (KIND 1; with few
+// columns they have a kernel of their own below) or FP32 (KIND 2).  One CTA per 64
+// rows and chunk; 128-wide slabs of A and B through shared memory; thread (r, g)
+// accumulates columns [8 g, 8 g + 8) of row r in FP32.  The chunks are summed in
+// FP64 by rr_reduce_kernel.
 // ---------------------------------------------------------------------------
 constexpr int RG_R = 64, RG_K = 128;
 
@@ -118,6 +119,10 @@ __device__ __forceinline__ float rg_code(uint32_t v) {
 template <int KIND>
 __device__ __forceinline__ float rg_load(const void *A, int64_t idx) {
     if (KIND == 0) return (float)reinterpret_cast<const int8_t *>(A)[idx];
+    if (KIND == 1) {
+        const uint8_t v = reinterpret_cast<const uint8_t *>(A)[idx];
+        return v == 0x38 ? 1.f : (v == 0x40 ? 2.f : (v == 0x48 ? 3.f : 0.f));
+    }
     return reinterpret_cast<const float *>(A)[idx];
 }
 
@@ -165,15 +170,14 @@ __global__ void __launch_bounds__(256) rr_rowgemm_kernel(const void *A, int64_t 
 }
 
 // The same products for the packed genotypes (E4M3 codes, rows 4-byte aligned,
-// lda a multiple of 128 with zero or finite padding), NQ = 8 or 16 columns from
-// column blockIdx.z NQ on: lanes run along the contraction, four genotypes a
-// load, and a lane keeps 64 / NQ rows x NQ sums in registers, so a genotype is
-// read once as part of a 128-byte warp load and a staged value of B serves 64 /
-// NQ rows.  The general kernel above reads bytes one by one and always forms 32
-// columns: 4096 rows, 16384 patients and 4 columns took 363 us, 149 us here (the
-// operand's 67 MB take 10 us; half the rows a lane with the next loads ahead 156,
-// a whole slab's loads ahead 218).  A lane sums every 32nd group of four, then the
-// lanes in a fixed tree.
+// lda a multiple of 128 with zero or finite padding), nq <= NQ = 8 or 16 columns:
+// lanes run along the contraction, four genotypes a load, and a lane keeps 64 / NQ
+// rows x NQ sums in registers, so a genotype is read once as part of a 128-byte
+// warp load and a staged value of B serves 64 / NQ rows.  The general kernel above
+// reads bytes one by one and always forms 32 columns: 4096 rows, 16384 patients and
+// 4 columns took 363 us, 149 us here (the operand's 67 MB take 10 us; half the rows a
+// lane with the next loads ahead 156, a whole slab's loads ahead 218).  A lane sums
+// every 32nd group of four, then the lanes in a fixed tree.
 constexpr int RP_WARPS = 8, RP_K = 512;
 
 template <int NQ>
@@ -184,7 +188,6 @@ __global__ void __launch_bounds__(32 * RP_WARPS)
     __shared__ __align__(16) float bs[NQ][RP_K + 4];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t r0 = ((int64_t)blockIdx.x * RP_WARPS + warp) * RW;
-    const int q0 = blockIdx.z * NQ;
     const int64_t kbeg = (int64_t)blockIdx.y * kchunk, kend = min(K, kbeg + kchunk);
     float acc[RW][NQ];
 #pragma unroll
@@ -195,7 +198,7 @@ __global__ void __launch_bounds__(32 * RP_WARPS)
         __syncthreads();
         for (int e = threadIdx.x; e < RP_K * NQ; e += 32 * RP_WARPS) {
             const int kk = e / NQ, q = e % NQ;
-            bs[q][kk] = (k0 + kk < kend && q0 + q < nq) ? B[(k0 + kk) * ldb + q0 + q] : 0.f;
+            bs[q][kk] = (k0 + kk < kend && q < nq) ? B[(k0 + kk) * ldb + q] : 0.f;
         }
         __syncthreads();
         for (int kk = 4 * lane; kk < RP_K && k0 + kk < kend; kk += 128) {
@@ -226,8 +229,8 @@ __global__ void __launch_bounds__(32 * RP_WARPS)
         for (int q = 0; q < NQ; ++q) {
             float v = acc[u][q];
             for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-            if (lane == 0 && r0 + u < rows && q0 + q < nq)
-                part[((int64_t)blockIdx.y * rows + r0 + u) * nq + q0 + q] = v;
+            if (lane == 0 && r0 + u < rows && q < nq)
+                part[((int64_t)blockIdx.y * rows + r0 + u) * nq + q] = v;
         }
 }
 
@@ -385,9 +388,15 @@ krr_status xt_times(Ctx *c, RRState *st, const float *B, int64_t ldb, int nq, do
     if (nc > 0) split(c, nc, K, &n2, &k2);
     const size_t need = (size_t)(n1 * m + n2 * nc) * nq;
     KRR_TRY(grow(c, &st->part, &st->part_cap, need, "ridge partial products"));
-    if (mixed(c)) {
+    // The packed kernel up to 8 columns, and up to 16 where there are enough rows for
+    // its blocks of 32: above 16 it would read the operand twice (30000 patients x 6000
+    // genotypes, 17 columns: 1.66 ms, the general kernel 0.88).  16384 patients, 9
+    // columns: 500 rows 106 and 99 us, 1000 rows 130 and 136, 4096 rows 329 and 384.
+    if (mixed(c) && (nq > 16 || (nq > 8 && m < 1000))) {
+        rowgemm<1>(c, c->g8, c->m_pad, m, K, B, ldb, nq, st->part, n1, k1);
+    } else if (mixed(c)) {
         const int nq8 = nq <= 8 ? 8 : 16;
-        const dim3 grid(cdivu(m, RP_WARPS * (64 / nq8)), (unsigned)n1, (unsigned)((nq + nq8 - 1) / nq8));
+        const dim3 grid(cdivu(m, RP_WARPS * (64 / nq8)), (unsigned)n1);
         const auto kernel = nq <= 8 ? rr_rowgemm_packed_kernel<8> : rr_rowgemm_packed_kernel<16>;
         count_launch(), kernel<<<grid, 32 * RP_WARPS, 0, c->stream>>>(c->g8, c->m_pad, m, K, k1, B, ldb, nq, st->part);
     } else
